@@ -84,7 +84,7 @@ int lsb_for_bound_host(double x) {
     return lsb < kMinLsb ? kMinLsb : lsb;
 }
 
-RowView view_of(const psf_csr_t& m) { return RowView{m.rowptr, m.rowptr + 1, m.col, m.val}; }
+RowView view_of(const psf_csr_t& m) { return RowView{m.rowptr, m.rowptr + 1, m.col, m.val, nullptr}; }
 
 int check_csr(const psf_csr_t* m, int n, const char* what) {
     if (!m) return fail(PSF_EINVAL, "%s: null matrix", what);
@@ -171,13 +171,15 @@ int status_to_code(int st) {
 }
 
 // Validate input matrices on the device and wait for the outcome: nothing
-// indexes with an input's columns before this returns PSF_OK.
+// indexes with an input's columns before this returns PSF_OK.  Notes whether
+// every row of every input so far spans consecutive columns (w.band).
 int validate_inputs(Work& w, std::initializer_list<const psf_csr_t*> ms) {
     for (const psf_csr_t* m : ms)
         if (m) CU(launch_validate(m->n, m->nnz, m->rowptr, m->col, m->val, w.C(), w.st));
     Ctl c;
     int rc = read_back(w, c, nullptr);
     if (rc) return rc;
+    w.band = !c.not_band;
     return status_to_code(c.status);
 }
 
@@ -204,9 +206,10 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
              unsigned long long reuse_fma = 0, double out_len = 0.0, bool wide_window = false,
              double fma_hint = 0.0) {
     if (add.size() > (size_t)kMaxAdd) return fail(PSF_ETOOBIG, "%zu addend terms (max %d)", add.size(), kMaxAdd);
-    int *rb, *re;
-    int rc = w.rows_for(slot, &rb, &re);
+    Rows R;
+    int rc = w.rows_for(slot, &R);
     if (rc) return rc;
+    int *rb = R.rb, *re = R.re;
     ProductArgs P{};
     P.n = w.n;
     if (A) {
@@ -217,6 +220,7 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
     for (size_t t = 0; t < add.size(); ++t) P.add[t] = add[t];
     P.out_rb = rb;
     P.out_re = re;
+    P.out_rd = R.rd;
     P.pool_col = w.pcol();
     P.pool_val = w.pval();
     P.ctl = w.C();
@@ -271,35 +275,39 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         // the bitmap map marks B rows from their column bitmaps (built here,
         // one launch over B); the chunked test settings keep the column marks
         const int bm = g_row_bitmaps.load();
-        if (A && !table && bm > 0 && w.bits_cap >= w.cap && w.chunk_cols <= 0 && w.chunk_slots <= 0 &&
+        const bool band = w.band && w.slot_map == 0 && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
+        if (A && !table && !band && bm > 0 && w.bits_cap >= w.cap && w.chunk_cols <= 0 && w.chunk_slots <= 0 &&
             (bm == 2 || (alen >= kBitmapMinA && blen >= kBitmapMinB))) {
             CU(launch_row_bitmaps(w.n, *B, w.bhdr.as<int2>(), w.pool_bits.as<unsigned>(), w.st));
             P.bhdr = w.bhdr.as<int2>();
             P.bbits = w.pool_bits.as<unsigned>();
         }
         const bool cta = A && !table && (w.slot_map == 4 || (w.slot_map == 0 && use_cta(w.n, alen, blen)));
-        CU(launch_product(P, table, w.st, out_len, wide_window || w.slot_map == 3, cta));
+        if (band) {
+            if ((rc = w.take_ticket(&P.ticket, w.st))) return rc;
+            CU(launch_band(P, A ? alen + blen : 0.0, w.st));
+        } else CU(launch_product(P, table, w.st, out_len, wide_window || w.slot_map == 3, cta));
     }
     if (reuse_k > 0) {
-        ReuseArgs R{};
-        R.n = w.n;
-        R.rb = rb;
-        R.re = re;
-        R.col = w.pcol();
-        R.val = w.pval();
-        R.k = reuse_k;
-        R.eps_g = eps_g;
-        R.e_lsb = P.e_lsb;
-        R.fma = reuse_fma;
-        R.words = P.words;
-        R.sticky = P.sticky;
-        R.cand_col = P.cand_col;
-        R.cand_x = P.cand_x;
-        R.cand_cap = P.cand_cap;
-        R.cand_chunk = P.cand_chunk;
-        R.ctl = w.C();
-        R.stat = P.stat;
-        CU(launch_reuse_pass1(R, w.st));
+        ReuseArgs U{};
+        U.n = w.n;
+        U.rb = rb;
+        U.re = re;
+        U.col = w.pcol();
+        U.val = w.pval();
+        U.k = reuse_k;
+        U.eps_g = eps_g;
+        U.e_lsb = P.e_lsb;
+        U.fma = reuse_fma;
+        U.words = P.words;
+        U.sticky = P.sticky;
+        U.cand_col = P.cand_col;
+        U.cand_x = P.cand_x;
+        U.cand_cap = P.cand_cap;
+        U.cand_chunk = P.cand_chunk;
+        U.ctl = w.C();
+        U.stat = P.stat;
+        CU(launch_reuse_pass1(U, w.st));
     }
     if (timed) {
         CU(cudaEventRecord(e1, w.st));
@@ -315,6 +323,7 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         a.n = w.n;
         a.rb = rb;
         a.re = re;
+        a.rd = R.rd;
         a.col = w.pcol();
         a.val = w.pval();
         a.eps_g = eps_g;
@@ -330,19 +339,19 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         a.far_shift = g_far_shift.load(std::memory_order_relaxed);
         CU(launch_alg1(a, w.st));
     }
-    *out = w.pooled(rb, re);
+    *out = w.pooled(R);
     return PSF_OK;
 }
 
 // Copy a canonical CSR input into the pool (4-entry aligned rows), as row
 // slot `slot`; the product kernels read every B row and addend row there.
 int pool_copy(Work& w, const psf_csr_t& m, size_t slot, RowView* out) {
-    int *rb, *re;
-    int rc = w.rows_for(slot, &rb, &re);
+    Rows R;
+    int rc = w.rows_for(slot, &R);
     if (rc) return rc;
-    CU(launch_copy_rows(m.n, m.rowptr, m.col, m.val, rb, re, w.pcol(), w.pval(), w.C(),
+    CU(launch_copy_rows(m.n, m.rowptr, m.col, m.val, R.rb, R.re, R.rd, w.pcol(), w.pval(), w.C(),
                         arena_for(m.n > 0 ? (double)m.nnz / m.n : 1.0), w.st));
-    *out = w.pooled(rb, re);
+    *out = w.pooled(R);
     return PSF_OK;
 }
 
@@ -369,7 +378,7 @@ int make_result(Work& w, const RowView& M, psf_result_t* out, psf_result_s** mad
             break;
         }
         if (w.n > 0) {
-            e = launch_scan_rows(w.n, M.rb, M.re, r->rowptr, w.C(), w.scan.as<long long>(), w.st);
+            e = launch_scan_rows(w.n, M.rb, M.re, M.rd, r->rowptr, w.C(), w.scan.as<long long>(), w.st);
         } else {
             e = cudaMemsetAsync(r->rowptr, 0, sizeof(int), w.st);
         }
@@ -637,10 +646,7 @@ int psf_product_filter(const psf_csr_t* A, const psf_csr_t* B, int32_t nadd, con
             if (addends[t]) {
                 RowView mv;
                 if ((rc = pool_copy(w, *addends[t], 2 + (size_t)t, &mv))) return rc;
-                T.rb = mv.rb;
-                T.re = mv.re;
-                T.col = mv.col;
-                T.val = mv.val;
+                T.rd = mv.rd;
             }
             add.push_back(T);
         }
@@ -960,10 +966,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     AddTerm T{};
                     T.alpha = alpha;
                     if (j >= 1) {
-                        T.rb = Zh[(size_t)j].rb;
-                        T.re = Zh[(size_t)j].re;
-                        T.col = Zh[(size_t)j].col;
-                        T.val = Zh[(size_t)j].val;
+                        T.rd = Zh[(size_t)j].rd;
                     }
                     add.push_back(T);
                 }
@@ -993,10 +996,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     if (alpha != 0.0) {
                         AddTerm T{};
                         T.alpha = alpha;
-                        T.rb = Zh[(size_t)q].rb;
-                        T.re = Zh[(size_t)q].re;
-                        T.col = Zh[(size_t)q].col;
-                        T.val = Zh[(size_t)q].val;
+                        T.rd = Zh[(size_t)q].rd;
                         add.push_back(T);
                     }
                     if ((rc = run_step(w, nullptr, nullptr, add, 0.0, 0.0, 1, si, sslot[nslot], &nxt))) return rc;

@@ -185,13 +185,25 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     const BatchSrc* dsrc = d_src.as<BatchSrc>();
     NormSlot* slots = d_slots.as<NormSlot>();
     CU(launch_inst_table(n, count, d_off.as<int>(), d_inst.as<int>(), st));
-    CU(launch_validate_batch(n, inst, dsrc, d_nnz.as<int>(), w.C(), st));
+    DevBuf d_isband;  // per instance: 1 while its rows span consecutive columns
+    CU(d_isband.alloc((size_t)count, st));
+    CU(cudaMemsetAsync(d_isband.p, 1, (size_t)count, st));
+    CU(launch_validate_batch(n, inst, dsrc, d_nnz.as<int>(), w.C(), d_isband.as<unsigned char>(), st));
+    std::vector<unsigned char> isband((size_t)count);
     {
         Ctl c;
+        CU(cudaMemcpyAsync(isband.data(), d_isband.p, (size_t)count, cudaMemcpyDeviceToHost, st));
         if ((rc = read_back(w, c, nullptr))) return rc;
         if (c.status & kDevBadInput) return fail(PSF_EINVAL, "a batch input is malformed (row pointers, column order "
                                                             "or range, or non-finite value)");
     }
+    // the instances whose rows k_band computes (the chunked and forced slot maps
+    // are for tests of the accumulator)
+    bool any_band = false, any_general = false;
+    for (int i = 0; i < count; ++i) (isband[(size_t)i] ? any_band : any_general) = true;
+    const unsigned char* d_band = nullptr;
+    if (any_band && w.slot_map == 0 && w.chunk_cols <= 0 && w.chunk_slots <= 0) d_band = d_isband.as<unsigned char>();
+    else any_general = true;
     const double zlen_all = n > 0 ? (double)nnz_tot / n : 0.0;
     const unsigned long long arena_z = arena_for(zlen_all > 0.0 ? zlen_all : 1.0);
 
@@ -233,19 +245,19 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             CU(cudaMemsetAsync(slots, 0, sizeof(NormSlot) * kMaxNorms * (size_t)count, st));
             CU(cudaMemsetAsync(d_zstat.p, 0, sizeof(StepStat) * 9 * (size_t)count, st));
             if ((rc = w.reset_pool(zcap))) return rc;
-            int *zrb, *zre;
-            if ((rc = w.rows_for(kRowsZ, &zrb, &zre))) return rc;
+            Rows zr;
+            if ((rc = w.rows_for(kRowsZ, &zr))) return rc;
             if ((rc = mark_pool(w, 0))) return rc;
-            CU(launch_copy_rows_batch(n, inst, dsrc, zrb, zre, w.pcol(), w.pval(), w.C(), arena_z, slots + 1,
+            CU(launch_copy_rows_batch(n, inst, dsrc, zr.rb, zr.re, zr.rd, w.pcol(), w.pval(), w.C(), arena_z, slots + 1,
                                       kMaxNorms, st));
             if ((rc = mark_pool(w, 1))) return rc;
-            const RowView zp = w.pooled(zrb, zre);
+            const RowView zp = w.pooled(zr);
             // norms by row tiles: matrix 0 is the pooled Z, matrix k-1 is Z^k
             NormRowsArgs nr{};
             nr.n = n;
             nr.count = 1;
-            nr.rb[0] = zrb;
-            nr.re[0] = zre;
+            nr.rb[0] = zr.rb;
+            nr.re[0] = zr.re;
             nr.col = w.pcol();
             nr.val = w.pval();
             nr.slots = slots + 1;
@@ -257,16 +269,17 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             if (any_chain) {
                 RowView prev = zp;
                 for (int k = 2; k <= 10; ++k) {
-                    int *rb, *re;
-                    if ((rc = w.rows_for(kRowsPow + (size_t)(k - 2), &rb, &re))) return rc;
-                    nr.rb[k - 1] = rb;
-                    nr.re[k - 1] = re;
+                    Rows R;
+                    if ((rc = w.rows_for(kRowsPow + (size_t)(k - 2), &R))) return rc;
+                    nr.rb[k - 1] = R.rb;
+                    nr.re[k - 1] = R.re;
                     ProductArgs P{};
                     P.n = n;
                     P.A = zp;
                     P.B = prev;
-                    P.out_rb = rb;
-                    P.out_re = re;
+                    P.out_rb = R.rb;
+                    P.out_re = R.re;
+                    P.out_rd = R.rd;
                     P.pool_col = w.pcol();
                     P.pool_val = w.pval();
                     P.ctl = w.C();
@@ -292,14 +305,19 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                         CU(cudaEventCreate(&t1));
                         CU(cudaEventRecord(t0, st));
                     }
-                    CU(launch_product(P, table, st, 0.0, wz));
+                    P.band = table ? nullptr : d_band;
+                    if (any_general || table) CU(launch_product(P, table, st, 0.0, wz));
+                    if (P.band) {
+                        if ((rc = w.take_ticket(&P.ticket, st))) return rc;
+                        CU(launch_band(P, 0.0, st));
+                    }
                     if (g_tune_rec) {
                         CU(cudaEventRecord(t1, st));
                         g_tune_rec->work.push_back(zlen_all * blen);
                         g_tune_rec->ev.emplace_back(t0, t1);
                     }
                     if ((rc = mark_pool(w, k))) return rc;
-                    prev = w.pooled(rb, re);
+                    prev = w.pooled(R);
                 }
                 nr.count = 10;
             }
@@ -528,9 +546,9 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     RowView zpow[11] = {};
     if (keep_powers)
         for (int k = 2; k <= 10; ++k) {
-            int *rb, *re;
-            if ((rc = w.rows_for(kRowsPow + (size_t)(k - 2), &rb, &re))) return rc;
-            zpow[k] = RowView{rb, re, zk_col.as<int>(), zk_val.as<double>()};
+            Rows R;
+            if ((rc = w.rows_for(kRowsPow + (size_t)(k - 2), &R))) return rc;
+            zpow[k] = RowView{R.rb, R.re, zk_col.as<int>(), zk_val.as<double>(), R.rd};
         }
     std::vector<int> sel((size_t)count);
     for (int i = 0; i < count; ++i) sel[(size_t)i] = ip[(size_t)i].trivial ? 1 : ip[(size_t)i].p.q;
@@ -553,7 +571,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         if (g_ps_per_row.load() == 0.0 && cap < est) cap = est;
         if (cap > kMaxPool) cap = kMaxPool;
     }
-    DevBuf d_rowptr, d_bounds;
+    DevBuf d_rowptr, d_bounds, d_tickets;
+    CU(d_tickets.alloc(sizeof(unsigned) * nst, st));
     CU(d_rowptr.alloc(sizeof(int) * ((size_t)n + 1), st));
     CU(d_bounds.alloc(sizeof(int) * ((size_t)count + 1), st));
     std::vector<int> bounds((size_t)count + 1);
@@ -562,23 +581,25 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     Ctl cfin{};
     for (int attempt = 0;; ++attempt) {
         if ((rc = w.reset_pool(cap))) return rc;
-        int *zrb, *zre, *qrb, *qre;
-        if ((rc = w.rows_for(kRowsZ, &zrb, &zre)) || (rc = w.rows_for(kRowsZq, &qrb, &qre))) return rc;
+        Rows zr, qr;
+        if ((rc = w.rows_for(kRowsZ, &zr)) || (rc = w.rows_for(kRowsZq, &qr))) return rc;
         // every row slot of the stages exists before the launches are enqueued
         // (a captured graph must not allocate)
         for (size_t si = 0; si < nst; ++si) {
-            int *rb0, *re0;
-            if ((rc = w.rows_for(slot_of(si), &rb0, &re0))) return rc;
+            Rows R;
+            if ((rc = w.rows_for(slot_of(si), &R))) return rc;
         }
-        int *lrb = nullptr, *lre = nullptr;
-        if (any_sq && (rc = w.rows_for(kRowsLeft, &lrb, &lre))) return rc;
+        Rows lr;
+        if (any_sq && (rc = w.rows_for(kRowsLeft, &lr))) return rc;
         // the whole PS phase: pool copy of Z, every stage, the row-length scan
         auto enqueue = [&](cudaStream_t st) -> int {
         CU(cudaMemsetAsync(d_stat.p, 0, sizeof(StepStat) * nst * (size_t)count, st));
         CU(cudaMemsetAsync(d_dropped.p, 0, sizeof(int) * (size_t)count, st));
+        unsigned* const tickets = d_tickets.as<unsigned>();  // k_band's tile counters, one per stage
+        CU(cudaMemsetAsync(tickets, 0, sizeof(unsigned) * nst, st));
 
-        CU(launch_copy_rows_batch(n, inst, dsrc, zrb, zre, w.pcol(), w.pval(), w.C(), arena_z, nullptr, 0, st));
-        const RowView zp = w.pooled(zrb, zre);
+        CU(launch_copy_rows_batch(n, inst, dsrc, zr.rb, zr.re, zr.rd, w.pcol(), w.pval(), w.C(), arena_z, nullptr, 0, st));
+        const RowView zp = w.pooled(zr);
         std::vector<RowView> baby((size_t)qmax + 1);
         baby[1] = zp;
         RowView left = zp;  // the baby steps' left factor (Z, or W per instance)
@@ -589,20 +610,16 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             const StageTab& T = tabs[si];
             if ((D.kind == 1 || D.kind == 2) && !zq_done) {
                 // Z-hat_(q_i) of every instance, for the giant steps and the g = 1 step
-                const int* rbs[kMaxAdd + 2];
-                const int* res[kMaxAdd + 2];
-                for (int k = 0; k <= qmax; ++k) {
-                    rbs[k] = baby[(size_t)(k >= 1 ? k : 1)].rb;
-                    res[k] = baby[(size_t)(k >= 1 ? k : 1)].re;
-                }
-                CU(launch_compose_rows(n, inst, d_sel.as<int>(), rbs, res, qmax + 1, qrb, qre, st));
+                const RowDesc* rds[kMaxAdd + 2];
+                for (int k = 0; k <= qmax; ++k) rds[k] = baby[(size_t)(k >= 1 ? k : 1)].rd;
+                CU(launch_compose_rows(n, inst, d_sel.as<int>(), rds, qmax + 1, qr.rb, qr.re, qr.rd, st));
                 zq_done = true;
             }
-            int *rb, *re;
-            if ((rc = w.rows_for(slot_of(si), &rb, &re))) return rc;
+            Rows R;
+            if ((rc = w.rows_for(slot_of(si), &R))) return rc;
             ProductArgs P{};
             P.n = n;
-            const RowView zq = w.pooled(qrb, qre);
+            const RowView zq = w.pooled(qr);
             if (D.kind == 0) {
                 P.A = left;
                 P.B = baby[(size_t)D.index - 1];
@@ -619,16 +636,12 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 const RowView* v = nullptr;
                 if (t == tz) v = &zq;
                 else if (t >= 1) v = &baby[(size_t)t];
-                if (v) {
-                    A.rb = v->rb;
-                    A.re = v->re;
-                    A.col = v->col;
-                    A.val = v->val;
-                }
+                if (v) A.rd = v->rd;
                 P.add[t] = A;
             }
-            P.out_rb = rb;
-            P.out_re = re;
+            P.out_rb = R.rb;
+            P.out_re = R.re;
+            P.out_rd = R.rd;
             P.pool_col = w.pcol();
             P.pool_val = w.pval();
             P.ctl = w.C();
@@ -663,13 +676,18 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             // giant stages mark their rows from column bitmaps of S's rows
             // (each S row is read by every row of Z-hat_(q) that needs it)
             const int bm = g_row_bitmaps.load();
-            if (D.kind == 1 && !table && !T.wide && bm > 0 && w.bits_cap >= w.cap && w.chunk_cols <= 0 &&
+            if (D.kind == 1 && any_general && !table && !T.wide && bm > 0 && w.bits_cap >= w.cap && w.chunk_cols <= 0 &&
                 w.chunk_slots <= 0 && (bm == 2 || fma_row >= kBitmapMinA * kBitmapMinB)) {
                 CU(launch_row_bitmaps(n, P.B, w.bhdr.as<int2>(), w.pool_bits.as<unsigned>(), st));
                 P.bhdr = w.bhdr.as<int2>();
                 P.bbits = w.pool_bits.as<unsigned>();
             }
-            CU(launch_product(P, table, st, 0.0, T.wide));
+            P.band = table ? nullptr : d_band;
+            if (any_general || table) CU(launch_product(P, table, st, 0.0, T.wide));
+            if (P.band) {
+                P.ticket = tickets + si;
+                CU(launch_band(P, 0.0, st));
+            }
             if (g_tune_rec) {
                 CU(cudaEventRecord(e1, st));
                 g_tune_rec->work.push_back(fma_row);
@@ -690,8 +708,9 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 a.ninst = count;
                 a.inst = inst;
                 a.bstep = P.bstep;
-                a.rb = rb;
-                a.re = re;
+                a.rb = R.rb;
+                a.re = R.re;
+                a.rd = R.rd;
                 a.col = w.pcol();
                 a.val = w.pval();
                 a.words = P.words;
@@ -706,22 +725,21 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 a.far_shift = g_far_shift.load(std::memory_order_relaxed);
                 CU(launch_alg1_batch(a, st));
             }
-            const RowView out = w.pooled(rb, re);
+            const RowView out = w.pooled(R);
             if (D.kind == 0) {
                 baby[(size_t)D.index] = out;
             } else if (D.kind == 3) {
                 // each instance's left factor and Z-hat_(1): Z, or its W
-                const int* rbs[2] = {zp.rb, out.rb};
-                const int* res[2] = {zp.re, out.re};
-                CU(launch_compose_rows(n, inst, d_lsel.as<int>(), rbs, res, 2, lrb, lre, st));
-                left = w.pooled(lrb, lre);
+                const RowDesc* rds[2] = {zp.rd, out.rd};
+                CU(launch_compose_rows(n, inst, d_lsel.as<int>(), rds, 2, lr.rb, lr.re, lr.rd, st));
+                left = w.pooled(lr);
                 baby[1] = left;
             } else {
                 S = out;
             }
         }
         F = S;
-        CU(launch_scan_rows(n, F.rb, F.re, d_rowptr.as<int>(), w.C(), w.scan.as<long long>(), st));
+        CU(launch_scan_rows(n, F.rb, F.re, F.rd, d_rowptr.as<int>(), w.C(), w.scan.as<long long>(), st));
         CU(launch_bounds(count, d_off.as<int>(), d_rowptr.as<int>(), d_bounds.as<int>(), st));
         return PSF_OK;
         };

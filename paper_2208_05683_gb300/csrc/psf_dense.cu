@@ -49,6 +49,8 @@ __global__ void k_dense_rows(int n, RowView M, double* D) {
 struct DenseAddArgs {
     int n;
     int nadd;
+    const int* col;  // the pool
+    const double* val;
     AddTerm add[kMaxAdd];
 };
 
@@ -60,12 +62,13 @@ __global__ void k_dense_addends(DenseAddArgs A, double* D) {
         double* row = D + (size_t)r * A.n;
         for (int t = 0; t < A.nadd; ++t) {
             const AddTerm& T = A.add[t];
-            if (!T.rb) {
+            if (!T.rd) {
                 if (lane == 0) row[r] = __fma_rn(T.alpha, 1.0, row[r]);
             } else {
-                for (int q = T.rb[r] + lane; q < T.re[r]; q += 32) {
-                    const double v = T.val[q];
-                    if (mag_bits(v) != 0ull) row[T.col[q]] = __fma_rn(T.alpha, v, row[T.col[q]]);
+                const RowDesc d = T.rd[r];
+                for (int q = d.rb + lane; q < d.re; q += 32) {
+                    const double v = A.val[q];
+                    if (mag_bits(v) != 0ull) row[A.col[q]] = __fma_rn(T.alpha, v, row[A.col[q]]);
                 }
             }
             __syncwarp();  // term t + 1 may touch the columns term t touched
@@ -168,30 +171,36 @@ __global__ void __launch_bounds__(256) k_dense_out(ProductArgs P, const double* 
     CandArena carena;
     for (int r = gw; r < n; r += nw) {
         const double* row = C + (size_t)r * n;
-        if (P.A.rb)
-            for (int p = P.A.rb[r] + lane; p < P.A.re[r]; p += 32) {
-                const int k = P.A.col[p];
-                my_fma += (unsigned long long)(P.B.re[k] - P.B.rb[k]);
-            }
+        if (P.A.rb) {
+            const int pa0 = P.A.rb[r], pa1 = P.A.re[r];
+            const bool a_holes = P.A.rd && pa1 - pa0 != rd_nnz(P.A.rd[r]);
+            for (int p = pa0 + lane; p < pa1; p += 32)
+                if (!(a_holes && P.A.val[p] == 0.0)) my_fma += (unsigned long long)rd_nnz(P.B.rd[P.A.col[p]]);
+        }
         if (lane == 0)
-            for (int t = 0; t < P.nadd; ++t)
-                my_fma += P.add[t].rb ? (unsigned long long)(P.add[t].re[r] - P.add[t].rb[r]) : 1ull;
+            for (int t = 0; t < P.nadd; ++t) my_fma += P.add[t].rd ? (unsigned long long)rd_nnz(P.add[t].rd[r]) : 1ull;
         int cnt = 0;
         for (int j0 = 0; j0 < n; j0 += 32) {
             const int j = j0 + lane;
             cnt += __popc(__ballot_sync(kFull, j < n && mag_bits(row[j]) != 0ull));
         }
         if (cnt == 0) {
-            if (lane == 0) P.out_rb[r] = P.out_re[r] = 0;
+            if (lane == 0) {
+                P.out_rb[r] = P.out_re[r] = 0;
+                P.out_rd[r] = RowDesc{0, 0, 0, 0};
+            }
             continue;
         }
         const unsigned long long span = ((unsigned long long)cnt + 3ull) & ~3ull;
         const long long base = arena_take(arena, span, P.arena, P.ctl, P.pool_val, lane);
         if (base < 0) {
-            if (lane == 0) P.out_rb[r] = P.out_re[r] = 0;
+            if (lane == 0) {
+                P.out_rb[r] = P.out_re[r] = 0;
+                P.out_rd[r] = RowDesc{0, 0, 0, 0};
+            }
             continue;
         }
-        int written = 0;
+        int written = 0, first = 0, last = 0;
         for (int j0 = 0; j0 < n; j0 += 32) {
             const int j = j0 + lane;
             const double x = j < n ? row[j] : 0.0;
@@ -199,6 +208,8 @@ __global__ void __launch_bounds__(256) k_dense_out(ProductArgs P, const double* 
             const bool nz = xb != 0ull;
             const unsigned m = __ballot_sync(kFull, nz);
             if (!m) continue;
+            if (written == 0) first = j0 + __ffs(m) - 1;
+            last = j0 + 31 - __clz(m);
             const bool cand = nz && filt && xb <= eps_bits;
             if (nz) {
                 const long long pos = base + written + __popc(m & lanemask_lt());
@@ -219,6 +230,7 @@ __global__ void __launch_bounds__(256) k_dense_out(ProductArgs P, const double* 
         if (lane == 0) {
             P.out_rb[r] = (int)base;
             P.out_re[r] = (int)(base + cnt);
+            P.out_rd[r] = rd_row((int)base, (int)(base + cnt), first, last);
             my_written += (unsigned long long)cnt;
         }
     }
@@ -249,6 +261,8 @@ cudaError_t launch_dense_product(const ProductArgs& P, double* Ad, double* Bd, d
     DenseAddArgs D{};
     D.n = n;
     D.nadd = P.nadd;
+    D.col = P.pool_col;
+    D.val = P.pool_val;
     for (int t = 0; t < P.nadd; ++t) D.add[t] = P.add[t];
     if (P.nadd > 0) {
         k_dense_addends<<<rows_blocks, 256, 0, st>>>(D, Cd);

@@ -46,7 +46,7 @@ struct Ctl {
     int pad1;
     unsigned bar_count;  // fields from here on survive a pool reset
     unsigned bar_gen;
-    int pad;
+    int not_band;  // an input has a row that does not span consecutive columns
     unsigned long long fma_total;  // algorithmic multiply-adds of all products
     unsigned long long mark[kMaxNorms + 1];  // pool counter snapshots delimiting the norm matrices
 };
@@ -67,21 +67,48 @@ struct NormSlot {
     unsigned long long result;  // bits of the 1-norm
 };
 
-// Row view of a matrix: row r spans [rb[r], re[r]) of col/val.
+// Descriptor of one row of a pooled matrix, one 16-byte load.  A full row
+// (sign bit of `first`) spans consecutive columns, one stored entry each: a
+// column without an entry is a stored exact zero (a hole), and `last` holds
+// the number of true entries.  Another row stores its entries alone and
+// `last` is its last column.
+struct __align__(16) RowDesc {
+    int rb, re;
+    int first, last;
+};
+constexpr int kFullRow = (int)0x80000000u;
+__host__ __device__ inline bool rd_full(const RowDesc& d) { return d.first < 0; }
+__host__ __device__ inline int rd_first(const RowDesc& d) { return d.first & 0x7fffffff; }
+__host__ __device__ inline int rd_last(const RowDesc& d) {
+    return d.first < 0 ? rd_first(d) + (d.re - d.rb) - 1 : d.last;
+}
+__host__ __device__ inline int rd_nnz(const RowDesc& d) { return d.first < 0 ? d.last : d.re - d.rb; }
+// row [rb, re) of nnz = re - rb entries with these first and last columns
+__host__ __device__ inline RowDesc rd_row(int rb, int re, int first, int last) {
+    if (re <= rb) return RowDesc{0, 0, 0, 0};
+    const bool full = re - rb == last - first + 1;
+    return RowDesc{rb, re, full ? first | kFullRow : first, full ? re - rb : last};
+}
+// full row [rb, re) from column first on with nnz true entries
+__host__ __device__ inline RowDesc rd_full_row(int rb, int re, int first, int nnz) {
+    return RowDesc{rb, re, first | kFullRow, nnz};
+}
+
+// Row view of a matrix: row r spans [rb[r], re[r]) of col/val; rd holds the
+// row descriptors of a pooled matrix (nullptr: a caller's CSR).
 struct RowView {
     const int* rb;
     const int* re;
     const int* col;
     const double* val;
+    const RowDesc* rd;
 };
 
-// One term alpha * M of a weighted sum; rb == nullptr means M = I.
+// One term alpha * M of a weighted sum, M a matrix of the pool given by its
+// row descriptors; rd == nullptr means M = I.
 struct AddTerm {
-    const int* rb;
-    const int* re;
-    const int* col;
-    const double* val;
     double alpha;
+    const RowDesc* rd;
 };
 
 // A batch of instances is one block-diagonal matrix: instance i owns the
@@ -113,6 +140,7 @@ struct ProductArgs {
     AddTerm add[kMaxAdd];
     int* out_rb;
     int* out_re;
+    RowDesc* out_rd;
     int* pool_col;
     double* pool_val;
     Ctl* ctl;
@@ -150,6 +178,9 @@ struct ProductArgs {
     // no bitmap)
     const int2* bhdr;
     const unsigned* bbits;
+    // batch: instances whose rows k_band computes (nullptr: none)
+    const unsigned char* band;
+    unsigned* ticket;           // k_band's tile counter, 0 at the launch
 };
 
 // Algorithm 1 passes 2, 3, ... and compaction for every filtered instance of
@@ -161,6 +192,7 @@ struct Alg1BatchArgs {
     const BatchStep* bstep;
     int* rb;
     int* re;
+    RowDesc* rd;
     int* col;
     double* val;
     unsigned long long* words;
@@ -189,6 +221,7 @@ struct Alg1Args {
     int n;
     int* rb;
     int* re;
+    RowDesc* rd;
     int* col;
     double* val;
     double eps_g, bound;
@@ -266,24 +299,14 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-__device__ __forceinline__ int warp_min(int v) {
-    for (int o = 16; o; o >>= 1) v = min(v, __shfl_xor_sync(kFull, v, o));
-    return v;
-}
-__device__ __forceinline__ int warp_max(int v) {
-    for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(kFull, v, o));
-    return v;
-}
-__device__ __forceinline__ int warp_sum(int v) {
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
+__device__ __forceinline__ int warp_min(int v) { return __reduce_min_sync(kFull, v); }
+__device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(kFull, v); }
+__device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(kFull, v); }
+// the upper halves' maximum, then the lower halves' among its holders
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-    for (int o = 16; o; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(kFull, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
+    const unsigned h = __reduce_max_sync(kFull, (unsigned)(v >> 32));
+    const unsigned l = __reduce_max_sync(kFull, (unsigned)(v >> 32) == h ? (unsigned)v : 0u);
+    return ((unsigned long long)h << 32) | l;
 }
 __device__ __forceinline__ int warp_excl_scan(int v, int lane) {
     int x = v;

@@ -140,6 +140,13 @@ extern std::atomic<int> g_row_bitmaps;
 constexpr double kBitmapMinA = 12.0;
 constexpr double kBitmapMinB = 32.0;
 
+// A matrix's row arrays: descriptors, first and end entries.
+struct Rows {
+    int* rb = nullptr;
+    int* re = nullptr;
+    RowDesc* rd = nullptr;
+};
+
 struct Work {
     int n = 0;
     cudaStream_t st = nullptr;
@@ -150,7 +157,11 @@ struct Work {
     double dense_xover = 1e300;  // dense tiles for a step with at least this many multiply-adds per n^3
     bool dense_estimate = false;  // a step without a recorded count may use the row-length estimate
     unsigned long long cap = 0, ccap = 0, bits_cap = 0;
-    std::vector<DevBuf*> rows;  // 2n ints each: rb then re
+    std::vector<DevBuf*> rows;  // per matrix: n row descriptors, then rb and re (n ints each)
+    DevBuf tickets;              // tile counters of k_band's launches (zero until used)
+    int next_ticket = 0;
+    static constexpr int kTickets = 128;
+    bool band = false;           // every input row spans consecutive columns: k_band computes the products
     int slot_map = 0;            // 0 auto (by products per row), 1 table, 2 bitmap, 3 wide window, 4 CTA per row
     int chunk_cols = 0, chunk_slots = 0;
 
@@ -208,6 +219,14 @@ struct Work {
         CU(cudaMemcpyAsync(ctl.p, &h, offsetof(Ctl, bar_count), cudaMemcpyHostToDevice, st));
         return PSF_OK;
     }
+    // A zero tile counter for one launch of k_band, in stream order on s.
+    int take_ticket(unsigned** out, cudaStream_t s) {
+        if (!tickets.p) CU(tickets.alloc(sizeof(unsigned) * kTickets, s));
+        if (next_ticket == 0) CU(cudaMemsetAsync(tickets.p, 0, sizeof(unsigned) * kTickets, s));
+        *out = tickets.as<unsigned>() + next_ticket;
+        next_ticket = (next_ticket + 1) % kTickets;
+        return PSF_OK;
+    }
     // Entries a warp reserves in a candidate list at a time: up to 128, so
     // that about 12k warps' unused chunk ends take at most a quarter of it.
     unsigned cand_chunk() const {
@@ -224,14 +243,16 @@ struct Work {
         return PSF_OK;
     }
     // row arrays of matrix slot i
-    int rows_for(size_t i, int** rb, int** re) {
+    int rows_for(size_t i, Rows* out) {
         while (rows.size() <= i) rows.push_back(new DevBuf());
-        if (!rows[i]->p) CU(rows[i]->alloc(sizeof(int) * 2 * (size_t)(n > 0 ? n : 1), st));
-        *rb = rows[i]->as<int>();
-        *re = *rb + n;
+        const size_t nn = (size_t)(n > 0 ? n : 1);
+        if (!rows[i]->p) CU(rows[i]->alloc((sizeof(RowDesc) + 2 * sizeof(int)) * nn, st));
+        out->rd = rows[i]->as<RowDesc>();
+        out->rb = reinterpret_cast<int*>(out->rd + nn);
+        out->re = out->rb + n;
         return PSF_OK;
     }
-    RowView pooled(int* rb, int* re) const { return RowView{rb, re, pool_col.as<int>(), pool_val.as<double>()}; }
+    RowView pooled(const Rows& r) const { return RowView{r.rb, r.re, pool_col.as<int>(), pool_val.as<double>(), r.rd}; }
     int* pcol() const { return pool_col.as<int>(); }
     double* pval() const { return pool_val.as<double>(); }
 };

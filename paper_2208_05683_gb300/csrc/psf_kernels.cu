@@ -10,6 +10,8 @@
 //                 instance parameters.
 //  k_product_cta  the same step with one output row per block of four warps
 //                 (matrices of at most one wave of rows with long B rows).
+//  k_band         the same step where rows span consecutive columns: outputs
+//                 folded in registers.
 //  k_row_bitmaps  column bitmaps of B's rows for the symbolic pass.
 //  k_reuse_pass1  a baby step equal to a power of the norm phase: the first
 //                 pass of Algorithm 1 on that power's rows.
@@ -139,12 +141,13 @@ __device__ __forceinline__ double* ka_of(ProdSmem<false, W>& S) { return S.acc +
 // whole row when `whole`).
 template <bool TAB, int W>
 __device__ __forceinline__ void load_segment(const ProductArgs& P, int seg, int cnt, bool whole, int c0, int c1,
-                                             int lane, ProdSmem<TAB, W>& S, bool store_a,
+                                             int lane, ProdSmem<TAB, W>& S, bool store_a, bool a_holes,
                                              unsigned long long* fma = nullptr, int* kwn = nullptr) {
     if (lane < cnt) {
         int k = P.A.col[seg + lane];
-        int b = P.B.rb[k], e = P.B.re[k];
-        if (fma) *fma += (unsigned long long)(e - b);
+        const RowDesc d = P.B.rd[k];
+        int b = d.rb, e = d.re;
+        if (fma && !(a_holes && P.A.val[seg + lane] == 0.0)) *fma += (unsigned long long)rd_nnz(d);
         if (kwn) {
             // B row k's bitmap: its first word's offset in the window (c0 is a
             // multiple of 32 and the window holds the whole row) and its words
@@ -305,7 +308,8 @@ __device__ __forceinline__ void clear_map(int wlen, int lane, ProdSmem<false, W>
 // until the end); the others are marked column by column as in build_map.
 template <int W>
 __device__ __forceinline__ void mark_from_bitmaps(const ProductArgs& P, int pa0, int pa1, int c0, int cend, int lane,
-                                                  ProdSmem<false, W>& S, bool store_a, unsigned long long* fma) {
+                                                  ProdSmem<false, W>& S, bool store_a, bool a_holes,
+                                                  unsigned long long* fma) {
     constexpr int R = (W + 31) / 32;
     unsigned reg[R];
 #pragma unroll
@@ -314,7 +318,7 @@ __device__ __forceinline__ void mark_from_bitmaps(const ProductArgs& P, int pa0,
     const unsigned* __restrict__ bits = P.bbits;
     for (int seg = pa0; seg < pa1; seg += 32) {
         const int cnt = min(32, pa1 - seg);
-        load_segment<false>(P, seg, cnt, true, c0, cend, lane, S, store_a, fma, kwn);
+        load_segment<false>(P, seg, cnt, true, c0, cend, lane, S, store_a, a_holes, fma, kwn);
         // rows without a bitmap: short ones one per lane, long ones by the warp
         const int my = lane < cnt && kwn[lane] == 0 ? S.kl[lane] : 0;
         mark_rows_short(P.B.col, cnt, c0, cend, lane, S, my > 0 && my <= 32);
@@ -363,30 +367,31 @@ __device__ __forceinline__ void mark_from_bitmaps(const ProductArgs& P, int pa0,
 template <bool TAB, bool BMP = false, bool PAIR = false, int W>
 __device__ __forceinline__ void build_map(const ProductArgs& P, const AddTerm* add, int nadd, unsigned tmask, int r,
                                           int c0, int cend, int pa0, int pa1, bool whole, int lane, ProdSmem<TAB, W>& S,
-                                          bool store_a, int ab, int ae, unsigned long long* fma = nullptr) {
+                                          bool store_a, int ab, int ae, bool a_holes = false,
+                                          unsigned long long* fma = nullptr) {
     clear_map(cend - c0, lane, S);
     __syncwarp();
     for (int t = 0; t < nadd; ++t) {
         if (!((tmask >> t) & 1u)) continue;
         const AddTerm& T = add[t];
-        if (!T.rb) {
+        if (!T.rd) {
             if (lane == 0 && r >= c0 && r < cend) mark_one(r - c0, S);
         } else {
             // (term t's row range is in lane t)
             const int s = __shfl_sync(kFull, ab, t), e = __shfl_sync(kFull, ae, t);
-            if constexpr (TAB) mark_row(T.col, s, e, c0, cend, lane, S);
-            else mark_row<true>(T.col, s, e, c0, cend, lane, S);
+            if constexpr (TAB) mark_row(P.pool_col, s, e, c0, cend, lane, S);
+            else mark_row<true>(P.pool_col, s, e, c0, cend, lane, S);
         }
     }
     if constexpr (!TAB && BMP) {
         if (whole && P.bhdr) {
-            mark_from_bitmaps(P, pa0, pa1, c0, cend, lane, S, store_a, fma);
+            mark_from_bitmaps(P, pa0, pa1, c0, cend, lane, S, store_a, a_holes, fma);
             return;
         }
     }
     for (int seg = pa0; seg < pa1; seg += 32) {
         const int cnt = min(32, pa1 - seg);
-        load_segment<TAB>(P, seg, cnt, whole, c0, cend, lane, S, store_a, fma);
+        load_segment<TAB>(P, seg, cnt, whole, c0, cend, lane, S, store_a, a_holes, fma);
         if constexpr (!TAB) {
             if (warp_max(lane < cnt ? S.kl[lane] : 0) <= 32) {
                 mark_rows_short(P.B.col, cnt, c0, cend, lane, S);
@@ -746,6 +751,18 @@ __device__ __forceinline__ void row_stats_batch(const ProductArgs& P, int inst, 
     }
 }
 
+__device__ __forceinline__ void write_desc(const ProductArgs& P, int r, const RowDesc& d) {
+    P.out_rb[r] = d.rb;
+    P.out_re[r] = d.re;
+    P.out_rd[r] = d;
+}
+// The descriptor of the entries written at [base, base + n), one per column
+// that has an entry (read back by a lane of the warp that wrote them).
+__device__ __forceinline__ RowDesc stored_row(const ProductArgs& P, long long base, int n) {
+    if (n <= 0) return RowDesc{0, 0, 0, 0};
+    return rd_row((int)base, (int)base + n, P.pool_col[base], P.pool_col[base + n - 1]);
+}
+
 // Per-warp state of the product kernel across the rows a warp processes.
 struct RowState {
     unsigned long long written = 0ull, cand = 0ull, absmax = 0ull, fma = 0ull;
@@ -786,10 +803,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
         // the row equals the norm phase's power: k_reuse_copy_batch writes it
         if (bs.reuse && __ldcg(P.inst_dropped + r_inst) == 0) return;
         if (bs.mode == kBatchSkip || bs.mode == kBatchPass) {
-            if (lane == 0) {
-                P.out_rb[r] = bs.mode == kBatchPass ? P.B.rb[r] : 0;
-                P.out_re[r] = bs.mode == kBatchPass ? P.B.re[r] : 0;
-            }
+            if (lane == 0) write_desc(P, r, bs.mode == kBatchPass ? P.B.rd[r] : RowDesc{0, 0, 0, 0});
             return;
         }
         prod = bs.mode == kBatchProduct;
@@ -830,43 +844,41 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     }
     // addend term t's row range, in lane t (the terms' loads in parallel;
     // the loops over the terms below take it with a shuffle)
-    int ab = 0, ae = 0;
+    RowDesc ad{0, 0, 0, 0};
     const bool my_term = lane < nadd && ((tmask >> lane) & 1u);
-    if (my_term && add[lane].rb) {
-        ab = add[lane].rb[r];
-        ae = add[lane].re[r];
-    }
+    if (my_term && add[lane].rd) ad = add[lane].rd[r];
+    const int ab = ad.rb, ae = ad.re;
     if (!fixed && my_term) {
-        const AddTerm& T = add[lane];
-        if (!T.rb) {
+        if (!add[lane].rd) {
             lo = min(lo, r);
             hi = max(hi, r);
         } else if (ab < ae) {
-            lo = min(lo, T.col[ab]);
-            hi = max(hi, T.col[ae - 1]);
+            lo = min(lo, rd_first(ad));
+            hi = max(hi, rd_last(ad));
         }
     }
     int pa0 = 0, pa1 = 0;
+    bool a_holes = false;  // A's row stores exact zeros, which are no terms
     if (prod) {
         pa0 = P.A.rb[r];
         pa1 = P.A.re[r];
+        a_holes = P.A.rd && pa1 - pa0 != rd_nnz(P.A.rd[r]);
     }
     for (int p = pa0 + lane; p < pa1 && !fixed; p += 32) {
-        int k = P.A.col[p];
-        int s = P.B.rb[k], e = P.B.re[k];
-        my_fma += (unsigned long long)(e - s);
-        if (s < e) {
-            lo = min(lo, P.B.col[s]);
-            hi = max(hi, P.B.col[e - 1]);
+        const RowDesc d = P.B.rd[P.A.col[p]];
+        if (!(a_holes && P.A.val[p] == 0.0)) my_fma += (unsigned long long)rd_nnz(d);
+        if (d.rb < d.re) {
+            lo = min(lo, rd_first(d));
+            hi = max(hi, rd_last(d));
         }
     }
-    if (my_term) my_fma += add[lane].rb ? (unsigned long long)(ae - ab) : 1ull;
+    if (my_term) my_fma += add[lane].rd ? (unsigned long long)rd_nnz(ad) : 1ull;
     lo = warp_min(lo);
     hi = warp_max(hi);
     const int row_span = fixed ? fixed_span : hi - lo + 1;  // the statistic: before any alignment
     my_span = max(my_span, row_span);
     if (hi < lo) {
-        if (lane == 0) P.out_rb[r] = P.out_re[r] = 0;
+        if (lane == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
         if constexpr (BATCH) row_stats_batch(P, r_inst, my_fma - fma0, 0ull, 0, 0ull, lane);
         return;
     }
@@ -879,7 +891,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     bool reuse = false;
     if (hi - lo + 1 <= kCols) {
         build_map<TAB, (!BATCH || W == kBmWords), !BATCH>(P, add, nadd, tmask, r, lo, hi + 1, pa0, pa1, true, lane, S,
-                                                   !WIDE, ab, ae, fixed ? &my_fma : nullptr);
+                                                   !WIDE, ab, ae, a_holes, fixed ? &my_fma : nullptr);
         total = count_marks(hi - lo + 1, lane, S);
         reuse = true;
     } else {
@@ -892,7 +904,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     }
     const long long base = arena_take(arena, (unsigned long long)((total + 3) & ~3LL), P.arena, P.ctl, P.pool_val, lane);
     if (base < 0) {
-        if (lane == 0) P.out_rb[r] = P.out_re[r] = 0;
+        if (lane == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
         return;
     }
     // a row of the narrow accumulator that fits every slot (kAccCap) in one
@@ -927,7 +939,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
             const AddTerm& T = add[t];
             // batch: the row's instance's coefficient (a small, cached table)
             const double alpha = BATCH ? P.alpha_tab[(size_t)t * P.ninst + r_inst] : T.alpha;
-            if (!T.rb) {
+            if (!T.rd) {
                 if (lane == 0 && r >= c0 && r < c1) {
                     int i = slot_lookup(S, r - c0);
                     S.acc[i] = __fma_rn(alpha, 1.0, S.acc[i]);
@@ -935,10 +947,10 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
             } else {
                 const int s = __shfl_sync(kFull, ab, t), e = __shfl_sync(kFull, ae, t);
                 for (int q = s + lane; q < e; q += 32) {
-                    int c = T.col[q];
+                    int c = P.pool_col[q];
                     if (c >= c0 && c < c1) {
                         int i = slot_lookup(S, c - c0);
-                        S.acc[i] = __fma_rn(alpha, T.val[q], S.acc[i]);
+                        S.acc[i] = __fma_rn(alpha, P.pool_val[q], S.acc[i]);
                     }
                 }
             }
@@ -948,7 +960,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
         // ---- product A B: k of row r ascending
         for (int seg = pa0; seg < pa1; seg += 32) {
             const int cnt_seg = min(32, pa1 - seg);
-            load_segment<TAB>(P, seg, cnt_seg, single, c0, c1, lane, S, !wide_row);
+            load_segment<TAB>(P, seg, cnt_seg, single, c0, c1, lane, S, !wide_row, false);
             accumulate_segment<WIDE>(P, seg, cnt_seg, c0, lane, S, wide_row);
         }
 
@@ -998,10 +1010,8 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     // the row's unused reserved slots read as exact zeros (never candidates)
     const long long rend = base + ((total + 3) & ~3LL);
     for (long long q = base + written + lane; q < rend; q += 32) P.pool_val[q] = 0.0;
-    if (lane == 0) {
-        P.out_rb[r] = (int)base;
-        P.out_re[r] = (int)(base + written);
-    }
+    __syncwarp();
+    if (lane == 0) write_desc(P, r, stored_row(P, base, written));
     if constexpr (BATCH) {
         row_stats_batch(P, r_inst, my_fma - fma0, my_cand - cand0, written, my_absmax, lane, row_span);
         my_absmax = 0ull;
@@ -1012,7 +1022,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
 
 template <bool TAB, bool BATCH, bool WIDE, int W = kBmWords>
 __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W>::kBlocksPerSm)
-    k_product(ProductArgs P) {
+    k_product(const __grid_constant__ ProductArgs P) {
     // a baby step whose product equals an already computed power (no entry
     // dropped so far) is done by k_reuse_pass1 instead (same value in all blocks)
     if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
@@ -1044,8 +1054,11 @@ __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W
         st.arena.next = blk_arena + (unsigned long long)wib * P.arena;
         st.arena.end = st.arena.next + P.arena;
     }
-    for (int r = blockIdx.x * kWarps + wib; r < P.n; r += gridDim.x * kWarps)
+    for (int r = blockIdx.x * kWarps + wib; r < P.n; r += gridDim.x * kWarps) {
+        if constexpr (BATCH)
+            if (P.band && P.band[P.inst[r]]) continue;  // k_band's rows
         product_row<TAB, BATCH, WIDE, W>(P, add, S, st, r, lane);
+    }
     // the unused end of this warp's arena reads as exact zeros too, and the
     // unused end of its candidate chunk as holes
     arena_close(st.arena, P.pool_val, lane);
@@ -1128,6 +1141,75 @@ __device__ __forceinline__ int compact_row(int* col, double* val, int s, int e, 
     return w;
 }
 
+// Keep the entries of row r (descriptor d) with |x| > fb, in place; returns
+// how many.  A full row stays full while at least three quarters of its
+// columns between the first and the last kept entry keep theirs: the others
+// become holes (exact zeros: they add nothing to any sum, fold or candidate
+// list), so nothing moves and a product finds an entry at its column's place.
+// Measured where rows are bands (half-bandwidth 5, n = 65536): the entries
+// near the threshold are dropped one here, one there, and 0.9 and more stay.
+__device__ __forceinline__ int filter_row(int* col, double* val, int* rb, int* re, RowDesc* rd, int r,
+                                          unsigned long long fb, int lane) {
+    const RowDesc d = rd[r];
+    int s = d.rb, e = d.re;
+    if (rd_full(d)) {
+        int kept = 0, first = -1, last = -1;
+        for (int q0 = s; q0 < e; q0 += 128) {
+            double x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = q0 + u * 32 + lane;
+                x[u] = q < e ? val[q] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q1 = q0 + u * 32;
+                if (q1 >= e) break;
+                const unsigned long long xb = mag_bits(x[u]);
+                const unsigned m = __ballot_sync(kFull, xb > fb);
+                if (xb != 0ull && xb <= fb) val[q1 + lane] = 0.0;
+                if (m) {
+                    if (first < 0) first = q1 + __ffs(m) - 1;
+                    last = q1 + 31 - __clz(m);
+                    kept += __popc(m);
+                }
+            }
+        }
+        if (kept == rd_nnz(d)) return kept;  // nothing dropped
+        if (kept == 0) {
+            if (lane == 0) {
+                rb[r] = re[r] = 0;
+                rd[r] = RowDesc{0, 0, 0, 0};
+            }
+            return 0;
+        }
+        const int c0 = rd_first(d) + (first - s);
+        s = first;
+        e = last + 1;
+        if (4ll * kept >= 3ll * (e - s)) {
+            if (lane == 0) {
+                rb[r] = s;
+                re[r] = e;
+                rd[r] = rd_full_row(s, e, c0, kept);
+            }
+            return kept;
+        }
+        __syncwarp();
+        fb = 0ull;  // too many holes: the kept entries alone
+    }
+    const int w = compact_row(col, val, s, e, fb, lane);
+    if (w != d.re || s != d.rb) {
+        __syncwarp();
+        if (lane == 0) {
+            const RowDesc n = w > s ? rd_row(s, w, col[s], col[w - 1]) : RowDesc{0, 0, 0, 0};
+            rb[r] = n.rb;
+            re[r] = n.re;
+            rd[r] = n;
+        }
+    }
+    return w - s;
+}
+
 // ---------------------------------------------------------------- k_product_cta
 // One output row per block of four warps: for matrices with fewer rows than
 // the warp-per-row kernel has resident warps, whose B rows are long.  The
@@ -1191,9 +1273,11 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
     const int nadd = P.nadd;
     const bool prod = P.A.rb != nullptr;
     int pa0 = 0, pa1 = 0;
+    bool a_holes = false;
     if (prod) {
         pa0 = P.A.rb[r];
         pa1 = P.A.re[r];
+        a_holes = P.A.rd && pa1 - pa0 != rd_nnz(P.A.rd[r]);
     }
     // ---- column window: the matrix itself when it is at most one map wide
     int lo = INT_MAX, hi = -1;
@@ -1206,20 +1290,22 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
         if (tid == 0)
             for (int t = 0; t < nadd; ++t) {
                 const AddTerm& T = add[t];
-                if (!T.rb) {
+                if (!T.rd) {
                     lo = min(lo, r);
                     hi = max(hi, r);
-                } else if (T.rb[r] < T.re[r]) {
-                    lo = min(lo, T.col[T.rb[r]]);
-                    hi = max(hi, T.col[T.re[r] - 1]);
+                } else {
+                    const RowDesc d = T.rd[r];
+                    if (d.rb < d.re) {
+                        lo = min(lo, rd_first(d));
+                        hi = max(hi, rd_last(d));
+                    }
                 }
             }
         for (int p = pa0 + tid; p < pa1; p += kT) {
-            const int k = P.A.col[p];
-            const int s = P.B.rb[k], e = P.B.re[k];
-            if (s < e) {
-                lo = min(lo, P.B.col[s]);
-                hi = max(hi, P.B.col[e - 1]);
+            const RowDesc d = P.B.rd[P.A.col[p]];
+            if (d.rb < d.re) {
+                lo = min(lo, rd_first(d));
+                hi = max(hi, rd_last(d));
             }
         }
         lo = warp_min(lo);
@@ -1238,7 +1324,7 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
         row_span = hi - lo + 1;
     }
     if (hi < lo) {  // no entry at all
-        if (tid == 0) P.out_rb[r] = P.out_re[r] = 0;
+        if (tid == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
         return;
     }
     st.span = max(st.span, row_span);
@@ -1260,10 +1346,11 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
     if (wib == 0) {
         for (int t = 0; t < nadd; ++t) {
             const AddTerm& T = add[t];
-            if (!T.rb) {
+            if (!T.rd) {
                 if (lane == 0 && r >= lo && r <= hi) mark_one(r - lo, M);
             } else {
-                mark_row<true>(T.col, T.rb[r], T.re[r], lo, hi + 1, lane, M);
+                const RowDesc d = T.rd[r];
+                mark_row<true>(P.pool_col, d.rb, d.re, lo, hi + 1, lane, M);
             }
         }
     }
@@ -1276,8 +1363,9 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
         const int cnt = min(32, pa1 - seg);
         if (lane < cnt) {
             const int k = P.A.col[seg + lane];
-            const int b = P.B.rb[k], e = P.B.re[k];
-            rf += (unsigned long long)(e - b);
+            const RowDesc d = P.B.rd[k];
+            const int b = d.rb, e = d.re;
+            if (!(a_holes && P.A.val[seg + lane] == 0.0)) rf += (unsigned long long)rd_nnz(d);
             S.kb[wib][lane] = b;
             S.kl[wib][lane] = e - b;
             int h = 0;
@@ -1324,7 +1412,7 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
         __syncwarp();
     }
     if (wib == 0 && lane == 0)
-        for (int t = 0; t < nadd; ++t) rf += add[t].rb ? (unsigned long long)(add[t].re[r] - add[t].rb[r]) : 1ull;
+        for (int t = 0; t < nadd; ++t) rf += add[t].rd ? (unsigned long long)rd_nnz(add[t].rd[r]) : 1ull;
 #pragma unroll
     for (int u = 0; u < R; ++u) {
         const int w = lane + 32 * u;
@@ -1376,21 +1464,22 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
     __syncthreads();
     const long long base = S.base;
     if (base < 0) {
-        if (tid == 0) P.out_rb[r] = P.out_re[r] = 0;
+        if (tid == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
         return;
     }
     // ---- numeric pass: the addends, t ascending
     for (int t = 0; t < nadd; ++t) {
         const AddTerm& T = add[t];
-        if (!T.rb) {
+        if (!T.rd) {
             if (tid == 0) {
                 const int i = slot_lookup(M, r - lo);
                 S.acc[i] = __fma_rn(T.alpha, 1.0, S.acc[i]);
             }
         } else {
-            for (int q = T.rb[r] + tid; q < T.re[r]; q += kT) {
-                const int i = slot_lookup(M, T.col[q] - lo);
-                S.acc[i] = __fma_rn(T.alpha, T.val[q], S.acc[i]);
+            const RowDesc d = T.rd[r];
+            for (int q = d.rb + tid; q < d.re; q += kT) {
+                const int i = slot_lookup(M, P.pool_col[q] - lo);
+                S.acc[i] = __fma_rn(T.alpha, P.pool_val[q], S.acc[i]);
             }
         }
         __syncthreads();
@@ -1482,15 +1571,14 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
     // the row's unused reserved slots read as exact zeros (never candidates)
     const long long rend = base + ((total + 3) & ~3);
     for (long long q = base + written + tid; q < rend; q += kT) P.pool_val[q] = 0.0;
+    __syncthreads();  // the map and the accumulator are free for the next row
     if (tid == 0) {
-        P.out_rb[r] = (int)base;
-        P.out_re[r] = (int)(base + written);
+        write_desc(P, r, stored_row(P, base, written));
         st.written += (unsigned long long)written;
     }
-    __syncthreads();  // the map and the accumulator are free for the next row
 }
 
-__global__ void __launch_bounds__(kCtaWarps * 32, 7) k_product_cta(ProductArgs P) {
+__global__ void __launch_bounds__(kCtaWarps * 32, 7) k_product_cta(const __grid_constant__ ProductArgs P) {
     if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AddTerm* add = reinterpret_cast<AddTerm*>(smem_raw);
@@ -1518,6 +1606,621 @@ __global__ void __launch_bounds__(kCtaWarps * 32, 7) k_product_cta(ProductArgs P
         if (P.absmax_slot && st.absmax) atomicMax(&P.absmax_slot->absmax, st.absmax);
     }
 }
+
+// ---------------------------------------------------------------- k_band
+// The product step for matrices whose rows span consecutive columns (banded
+// and 1D operators, their powers and the filtered sums of those).  Where
+// every term of an output row is full (RowDesc) the row is folded output by
+// output in registers: no symbolic pass, slot map, shared-memory
+// read-modify-write or barrier between B rows.  A tile is R consecutive output
+// rows by 64 columns; a lane owns the columns c and c + 32 of the tile's rows.
+// The addends are folded in order, then k ascending over the union of the
+// rows' ranges of A: B row k's entry of column c is at position c - first, is
+// loaded once and folded into every row of the tile that has k
+// (acc = fma(a_rk, b_kc, acc)).  Every output's fold is k_product's, in its
+// order, and the results are bitwise the same.
+//
+// Bound by the FP64 pipe: one instruction per (row, k, 32 columns that B row k
+// meets).  R = 4 rows share a load, so that loads are a quarter of them (with
+// one row per tile the same fold waited on L2: L1 holds 15-40 % of what
+// neighbouring rows, in other warps, read again).  Measured against the
+// accumulator kernel, whose slot lookups and read-modify-writes it saves:
+// banded n = 65536, half-bandwidth 5: Z Z^9 361 -> 200 us, the giant steps
+// 470-527 -> 324-423 us (77-81 % of the pipe); banded N(0, 1) n = 20000,
+// w = 15: giant steps 2.31-6.22 -> 1.92-4.59 ms (93-98 %).
+//
+// TEAM: the block's four warps share a tile and take its column groups in
+// turn (long rows, or few).  A row with a term that is not full, or whose
+// range from its first to its last column is longer than its terms together,
+// is computed by the accumulator's code (product_row) in the same memory;
+// rows whose ranges lie apart are folded one by one.
+constexpr int kBandWarps = 4;
+using BandMap = ProdSmem<false, kBmWords>;
+template <int R, bool TEAM>
+struct BandStage {  // terms k of the tile's rows
+    static constexpr int kBytes = TEAM ? (int)sizeof(BandMap) * kBandWarps : (int)sizeof(BandMap);
+    static constexpr int N = (kBytes / (8 * R + 16)) & ~7;
+    int4 d[N];  // {pool position of column 0, first, last column, the tile's rows that have k}
+    double a[N][R];
+};
+
+// acc[r][u] = fma(a[r], x[u], acc[r][u]) for the rows [R0, R1] and the pieces
+// [U0, U1], the columns this lane has (in[u])
+template <int R, int U0, int U1, int R0, int R1>
+__device__ __forceinline__ void fold_rows(const double* __restrict__ a, const double (&x)[2], const bool (&in)[2],
+                                          double (&acc)[R][2]) {
+#pragma unroll
+    for (int r = R0; r <= R1; ++r) {
+        const double ar = a[r];
+#pragma unroll
+        for (int u = U0; u <= U1; ++u)
+            if (in[u]) acc[r][u] = __fma_rn(ar, x[u], acc[r][u]);
+    }
+}
+// ... for the rows that have k (a bit each).  They are chosen by a jump, not
+// by an `if` around each: the compiler turns those into predicates, and an
+// FP64 instruction holds its pipe for 64 cycles a warp even when no lane takes
+// part (a chain with every lane predicated off measured the time of a full
+// one).
+template <int R, int U0, int U1>
+__device__ __forceinline__ void fold_term(int rows, const double* __restrict__ a, const double (&x)[2],
+                                          const bool (&in)[2], double (&acc)[R][2]) {
+    if constexpr (R == 1) {
+        fold_rows<R, U0, U1, 0, 0>(a, x, in, acc);
+    } else {
+        static_assert(R == 4);
+        switch (rows) {
+            case 15: fold_rows<R, U0, U1, 0, 3>(a, x, in, acc); break;
+            case 1: fold_rows<R, U0, U1, 0, 0>(a, x, in, acc); break;
+            case 3: fold_rows<R, U0, U1, 0, 1>(a, x, in, acc); break;
+            case 7: fold_rows<R, U0, U1, 0, 2>(a, x, in, acc); break;
+            case 8: fold_rows<R, U0, U1, 3, 3>(a, x, in, acc); break;
+            case 12: fold_rows<R, U0, U1, 2, 3>(a, x, in, acc); break;
+            case 14: fold_rows<R, U0, U1, 1, 3>(a, x, in, acc); break;
+            case 2: fold_rows<R, U0, U1, 1, 1>(a, x, in, acc); break;
+            case 4: fold_rows<R, U0, U1, 2, 2>(a, x, in, acc); break;
+            case 6: fold_rows<R, U0, U1, 1, 2>(a, x, in, acc); break;
+            case 0: break;
+            default:  // rows with gaps between them
+                if (rows & 1) fold_rows<R, U0, U1, 0, 0>(a, x, in, acc);
+                if (rows & 2) fold_rows<R, U0, U1, 1, 1>(a, x, in, acc);
+                if (rows & 4) fold_rows<R, U0, U1, 2, 2>(a, x, in, acc);
+                if (rows & 8) fold_rows<R, U0, U1, 3, 3>(a, x, in, acc);
+                break;
+        }
+    }
+}
+
+// The columns gmin + lane + 32 u <= gmax of a group over the staged terms
+// [0, nt) in order, the pieces that B row k meets.
+template <int R, bool TEAM>
+__device__ __forceinline__ void fold_group(const BandStage<R, TEAM>& G, int nt, const double* __restrict__ val,
+                                           int gmin, int gmax, int lane, double (&acc)[R][2]) {
+    const double* const v = val + gmin + lane;
+#pragma unroll 1
+    for (int q = 0; q < nt; ++q) {
+        const int4 d = G.d[q];
+        if (d.y > gmax || d.z < gmin) continue;
+        double x[2];
+        bool in[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = gmin + lane + 32 * u;
+            in[u] = c >= d.y && c <= d.z;
+            if (in[u]) x[u] = v[(long long)d.x + 32 * u];
+        }
+        const double* a = G.a[q];
+        switch ((d.y < gmin + 32 ? 1 : 0) | (d.z >= gmin + 32 && gmax >= gmin + 32 ? 2 : 0)) {
+            case 3: fold_term<R, 0, 1>(d.w, a, x, in, acc); break;
+            case 1: fold_term<R, 0, 0>(d.w, a, x, in, acc); break;
+            case 2: fold_term<R, 1, 1>(d.w, a, x, in, acc); break;
+            default: break;
+        }
+    }
+}
+
+constexpr int kBandMaxRow = 1 << 20;   // columns of a row folded here
+constexpr int kBandMaxWork = 1 << 24;  // and entries of its terms
+
+template <bool BATCH>
+__device__ __noinline__ void general_row(const ProductArgs& P, const AddTerm* add, BandMap& S, RowState& st, int r,
+                                         int lane) {
+    product_row<false, BATCH, !BATCH, kBmWords>(P, add, S, st, r, lane);
+}
+
+// One row's columns gmin + lane + 32 u within [lo, hi] to pool positions
+// base + (column - lo), holes as exact zeros; FILT: Algorithm 1's first pass
+// as in k_product.  Returns the true entries.  (The pieces are a loop and not
+// two copies: with a copy for each of the tile's rows and pieces the kernel's
+// code outgrew its instruction cache.)
+template <bool FILT>
+__device__ __forceinline__ int write_group(const ProductArgs& P, CandArena& carena, long long base, int lo, int hi,
+                                           int gmin, const double (&acc)[2], unsigned long long r_eps, int r_lsb,
+                                           int lane, int& cand_n, unsigned long long& absmax) {
+    int nnz = 0;
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+        if (gmin + 32 * u > hi || gmin + 32 * u + 31 < lo) continue;
+        const int c = gmin + 32 * u + lane;
+        const bool in = c >= lo && c <= hi;
+        const double x = u ? acc[1] : acc[0];
+        const unsigned long long xb = mag_bits(x);
+        const bool nz = in && xb != 0ull;
+        if (in) {
+            P.pool_col[base + (c - lo)] = c;
+            P.pool_val[base + (c - lo)] = nz ? x : 0.0;
+        }
+        if (nz && xb > absmax) absmax = xb;
+        if constexpr (FILT) {
+            const bool cand = nz && xb <= r_eps;  // (r_eps 0: the row is not filtered)
+            if (cand) {
+                exact_add(P.words + c, (size_t)P.n, P.sticky + c, xb, r_lsb);
+                ++cand_n;
+            }
+            cand_push(carena, cand, c, xb, P.cand_col, P.cand_x, &P.ctl->cand_cnt[0], P.cand_cap, P.cand_chunk,
+                      &P.ctl->cand_over, lane);
+        }
+        nnz += __popc(__ballot_sync(kFull, nz));
+    }
+    return nnz;
+}
+
+// The descriptor of the row written at [base, base + total) with nnz true
+// entries: full while at least three quarters of its columns have one, else
+// its entries alone (by one warp).
+__device__ __forceinline__ void band_desc(const ProductArgs& P, int r, long long base, int total, int lo, int nnz,
+                                          int lane) {
+    // the row's unused reserved slots read as exact zeros (never candidates)
+    if (lane < (-total & 3)) P.pool_val[base + total + lane] = 0.0;
+    if (nnz == 0) {
+        if (lane == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
+    } else if (4ll * nnz >= 3ll * total) {
+        if (lane == 0) write_desc(P, r, rd_full_row((int)base, (int)base + total, lo, nnz));
+    } else {
+        __syncwarp();
+        compact_row(P.pool_col, P.pool_val, (int)base, (int)base + total, 0ull, lane);
+        __syncwarp();
+        if (lane == 0) write_desc(P, r, stored_row(P, base, nnz));
+    }
+}
+
+template <bool BATCH, bool TEAM, int R, bool FILT>
+__global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_constant__ ProductArgs P) {
+    if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
+    using Stage = BandStage<R, TEAM>;
+    constexpr int N = Stage::N;
+    constexpr int NT = TEAM ? kBandWarps * 32 : 32;  // threads of a tile
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    AddTerm* add = reinterpret_cast<AddTerm*>(smem_raw);
+    unsigned char* const mem = smem_raw + sizeof(AddTerm) * kMaxAdd;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int tid = TEAM ? (int)threadIdx.x : lane;
+    const bool lead = !TEAM || wib == 0;
+    BandMap& S = reinterpret_cast<BandMap*>(mem)[TEAM ? 0 : wib];
+    Stage& G = *reinterpret_cast<Stage*>(&S);
+    __shared__ long long s_base;
+    __shared__ int s_lo[R], s_hi[R], s_nnz[R], s_ok;
+    __shared__ unsigned s_sum[R];
+    const int nadd = P.nadd;
+    for (int t = threadIdx.x; t < nadd; t += blockDim.x) add[t] = P.add[t];
+    __syncthreads();
+    auto sync = [] {
+        if constexpr (TEAM) __syncthreads();
+        else __syncwarp();
+    };
+    RowState st;
+    // tiles are handed out as warps (blocks) come free: their work differs by
+    // an order of magnitude in a batch, and a matrix has a few per warp.  The
+    // next one's number is fetched while this one is computed.
+    const int tiles = (P.n + R - 1) / R;
+    const int first = TEAM ? gridDim.x : gridDim.x * kBandWarps;
+    __shared__ int s_next;
+    int tile = TEAM ? blockIdx.x : blockIdx.x * kBandWarps + wib;
+    while (tile < tiles) {
+        int next = 0;
+        if (lead && lane == 0) next = first + (int)atomicAdd(P.ticket, 1u);
+        const int r0 = tile * R;
+        // ---- lane i < R: row r0 + i's part of A, and what becomes of it (1:
+        // folded here, 2: by the accumulator, 0: done)
+        int my_kind = 0, my_inst = 0, my_pa = 0, my_k = 0, my_na = 0;
+        bool my_holes = false;
+        if (lane < R && r0 + lane < P.n) {
+            const int r = r0 + lane;
+            my_kind = 1;
+            bool prod = P.A.rb != nullptr;
+            if constexpr (BATCH) {
+                my_inst = P.inst[r];
+                if (!P.band[my_inst]) {
+                    my_kind = 0;
+                } else {
+                    const BatchStep& bs = P.bstep[my_inst];
+                    if (bs.reuse && __ldcg(P.inst_dropped + my_inst) == 0) {
+                        my_kind = 0;  // k_reuse_copy_batch writes it
+                    } else if (bs.mode == kBatchSkip || bs.mode == kBatchPass) {
+                        if (lead) write_desc(P, r, bs.mode == kBatchPass ? P.B.rd[r] : RowDesc{0, 0, 0, 0});
+                        my_kind = 0;
+                    }
+                    prod = bs.mode == kBatchProduct;
+                }
+            }
+            if (my_kind && prod) {
+                my_pa = P.A.rb[r];
+                my_na = P.A.re[r] - my_pa;
+                if (my_na > 0) {
+                    if (P.A.rd) {
+                        const RowDesc d = P.A.rd[r];
+                        my_k = rd_first(d);
+                        my_holes = my_na != rd_nnz(d);
+                        if (!rd_full(d)) my_kind = 2;
+                    } else {
+                        my_k = P.A.col[my_pa];  // (a caller's row: consecutive, checked on input)
+                    }
+                }
+            }
+        }
+        unsigned todo = __ballot_sync(kFull, my_kind == 1), late = __ballot_sync(kFull, my_kind == 2);
+        bool joint = true;
+        while (todo) {
+            const unsigned m = joint ? todo : todo & (0u - todo);  // rows folded together
+            const bool mine = lane < R && ((m >> lane) & 1u);
+            const bool many = (m & (m - 1u)) != 0u;
+            const int kb = warp_min(mine && my_na > 0 ? my_k : INT_MAX);
+            const int ke = max(kb, warp_max(mine && my_na > 0 ? my_k + my_na : 0));
+            const int nk = kb == INT_MAX ? 0 : ke - kb;
+            if (many && nk > warp_sum(mine ? min(my_na, 1 << 24) : 0) + 32) {
+                joint = false;  // ranges of A far apart
+                continue;
+            }
+            // ---- the terms: stage them; the rows' column ranges and work
+            int kf[R], kn[R], pa[R];
+            unsigned holes = __ballot_sync(kFull, my_holes);
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                kf[i] = __shfl_sync(kFull, my_k, i);
+                kn[i] = (m >> i) & 1u ? __shfl_sync(kFull, my_na, i) : (__shfl_sync(kFull, my_na, i), 0);
+                pa[i] = __shfl_sync(kFull, my_pa, i);
+            }
+            // (entries of the terms, holes included, saturating at 2^24 a thread;
+            // multiply-adds, exact below that)
+            int lo[R], hi[R];
+            unsigned sum[R], fma[R];
+            unsigned bad = 0u;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                lo[i] = INT_MAX;
+                hi[i] = -1;
+                sum[i] = fma[i] = 0u;
+            }
+            auto stage = [&](int q0, int q1, bool count) {  // k of [kb + q0, kb + q1)
+                for (int q = q0 + tid; q < q1; q += NT) {
+                    const int k = kb + q;
+                    const RowDesc d = P.B.rd[k];
+                    const int f = rd_first(d), len = d.re - d.rb;
+                    unsigned rows = 0u;
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        const int at = k - kf[i];
+                        const bool in = (unsigned)at < (unsigned)kn[i];
+                        const double a = in ? P.A.val[pa[i] + at] : 0.0;
+                        G.a[q - q0][i] = a;
+                        if (in && !((holes >> i & 1u) && a == 0.0) && len > 0) {
+                            rows |= 1u << i;
+                            if (count) {
+                                lo[i] = min(lo[i], f);
+                                hi[i] = max(hi[i], f + len - 1);
+                                sum[i] = min(sum[i] + (unsigned)min(len, kBandMaxWork), (unsigned)kBandMaxWork);
+                                fma[i] += (unsigned)rd_nnz(d);
+                                if (!rd_full(d)) bad |= 1u << i;
+                            }
+                        }
+                    }
+                    G.d[q - q0] = make_int4(d.rb - f, len > 0 ? f : INT_MAX, f + len - 1, (int)rows);
+                }
+            };
+            if constexpr (TEAM) {
+                __syncthreads();
+                if (threadIdx.x < R) {
+                    s_lo[threadIdx.x] = INT_MAX;
+                    s_hi[threadIdx.x] = -1;
+                    s_sum[threadIdx.x] = s_nnz[threadIdx.x] = 0;
+                    if (threadIdx.x == 0) s_ok = 0;
+                }
+            }
+            for (int q0 = 0; q0 < nk; q0 += N) {
+                sync();
+                stage(q0, min(nk, q0 + N), true);
+            }
+            if (lead)
+                for (int x = lane; x < nadd * R; x += 32) {
+                    const int t = x / R, i = x - t * R;
+                    if (!((m >> i) & 1u)) continue;
+                    if (BATCH && __double_as_longlong(P.alpha_tab[(size_t)t * P.ninst + P.inst[r0 + i]]) == 0ll) continue;
+                    int f = r0 + i, l = f, len = 1, nnz = 1;
+                    bool full = true;
+                    if (add[t].rd) {
+                        const RowDesc d = add[t].rd[r0 + i];
+                        len = d.re - d.rb;
+                        if (len <= 0) continue;
+                        f = rd_first(d);
+                        l = rd_last(d);
+                        nnz = rd_nnz(d);
+                        full = rd_full(d);
+                    }
+#pragma unroll
+                    for (int e = 0; e < R; ++e)
+                        if (e == i) {
+                            lo[e] = min(lo[e], f);
+                            hi[e] = max(hi[e], l);
+                            sum[e] = min(sum[e] + (unsigned)min(len, kBandMaxWork), (unsigned)kBandMaxWork);
+                            fma[e] += (unsigned)nnz;
+                            if (!full) bad |= 1u << e;
+                        }
+                }
+            bad = __reduce_or_sync(kFull, bad);
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                lo[i] = warp_min(lo[i]);
+                hi[i] = warp_max(hi[i]);
+                sum[i] = __reduce_add_sync(kFull, sum[i]);
+            }
+            if constexpr (TEAM) {
+                __syncthreads();
+                if (lane == 0) {
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        atomicMin(&s_lo[i], lo[i]);
+                        atomicMax(&s_hi[i], hi[i]);
+                        atomicAdd(&s_sum[i], sum[i]);
+                    }
+                    if (bad) atomicOr(&s_ok, (int)bad);
+                }
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    lo[i] = s_lo[i];
+                    hi[i] = s_hi[i];
+                    sum[i] = s_sum[i];
+                }
+                bad = (unsigned)s_ok;
+            }
+            unsigned fold = 0u;
+            int glo = INT_MAX, ghi = -1;
+            long long width = 0;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                if (!((m >> i) & 1u) || hi[i] < lo[i]) continue;
+                const int total = hi[i] - lo[i] + 1;
+                if ((bad >> i & 1u) || total > kBandMaxRow || (unsigned)total > sum[i] || sum[i] >= (unsigned)kBandMaxWork) {
+                    bad |= 1u << i;
+                    continue;
+                }
+                fold |= 1u << i;
+                glo = min(glo, lo[i]);
+                ghi = max(ghi, hi[i]);
+                width += total;
+            }
+            if (many && ghi - glo + 1 > width) {
+                joint = false;  // columns far apart
+                continue;
+            }
+            // ---- settled: the empty rows, the accumulator's rows
+            int need = 0, at[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                at[i] = need;
+                if (!((m >> i) & 1u)) continue;
+                if (hi[i] < lo[i]) {
+                    if (lead && lane == 0) write_desc(P, r0 + i, RowDesc{0, 0, 0, 0});
+                    if constexpr (!BATCH) st.fma += fma[i];
+                } else if (bad >> i & 1u) {
+                    late |= 1u << i;
+                } else {
+                    need += (hi[i] - lo[i] + 4) & ~3;
+                    if constexpr (!BATCH) st.fma += fma[i];
+                    st.span = max(st.span, hi[i] - lo[i] + 1);
+                }
+            }
+            long long base = 0;
+            if (fold) {
+                if (lead) base = arena_take(st.arena, (unsigned long long)need, P.arena, P.ctl, P.pool_val, lane);
+                if constexpr (TEAM) {
+                    if (threadIdx.x == 0) s_base = base;
+                    __syncthreads();
+                    base = s_base;
+                }
+                if (base < 0) {  // the pool is full (recorded): the phase is run again
+                    if (lead && lane < R && (fold >> lane & 1u)) write_desc(P, r0 + lane, RowDesc{0, 0, 0, 0});
+                    fold = 0u;
+                }
+            }
+            if (fold) {
+                sync();
+                int nnz[R], cand[BATCH ? R : 1];
+                unsigned long long amax[BATCH ? R : 1];  // per row in a batch, else the thread's totals
+                if constexpr (!BATCH) {
+                    cand[0] = (int)st.cand;
+                    amax[0] = st.absmax;
+                }
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    nnz[i] = 0;
+                    if constexpr (BATCH) {
+                        cand[i] = 0;
+                        amax[i] = 0ull;
+                    }
+                }
+                const int groups = (ghi - glo + 64) >> 6;
+                for (int g0 = 0; g0 < groups; g0 += TEAM ? kBandWarps : 1) {
+                    const int gmin = glo + 64 * (g0 + (TEAM ? wib : 0)), gmax = min(ghi, gmin + 63);
+                    double acc[R][2];
+#pragma unroll
+                    for (int i = 0; i < R; ++i) acc[i][0] = acc[i][1] = 0.0;
+                    if (gmin <= gmax) {
+                        // the addends, t ascending
+                        for (int t = 0; t < nadd; ++t) {
+#pragma unroll
+                            for (int i = 0; i < R; ++i) {
+                                if (!(fold >> i & 1u)) continue;
+                                const int r = r0 + i;
+                                const double alpha = BATCH ? P.alpha_tab[(size_t)t * P.ninst + __shfl_sync(kFull, my_inst, i)]
+                                                           : add[t].alpha;
+                                if (BATCH && __double_as_longlong(alpha) == 0ll) continue;
+                                if (!add[t].rd) {
+#pragma unroll
+                                    for (int u = 0; u < 2; ++u)
+                                        if (gmin + lane + 32 * u == r) acc[i][u] = __fma_rn(alpha, 1.0, acc[i][u]);
+                                    continue;
+                                }
+                                const RowDesc d = add[t].rd[r];
+                                const int f = rd_first(d), l = f + (d.re - d.rb) - 1;
+                                if (f > gmax || l < gmin) continue;
+#pragma unroll
+                                for (int u = 0; u < 2; ++u) {
+                                    const int c = gmin + lane + 32 * u;
+                                    if (c >= f && c <= l) acc[i][u] = __fma_rn(alpha, P.pool_val[d.rb + (c - f)], acc[i][u]);
+                                }
+                            }
+                        }
+                    }
+                    // the product, k ascending
+                    for (int q0 = 0; q0 < nk; q0 += N) {
+                        if (nk > N) {
+                            sync();
+                            stage(q0, min(nk, q0 + N), false);
+                            sync();
+                        }
+                        if (gmin > gmax) continue;
+                        fold_group<R, TEAM>(G, min(nk - q0, N), P.pool_val, gmin, gmax, lane, acc);
+                    }
+                    if (gmin > gmax) continue;
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        if (!(fold >> i & 1u)) continue;
+                        unsigned long long r_eps = (unsigned long long)__double_as_longlong(P.eps_g);
+                        int r_lsb = P.e_lsb;
+                        if constexpr (BATCH && FILT) {
+                            const BatchStep& bs = P.bstep[__shfl_sync(kFull, my_inst, i)];
+                            r_eps = (unsigned long long)__double_as_longlong(bs.eps_g);
+                            r_lsb = bs.e_lsb;
+                        }
+                        nnz[i] += write_group<FILT>(P, st.carena, base + at[i], lo[i], hi[i], gmin, acc[i], r_eps, r_lsb,
+                                                    lane, cand[BATCH ? i : 0], amax[BATCH ? i : 0]);
+                    }
+                }
+                if constexpr (!BATCH) {
+                    st.cand = (unsigned long long)cand[0];
+                    st.absmax = amax[0];
+                }
+                if constexpr (TEAM) {
+                    if (lane == 0) {
+#pragma unroll
+                        for (int i = 0; i < R; ++i)
+                            if (nnz[i]) atomicAdd(&s_nnz[i], nnz[i]);
+                    }
+                    __syncthreads();
+#pragma unroll
+                    for (int i = 0; i < R; ++i) nnz[i] = s_nnz[i];
+                }
+                if (lead) {
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        if (!(fold >> i & 1u)) continue;
+                        band_desc(P, r0 + i, base + at[i], hi[i] - lo[i] + 1, lo[i], nnz[i], lane);
+                        if (!BATCH && lane == 0) st.written += (unsigned long long)nnz[i];
+                    }
+                }
+                if constexpr (BATCH) {
+                    // lane i adds row i's candidates, entries and largest |x|
+                    // to its instance's record
+                    int my_cand = 0, my_nnz = 0, my_span = 0;
+                    unsigned long long my_max = 0ull;
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        const int ci = FILT ? warp_sum(cand[i]) : 0;
+                        const unsigned long long mi = P.absmax_slot ? warp_max_u64(amax[i]) : 0ull;
+                        if (lane == i && (fold >> i & 1u)) {
+                            my_cand = ci;
+                            my_max = mi;
+                            my_nnz = nnz[i];
+                            my_span = hi[i] - lo[i] + 1;
+                        }
+                    }
+                    if (my_nnz > 0) {
+                        if (P.stat_tab) {
+                            StepStat* rec = P.stat_tab + my_inst;
+                            atomicAdd(&rec->nnz_pre, (unsigned long long)my_nnz);
+                            if (my_cand) atomicAdd(&rec->ncand, (unsigned long long)my_cand);
+                            atomicMax(&rec->span_max, (unsigned)my_span);
+                        }
+                        if (my_max) atomicMax(&(P.absmax_slot + (size_t)my_inst * P.absmax_stride)->absmax, my_max);
+                    }
+                }
+            }
+            if constexpr (BATCH) {  // the multiply-adds of the rows settled here
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const unsigned f = __reduce_add_sync(kFull, fma[i]);
+                    if (lane == i && ((m & ~bad) >> i & 1u) && f && P.stat_tab)
+                        atomicAdd(&P.stat_tab[my_inst].fma, (unsigned long long)f);
+                }
+            }
+            todo &= ~m;
+        }
+        if (late) {
+            sync();
+            if (lead)
+                while (late) {
+                    const int i = __ffs(late) - 1;
+                    late &= late - 1u;
+                    general_row<BATCH>(P, add, S, st, r0 + i, lane);
+                    __syncwarp();
+                }
+        }
+        if constexpr (TEAM) {
+            if (threadIdx.x == 0) s_next = next;
+            __syncthreads();  // the tile's memory is free
+            tile = s_next;
+            __syncthreads();
+        } else {
+            tile = __shfl_sync(kFull, next, 0);
+        }
+    }
+    if (lead) arena_close(st.arena, P.pool_val, lane);
+    if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
+    if constexpr (BATCH) return;
+    // ---- the step statistics, once per block
+    __shared__ unsigned long long blk_written, blk_cand, blk_absmax, blk_fma;
+    __shared__ int blk_span;
+    if (threadIdx.x == 0) {
+        blk_written = blk_cand = blk_absmax = blk_fma = 0ull;
+        blk_span = 0;
+    }
+    __syncthreads();
+    st.cand = (unsigned long long)warp_sum((int)st.cand);
+    st.absmax = warp_max_u64(st.absmax);
+    st.written = __shfl_sync(kFull, st.written, 0);
+    for (int o = 16; o; o >>= 1) st.fma += __shfl_xor_sync(kFull, st.fma, o);
+    if (lane == 0) {
+        atomicAdd(&blk_fma, st.fma);
+        atomicAdd(&blk_written, st.written);
+        atomicAdd(&blk_cand, st.cand);
+        atomicMax(&blk_absmax, st.absmax);
+        atomicMax(&blk_span, st.span);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (blk_fma) atomicAdd(&P.ctl->fma_total, blk_fma);
+        if (P.stat) {
+            if (blk_span > 0) atomicMax(&P.stat->span_max, (unsigned)blk_span);
+            if (blk_fma) atomicAdd(&P.stat->fma, blk_fma);
+            if (blk_written) atomicAdd(&P.stat->nnz_pre, blk_written);
+            if (blk_cand) atomicAdd(&P.stat->ncand, blk_cand);
+        }
+        if (P.absmax_slot && blk_absmax) atomicMax(&P.absmax_slot->absmax, blk_absmax);
+    }
+}
+size_t band_smem_bytes() { return sizeof(AddTerm) * kMaxAdd + sizeof(BandMap) * kBandWarps; }
 
 // ---------------------------------------------------------------- k_reuse_pass1
 // A baby step Z-hat_(k) = filter(Z Z-hat_(k-1)) while no earlier step has
@@ -1602,20 +2305,20 @@ __global__ void __launch_bounds__(256) k_reuse_copy_batch(ProductArgs P) {
         const BatchStep bs = P.bstep[i];
         if (!bs.reuse || __ldcg(P.inst_dropped + i) != 0) continue;
         unsigned long long fma = 0ull;
-        for (int p = P.A.rb[r] + lane; p < P.A.re[r]; p += 32) {
-            const int k = P.A.col[p];
-            fma += (unsigned long long)(P.B.re[k] - P.B.rb[k]);
-        }
+        const int pa0 = P.A.rb[r], pa1 = P.A.re[r];
+        const bool a_holes = pa1 - pa0 != rd_nnz(P.A.rd[r]);
+        for (int p = pa0 + lane; p < pa1; p += 32)
+            if (!(a_holes && P.A.val[p] == 0.0)) fma += (unsigned long long)rd_nnz(P.B.rd[P.A.col[p]]);
         const int s = P.power.rb[r], len = P.power.re[r] - s;
         if (len <= 0) {
-            if (lane == 0) P.out_rb[r] = P.out_re[r] = 0;
+            if (lane == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
             row_stats_batch(P, i, fma, 0ull, 0, 0ull, lane);
             continue;
         }
         const unsigned long long span = ((unsigned long long)len + 3ull) & ~3ull;
         const long long base = arena_take(arena, span, P.arena, P.ctl, P.pool_val, lane);
         if (base < 0) {
-            if (lane == 0) P.out_rb[r] = P.out_re[r] = 0;
+            if (lane == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
             continue;
         }
         const bool filt = bs.eps_g > 0.0;
@@ -1641,11 +2344,11 @@ __global__ void __launch_bounds__(256) k_reuse_copy_batch(ProductArgs P) {
                           &P.ctl->cand_over, lane);
         }
         for (long long q = base + len + lane; q < base + (long long)span; q += 32) P.pool_val[q] = 0.0;
-        if (lane == 0) {
-            P.out_rb[r] = (int)base;
-            P.out_re[r] = (int)(base + len);
-        }
-        row_stats_batch(P, i, fma, cand, len, 0ull, lane);
+        RowDesc d = P.power.rd[r];
+        d.rb = (int)base;
+        d.re = (int)(base + len);
+        if (lane == 0) write_desc(P, r, d);
+        row_stats_batch(P, i, fma, cand, rd_nnz(d), 0ull, lane);
     }
     arena_close(arena, P.pool_val, lane);
     if (P.cand_col) cand_close(carena, P.cand_x, lane);
@@ -1900,12 +2603,8 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
     const unsigned long long fb = (unsigned long long)__double_as_longlong(eps_f);
     unsigned long long kept = 0ull;
     for (int r = gw; r < A.n; r += nwarps) {
-        const int s = A.rb[r], e = A.re[r];
-        const int w = compact_row(A.col, A.val, s, e, fb, lane);
-        if (lane == 0) {
-            A.re[r] = w;
-            kept += (unsigned long long)(w - s);
-        }
+        const int k = filter_row(A.col, A.val, A.rb, A.re, A.rd, r, fb, lane);
+        if (lane == 0) kept += (unsigned long long)k;
     }
     if (lane == 0 && kept) atomicAdd(&A.stat->nnz_post, kept);
     if (gt == 0) {
@@ -2228,12 +2927,8 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1_batch(A
         const int i = A.inst[r];
         if (s_state[i] != 1 || !(s_c[i] > 0.0)) continue;
         const unsigned long long fb = (unsigned long long)__double_as_longlong(s_eps[i]);
-        const int s = A.rb[r], e = A.re[r];
-        const int w = compact_row(A.col, A.val, s, e, fb, lane);
-        if (lane == 0) {
-            A.re[r] = w;
-            if (w > s) atomicAdd(&A.stat_tab[i].nnz_post, (unsigned long long)(w - s));
-        }
+        const int k = filter_row(A.col, A.val, A.rb, A.re, A.rd, r, fb, lane);
+        if (lane == 0 && k) atomicAdd(&A.stat_tab[i].nnz_post, (unsigned long long)k);
     }
 }
 
@@ -2585,12 +3280,14 @@ __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, co
                 }
                 prev = c;
             }
+            if (e > s && prev - col[s] != e - s - 1) ctl->not_band = 1;
         }
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
 }
 
-// Exclusive scan of row lengths re - rb into rowptr (n + 1 entries), in
+// Exclusive scan of row lengths (re - rb, or a pooled matrix's true entries
+// when rd is given) into rowptr (n + 1 entries), in
 // three launches over tiles of kScanTile rows: tile sums, a scan of the tile
 // sums (one block), and the scan inside each tile plus its tile's offset.
 // `sums` holds ceil(n / kScanTile) + 1 values.
@@ -2621,10 +3318,11 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long* par
     return before + x - v;
 }
 
-__global__ void __launch_bounds__(kScanTile) k_scan_tile_sums(int n, const int* rb, const int* re, long long* sums) {
+__global__ void __launch_bounds__(kScanTile) k_scan_tile_sums(int n, const int* rb, const int* re, const RowDesc* rd,
+                                                              long long* sums) {
     __shared__ long long part[32];
     const long long r = (long long)blockIdx.x * kScanTile + threadIdx.x;
-    const long long len = r < n ? (long long)(re[r] - rb[r]) : 0;
+    const long long len = r < n ? (long long)(rd ? rd_nnz(rd[r]) : re[r] - rb[r]) : 0;
     long long total;
     block_excl_scan(len, part, &total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
@@ -2650,35 +3348,55 @@ __global__ void __launch_bounds__(kScanTile) k_scan_tiles(int ntiles, long long*
     }
 }
 
-__global__ void __launch_bounds__(kScanTile) k_scan_apply(int n, const int* rb, const int* re, const long long* sums,
-                                                           int* rowptr) {
+__global__ void __launch_bounds__(kScanTile) k_scan_apply(int n, const int* rb, const int* re, const RowDesc* rd,
+                                                           const long long* sums, int* rowptr) {
     __shared__ long long part[32];
     const long long r = (long long)blockIdx.x * kScanTile + threadIdx.x;
-    const long long len = r < n ? (long long)(re[r] - rb[r]) : 0;
+    const long long len = r < n ? (long long)(rd ? rd_nnz(rd[r]) : re[r] - rb[r]) : 0;
     long long total;
     const long long ex = block_excl_scan(len, part, &total) + sums[blockIdx.x];
     if (r < n) rowptr[r] = (int)ex;  // the host rejects totals of 2^31 and more
     if (r == n - 1 || (n == 0 && r == 0)) rowptr[n] = (int)sums[gridDim.x];
 }
 
+// A row's true entries to col/val at d on, columns less `shift`, by one warp.
+__device__ __forceinline__ void gather_row(const RowView& src, int r, long long d, int shift, int* col, double* val,
+                                           int lane) {
+    const RowDesc rd = src.rd[r];
+    const int s = rd.rb, len = rd.re - s;
+    if (rd_nnz(rd) == len) {
+        for (int q = lane; q < len; q += 32) {
+            col[d + q] = src.col[s + q] - shift;
+            val[d + q] = src.val[s + q];
+        }
+        return;
+    }
+    for (int q0 = 0; q0 < len; q0 += 32) {  // without the holes
+        const int q = q0 + lane;
+        const double x = q < len ? src.val[s + q] : 0.0;
+        const bool nz = mag_bits(x) != 0ull;
+        const unsigned m = __ballot_sync(kFull, nz);
+        if (nz) {
+            const long long at = d + __popc(m & lanemask_lt());
+            col[at] = src.col[s + q] - shift;
+            val[at] = x;
+        }
+        d += __popc(m);
+    }
+}
+
 __global__ void k_gather(int n, RowView src, const int* rowptr, int* col, double* val) {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int r = gw; r < n; r += nwarps) {
-        int s = src.rb[r], e = src.re[r], d = rowptr[r];
-        for (int q = lane; q < e - s; q += 32) {
-            col[d + q] = src.col[s + q];
-            val[d + q] = src.val[s + q];
-        }
-    }
+    for (int r = gw; r < n; r += nwarps) gather_row(src, r, rowptr[r], 0, col, val, lane);
 }
 
 // Copy a canonical CSR matrix into the pool: each row gets a 4-entry aligned
 // slot of round-up(len, 4) entries (rows start 16-byte aligned, like the
 // product kernel's rows).
 __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
-                            int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size) {
+                            RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size) {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -2687,7 +3405,10 @@ __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const doub
         int s = rowptr[r], e = rowptr[r + 1];
         const long long base = arena_take(arena, (unsigned long long)((e - s + 3) & ~3), arena_size, ctl, pool_val, lane);
         if (base < 0) {
-            if (lane == 0) rb[r] = re[r] = 0;
+            if (lane == 0) {
+                rb[r] = re[r] = 0;
+                rd[r] = RowDesc{0, 0, 0, 0};
+            }
             continue;
         }
         const int padded = (e - s + 3) & ~3;
@@ -2698,6 +3419,7 @@ __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const doub
         if (lane == 0) {
             rb[r] = (int)base;
             re[r] = (int)base + (e - s);
+            rd[r] = rd_row((int)base, (int)base + (e - s), e > s ? col[s] : 0, e > s ? col[e - 1] : 0);
         }
     }
     arena_close(arena, pool_val, lane);
@@ -2739,7 +3461,8 @@ __global__ void k_inst_table(int n, int ninst, const int* off, int* inst) {
 }
 
 // Check every input of a batch like k_validate: thread per global row.
-__global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, const int* nnz, Ctl* ctl) {
+__global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, const int* nnz, Ctl* ctl,
+                                 unsigned char* band) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int i = inst[r];
@@ -2762,6 +3485,7 @@ __global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, co
             }
             prev = c;
         }
+        if (e > s && prev - S.col[s] != e - s - 1) band[i] = 0;
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
 }
@@ -2769,8 +3493,8 @@ __global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, co
 // Copy the inputs of a batch into the pool as the block-diagonal matrix
 // (columns shifted to global), rows padded to 4 entries; records each
 // instance's max |x| in absmax[i * stride].
-__global__ void k_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, int* pool_col,
-                                  double* pool_val, Ctl* ctl, unsigned long long arena_size, NormSlot* absmax,
+__global__ void k_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, RowDesc* rd,
+                                  int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size, NormSlot* absmax,
                                   int stride) {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2783,7 +3507,10 @@ __global__ void k_copy_rows_batch(int n, const int* inst, const BatchSrc* src, i
         const int s = S.rowptr[l], e = S.rowptr[l + 1];
         const long long base = arena_take(arena, (unsigned long long)((e - s + 3) & ~3), arena_size, ctl, pool_val, lane);
         if (base < 0) {
-            if (lane == 0) rb[r] = re[r] = 0;
+            if (lane == 0) {
+                rb[r] = re[r] = 0;
+                rd[r] = RowDesc{0, 0, 0, 0};
+            }
             continue;
         }
         const int padded = (e - s + 3) & ~3;
@@ -2800,23 +3527,26 @@ __global__ void k_copy_rows_batch(int n, const int* inst, const BatchSrc* src, i
         if (lane == 0) {
             rb[r] = (int)base;
             re[r] = (int)base + (e - s);
+            rd[r] = rd_row((int)base, (int)base + (e - s), e > s ? S.col[s] + S.off : 0,
+                           e > s ? S.col[e - 1] + S.off : 0);
             if (absmax && mx) atomicMax(&absmax[(size_t)i * stride].absmax, mx);
         }
     }
     arena_close(arena, pool_val, lane);
 }
 
-// out rows <- the rows of matrix sel[inst[r]] of a table of row arrays.
+// out rows <- the rows of matrix sel[inst[r]] of a table of row descriptors.
 struct RowTable {
-    const int* rb[kMaxAdd + 2];
-    const int* re[kMaxAdd + 2];
+    const RowDesc* rd[kMaxAdd + 2];
 };
-__global__ void k_compose_rows(int n, const int* inst, const int* sel, RowTable T, int* out_rb, int* out_re) {
+__global__ void k_compose_rows(int n, const int* inst, const int* sel, RowTable T, int* out_rb, int* out_re,
+                               RowDesc* out_rd) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const int k = sel[inst[r]];
-    out_rb[r] = T.rb[k][r];
-    out_re[r] = T.re[k][r];
+    const RowDesc d = T.rd[sel[inst[r]]][r];
+    out_rb[r] = d.rb;
+    out_re[r] = d.re;
+    out_rd[r] = d;
 }
 
 // Split the block-diagonal result (global row pointers rowptr) into the
@@ -2834,12 +3564,9 @@ __global__ void k_gather_batch(int n, int ninst, const int* inst, const int* off
     for (int r = gw; r < n; r += nwarps) {
         const int i = inst[r];
         const int o = off[i];
-        const int s = src.rb[r], e = src.re[r], d = rowptr[r];
+        const int d = rowptr[r];
         if (lane == 0) out_rp[r + i] = d - rowptr[o];
-        for (int q = lane; q < e - s; q += 32) {
-            col[d + q] = src.col[s + q] - o;
-            val[d + q] = src.val[s + q];
-        }
+        gather_row(src, r, d, o, col, val, lane);
     }
 }
 
@@ -2913,6 +3640,16 @@ cudaError_t kernels_init() {
     err = cudaFuncSetAttribute((const void*)k_product_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)cta_smem_bytes());
     if (err != cudaSuccess) return err;
+    const void* bands[10] = {
+        (const void*)k_band<false, false, 1, false>, (const void*)k_band<false, false, 4, false>,
+        (const void*)k_band<false, true, 1, false>,  (const void*)k_band<false, true, 4, false>,
+        (const void*)k_band<true, false, 4, false>,  (const void*)k_band<false, false, 1, true>,
+        (const void*)k_band<false, false, 4, true>,  (const void*)k_band<false, true, 1, true>,
+        (const void*)k_band<false, true, 4, true>,   (const void*)k_band<true, false, 4, true>};
+    for (const void* k : bands) {
+        err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)band_smem_bytes());
+        if (err != cudaSuccess) return err;
+    }
     err = cudaFuncSetAttribute((const void*)k_norms_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)norms_rows_smem_bytes());
     if (err != cudaSuccess) return err;
@@ -2974,6 +3711,34 @@ cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, do
     return prod_launch<false, false, false>(P, st);
 }
 
+template <bool BATCH, bool TEAM, int R>
+static void band_launch(const ProductArgs& P, cudaStream_t st) {
+    const long long cap = (long long)sms_now() * 7, tiles = ((long long)P.n + R - 1) / R;
+    const long long blocks = TEAM ? tiles : (tiles + kBandWarps - 1) / kBandWarps;
+    const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
+    // (a batch's rows may be filtered when candidate lists are given)
+    const bool filt = P.cand_col != nullptr;
+    if (filt) k_band<BATCH, TEAM, R, true><<<grid, kBandWarps * 32, band_smem_bytes(), st>>>(P);
+    else k_band<BATCH, TEAM, R, false><<<grid, kBandWarps * 32, band_smem_bytes(), st>>>(P);
+}
+
+cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
+    if (P.n <= 0) return cudaSuccess;
+    const long long warps = (long long)sms_now() * 7 * kBandWarps;
+    const bool team = row_len > 192.0 || (P.n <= warps / kBandWarps && row_len > 64.0);
+    if (P.inst) {
+        band_launch<true, false, 4>(P, st);
+    } else if (team) {
+        if (P.n >= 2 * warps / kBandWarps * 4) band_launch<false, true, 4>(P, st);
+        else band_launch<false, true, 1>(P, st);
+    } else {
+        if (P.n >= 2 * warps * 4) band_launch<false, false, 4>(P, st);
+        else band_launch<false, false, 1>(P, st);
+    }
+    ++g_launches;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bits, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     long long blocks = ((long long)n + 7) / 8;
@@ -3020,11 +3785,11 @@ cudaError_t launch_validate(int n, int nnz, const int* rowptr, const int* col, c
 
 size_t scan_scratch_len(int n) { return (size_t)((n + kScanTile - 1) / kScanTile) + 2; }
 
-cudaError_t launch_scan_rows(int n, const int* rb, const int* re, int* rowptr, Ctl* ctl, long long* sums,
-                             cudaStream_t st) {
+cudaError_t launch_scan_rows(int n, const int* rb, const int* re, const RowDesc* rd, int* rowptr, Ctl* ctl,
+                             long long* sums, cudaStream_t st) {
     const int ntiles = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
     if (n > 0) {
-        k_scan_tile_sums<<<ntiles, kScanTile, 0, st>>>(n, rb, re, sums);
+        k_scan_tile_sums<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums);
         ++g_launches;
     } else {
         cudaError_t err = cudaMemsetAsync(sums, 0, sizeof(long long), st);
@@ -3032,7 +3797,7 @@ cudaError_t launch_scan_rows(int n, const int* rb, const int* re, int* rowptr, C
     }
     k_scan_tiles<<<1, kScanTile, 0, st>>>(ntiles, sums, ctl);
     ++g_launches;
-    k_scan_apply<<<ntiles, kScanTile, 0, st>>>(n, rb, re, sums, rowptr);
+    k_scan_apply<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums, rowptr);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -3084,14 +3849,15 @@ cudaError_t launch_identity(int n, double alpha, int* rowptr, int* col, double* 
 }
 
 cudaError_t launch_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
-                             int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
+                             RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
                              cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     // about four rows per warp: each row is a dependent load pair, so the
     // copy is latency-bound and wants many warps in flight
     long long blocks = ((long long)n + 31) / 32;
     if (blocks > (long long)sms_now() * 8) blocks = (long long)sms_now() * 8;
-    k_copy_rows<<<(unsigned)blocks, 256, 0, st>>>(n, rowptr, col, val, rb, re, pool_col, pool_val, ctl, arena_size);
+    k_copy_rows<<<(unsigned)blocks, 256, 0, st>>>(n, rowptr, col, val, rb, re, rd, pool_col, pool_val, ctl,
+                                                  arena_size);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -3126,35 +3892,32 @@ cudaError_t launch_inst_table(int n, int ninst, const int* off, int* inst, cudaS
 }
 
 cudaError_t launch_validate_batch(int n, const int* inst, const BatchSrc* src, const int* nnz, Ctl* ctl,
-                                  cudaStream_t st) {
+                                  unsigned char* band, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_validate_batch<<<(n + 255) / 256, 256, 0, st>>>(n, inst, src, nnz, ctl);
+    k_validate_batch<<<(n + 255) / 256, 256, 0, st>>>(n, inst, src, nnz, ctl, band);
     ++g_launches;
     return cudaGetLastError();
 }
 
-cudaError_t launch_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, int* pool_col,
-                                   double* pool_val, Ctl* ctl, unsigned long long arena_size, NormSlot* absmax,
+cudaError_t launch_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, RowDesc* rd,
+                                   int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size, NormSlot* absmax,
                                    int stride, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     int blocks = (n + 7) / 8;
     if (blocks > sms_now() * 8) blocks = sms_now() * 8;
-    k_copy_rows_batch<<<blocks, 256, 0, st>>>(n, inst, src, rb, re, pool_col, pool_val, ctl, arena_size, absmax,
+    k_copy_rows_batch<<<blocks, 256, 0, st>>>(n, inst, src, rb, re, rd, pool_col, pool_val, ctl, arena_size, absmax,
                                               stride);
     ++g_launches;
     return cudaGetLastError();
 }
 
-cudaError_t launch_compose_rows(int n, const int* inst, const int* sel, const int* const* rbs, const int* const* res,
-                                int count, int* out_rb, int* out_re, cudaStream_t st) {
+cudaError_t launch_compose_rows(int n, const int* inst, const int* sel, const RowDesc* const* rds, int count,
+                                int* out_rb, int* out_re, RowDesc* out_rd, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     if (count > kMaxAdd + 2) return cudaErrorInvalidValue;
     RowTable T{};
-    for (int k = 0; k < count; ++k) {
-        T.rb[k] = rbs[k];
-        T.re[k] = res[k];
-    }
-    k_compose_rows<<<(n + 255) / 256, 256, 0, st>>>(n, inst, sel, T, out_rb, out_re);
+    for (int k = 0; k < count; ++k) T.rd[k] = rds[k];
+    k_compose_rows<<<(n + 255) / 256, 256, 0, st>>>(n, inst, sel, T, out_rb, out_re, out_rd);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -27,6 +27,10 @@ constexpr int kBitmapColumns = 4608;
 // steps with long B rows and fewer rows than resident warps
 cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, double out_len = 0.0,
                            bool wide_window = false, bool cta = false);
+// the same step for matrices whose rows span consecutive columns (k_band; in
+// a batch, the rows of the instances in P.band); row_len: expected columns of
+// an output row
+cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st);
 // column bitmaps of B's rows for the product's symbolic pass
 // (ProductArgs::bhdr, bbits); bits has one word per entry of B's index space
 cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bits, cudaStream_t st);
@@ -39,13 +43,14 @@ cudaError_t launch_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlo
 cudaError_t launch_validate(int n, int nnz, const int* rowptr, const int* col, const double* val, Ctl* ctl,
                             cudaStream_t st);
 size_t scan_scratch_len(int n);  // long longs of scratch launch_scan_rows needs
-cudaError_t launch_scan_rows(int n, const int* rb, const int* re, int* rowptr, Ctl* ctl, long long* sums,
-                             cudaStream_t st);
+// (rd: the rows' true entries instead of re - rb)
+cudaError_t launch_scan_rows(int n, const int* rb, const int* re, const RowDesc* rd, int* rowptr, Ctl* ctl,
+                             long long* sums, cudaStream_t st);
 cudaError_t launch_gather(int n, const RowView& src, const int* rowptr, int* col, double* val,
                           cudaStream_t st);
 cudaError_t launch_identity(int n, double alpha, int* rowptr, int* col, double* val, cudaStream_t st);
 cudaError_t launch_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
-                             int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
+                             RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
                              cudaStream_t st);
 cudaError_t launch_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long long* words, unsigned* sticky, int n,
                                      long long nnz, cudaStream_t st);
@@ -53,13 +58,15 @@ cudaError_t launch_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long lon
 constexpr int kMaxBatchInst = 1024;
 cudaError_t launch_alg1_batch(const Alg1BatchArgs& A, cudaStream_t st);
 cudaError_t launch_inst_table(int n, int ninst, const int* off, int* inst, cudaStream_t st);
+// (band[i] is cleared if a row of instance i does not span consecutive columns)
 cudaError_t launch_validate_batch(int n, const int* inst, const BatchSrc* src, const int* nnz, Ctl* ctl,
-                                  cudaStream_t st);
-cudaError_t launch_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, int* pool_col,
+                                  unsigned char* band, cudaStream_t st);
+cudaError_t launch_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, RowDesc* rd,
+                                   int* pool_col,
                                    double* pool_val, Ctl* ctl, unsigned long long arena_size, NormSlot* absmax,
                                    int stride, cudaStream_t st);
-cudaError_t launch_compose_rows(int n, const int* inst, const int* sel, const int* const* rbs, const int* const* res,
-                                int count, int* out_rb, int* out_re, cudaStream_t st);
+cudaError_t launch_compose_rows(int n, const int* inst, const int* sel, const RowDesc* const* rds, int count,
+                                int* out_rb, int* out_re, RowDesc* out_rd, cudaStream_t st);
 cudaError_t launch_gather_batch(int n, int ninst, const int* inst, const int* off, const RowView& src,
                                 const int* rowptr, int* out_rp, int* col, double* val, cudaStream_t st);
 cudaError_t launch_bounds(int ninst, const int* off, const int* rowptr, int* bounds, cudaStream_t st);

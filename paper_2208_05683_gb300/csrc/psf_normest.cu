@@ -291,7 +291,7 @@ int estimate_power_norms(Work& w, const psf_csr_t& Z, double* norms, bool* fallb
         *fallback = true;
         return PSF_OK;
     }
-    CU(launch_scan_rows(n, zeros.as<int>(), counts.as<int>(), rpt.as<int>(), w.C(), w.scan.as<long long>(), st));
+    CU(launch_scan_rows(n, zeros.as<int>(), counts.as<int>(), nullptr, rpt.as<int>(), w.C(), w.scan.as<long long>(), st));
     k_transpose_fill<<<grid(n), kThreads, 0, st>>>(n, Z.rowptr, Z.col, Z.val, rpt.as<int>(), cursor.as<int>(),
                                                    scol.as<int>(), sval.as<double>());
     if ((rc = launched())) return rc;
