@@ -124,37 +124,36 @@ void mailbox_give(std::pair<void*, void*> m) {
     std::lock_guard<std::mutex> g(g_mbox_mu);
     g_mbox_free.push_back(m);
 }
-// Step records (bytes of device memory at src) to dst on the host, after
-// the stream's work: through the mailbox when they fit, else a copy.
-int read_stats(Work& w, void* dst, const void* src, size_t bytes) {
-    if (w.mbox.first && bytes % 4 == 0 && bytes <= kMboxBytes - kMboxStats) {
-        w.mbox_pending = true;
-        CU(launch_export(src, static_cast<char*>(w.mbox.second) + kMboxStats, bytes, w.st));
-        CU(cudaStreamSynchronize(w.st));
-        w.mbox_pending = false;
-        memcpy(dst, static_cast<char*>(w.mbox.first) + kMboxStats, bytes);
-        return PSF_OK;
+// The control block (and the norm slots, and `count` step records at
+// dev_stats) to the host, after the stream's work: one kernel for what lies in
+// the workspace's front, one synchronisation.
+int read_back(Work& w, Ctl& c, NormSlot* slots, StepStat* stats, const StepStat* dev_stats, size_t count) {
+    size_t front = slots ? kFrontStats : sizeof(Ctl);
+    const size_t b_stats = sizeof(StepStat) * (stats ? count : 0);
+    size_t off = 0;  // of the records in the mailbox
+    const bool in_front = stats && dev_stats >= w.front_stats() && dev_stats < w.front_stats() + kFrontRecords;
+    if (in_front) {
+        off = kFrontStats + sizeof(StepStat) * (size_t)(dev_stats - w.front_stats());
+        front = off + b_stats;
+    } else if (stats) {
+        off = kFrontBytes;
     }
-    CU(cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost));
-    return PSF_OK;
-}
-
-// The control block (and the norm slots) to the host, after the stream's work.
-int read_back(Work& w, Ctl& c, NormSlot* slots) {
-    if (w.mbox.first) {
+    if (w.mbox.first && off + b_stats <= kMboxBytes) {
         char* hd = static_cast<char*>(w.mbox.second);
         w.mbox_pending = true;
-        CU(launch_export(w.ctl.p, hd, sizeof(Ctl), w.st));
-        if (slots) CU(launch_export(w.slots.p, hd + kMboxSlots, sizeof(NormSlot) * kMaxNorms, w.st));
+        CU(launch_export(w.slab.p, hd, front, w.st));
+        if (b_stats && !in_front) CU(launch_export(dev_stats, hd + off, b_stats, w.st));
         CU(cudaStreamSynchronize(w.st));
         w.mbox_pending = false;
         const char* hh = static_cast<const char*>(w.mbox.first);
         memcpy(&c, hh, sizeof(Ctl));
-        if (slots) memcpy(slots, hh + kMboxSlots, sizeof(NormSlot) * kMaxNorms);
+        if (slots) memcpy(slots, hh + kFrontSlots, sizeof(NormSlot) * kMaxNorms);
+        if (b_stats) memcpy(stats, hh + off, b_stats);
         return PSF_OK;
     }
-    CU(cudaMemcpyAsync(&c, w.ctl.p, sizeof(Ctl), cudaMemcpyDeviceToHost, w.st));
-    if (slots) CU(cudaMemcpyAsync(slots, w.slots.p, sizeof(NormSlot) * kMaxNorms, cudaMemcpyDeviceToHost, w.st));
+    CU(cudaMemcpyAsync(&c, w.slab.p, sizeof(Ctl), cudaMemcpyDeviceToHost, w.st));
+    if (slots) CU(cudaMemcpyAsync(slots, w.slots(), sizeof(NormSlot) * kMaxNorms, cudaMemcpyDeviceToHost, w.st));
+    if (b_stats) CU(cudaMemcpyAsync(stats, dev_stats, b_stats, cudaMemcpyDeviceToHost, w.st));
     CU(cudaStreamSynchronize(w.st));
     return PSF_OK;
 }
@@ -173,11 +172,11 @@ int status_to_code(int st) {
 // Validate input matrices on the device and wait for the outcome: nothing
 // indexes with an input's columns before this returns PSF_OK.  Notes whether
 // every row of every input so far spans consecutive columns (w.band).
-int validate_inputs(Work& w, std::initializer_list<const psf_csr_t*> ms) {
+int validate_inputs(Work& w, const std::vector<const psf_csr_t*>& ms) {
     for (const psf_csr_t* m : ms)
         if (m) CU(launch_validate(m->n, m->nnz, m->rowptr, m->col, m->val, w.C(), w.st));
     Ctl c;
-    int rc = read_back(w, c, nullptr);
+    int rc = read_back(w, c);
     if (rc) return rc;
     w.band = !c.not_band;
     return status_to_code(c.status);
@@ -201,10 +200,10 @@ unsigned long long arena_for(double row_len) {
 // norm phase's Z^k; while no entry has been dropped (a device flag), the
 // product is skipped and k_reuse_pass1 does the step on those rows.
 int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddTerm>& add,
-             double threshold, double e_r, int maxit, int stat_index, size_t slot, RowView* out,
+             double threshold, double e_r, int maxit, StepStat* stat, size_t slot, RowView* out,
              NormSlot* absmax_slot = nullptr, double blen = 0.0, double alen = 0.0, int reuse_k = 0,
              unsigned long long reuse_fma = 0, double out_len = 0.0, bool wide_window = false,
-             double fma_hint = 0.0) {
+             double fma_hint = 0.0, int mark = 0) {
     if (add.size() > (size_t)kMaxAdd) return fail(PSF_ETOOBIG, "%zu addend terms (max %d)", add.size(), kMaxAdd);
     Rows R;
     int rc = w.rows_for(slot, &R);
@@ -229,9 +228,14 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
     P.filtering = filt ? 1 : 0;
     P.eps_g = eps_g;
     P.e_lsb = lsb_for_bound_host(eps_g);
-    P.words = w.words.as<unsigned long long>();
-    P.sticky = w.sticky.as<unsigned>();
-    P.stat = stat_index >= 0 ? w.stats.as<StepStat>() + stat_index : nullptr;
+    P.words = w.words;
+    P.sticky = w.sticky;
+    P.stat = stat;
+    P.mark = mark;
+    if (filt) {
+        P.cslot = w.C()->cslot;
+        P.ncslot = 2;
+    }
     P.absmax_slot = absmax_slot;
     P.chunk_cols = w.chunk_cols;
     P.chunk_slots = w.chunk_slots;
@@ -242,8 +246,6 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         P.cand_cap = w.ccap;
         P.cand_chunk = w.cand_chunk();
     }
-    if (P.stat) CU(cudaMemcpyAsync(&P.stat->pool_start, &w.C()->pool_used, sizeof(unsigned long long),
-                                   cudaMemcpyDeviceToDevice, w.st));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     const bool timed = g_prof.on || g_tune_rec;
     if (timed) {
@@ -283,10 +285,8 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
             P.bbits = w.pool_bits.as<unsigned>();
         }
         const bool cta = A && !table && (w.slot_map == 4 || (w.slot_map == 0 && use_cta(w.n, alen, blen)));
-        if (band) {
-            if ((rc = w.take_ticket(&P.ticket, w.st))) return rc;
-            CU(launch_band(P, A ? alen + blen : 0.0, w.st));
-        } else CU(launch_product(P, table, w.st, out_len, wide_window || w.slot_map == 3, cta));
+        if (band) CU(launch_band(P, A ? alen + blen : 0.0, w.st));
+        else CU(launch_product(P, table, w.st, out_len, wide_window || w.slot_map == 3, cta));
     }
     if (reuse_k > 0) {
         ReuseArgs U{};
@@ -345,25 +345,18 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
 
 // Copy a canonical CSR input into the pool (4-entry aligned rows), as row
 // slot `slot`; the product kernels read every B row and addend row there.
-int pool_copy(Work& w, const psf_csr_t& m, size_t slot, RowView* out) {
+int pool_copy(Work& w, const psf_csr_t& m, size_t slot, RowView* out, NormSlot* absmax = nullptr) {
     Rows R;
     int rc = w.rows_for(slot, &R);
     if (rc) return rc;
     CU(launch_copy_rows(m.n, m.rowptr, m.col, m.val, R.rb, R.re, R.rd, w.pcol(), w.pval(), w.C(),
-                        arena_for(m.n > 0 ? (double)m.nnz / m.n : 1.0), w.st));
+                        arena_for(m.n > 0 ? (double)m.nnz / m.n : 1.0), absmax, w.st));
     *out = w.pooled(R);
     return PSF_OK;
 }
 
 constexpr size_t kSlotZp = 60;  // row slot of the pooled copy of Z
 constexpr size_t kSlotW = 61;   // row slot of W = Z Z (PSF_Z_SQUARE) when computed in the PS phase
-
-// ctl->mark[i] <- the pool counter, in stream order
-int mark_pool(Work& w, int i) {
-    CU(cudaMemcpyAsync(&w.C()->mark[i], &w.C()->pool_used, sizeof(unsigned long long), cudaMemcpyDeviceToDevice,
-                       w.st));
-    return PSF_OK;
-}
 
 int make_result(Work& w, const RowView& M, psf_result_t* out, psf_result_s** made) {
     psf_result_s* r = new (std::nothrow) psf_result_s();
@@ -564,24 +557,12 @@ int psf_norm1(const psf_csr_t* M, void* stream, double* out) {
         *out = 0.0;
         return PSF_OK;
     }
+    // M's entries are read in place; its check's outcome comes with the norm
+    // (the norm kernels never index with a column outside [0, n)), so there is
+    // one synchronisation
     Work w;
-    if ((rc = w.init(M->n, st, 1))) return rc;
-    if ((rc = validate_inputs(w, {M}))) return rc;
-    if ((rc = w.reset_pool((unsigned long long)M->nnz + 4ull * M->n + 2048ull * num_sms() * 8))) return rc;
-    RowView v;
-    if ((rc = mark_pool(w, 0)) || (rc = pool_copy(w, *M, 0, &v)) || (rc = mark_pool(w, 1))) return rc;
-    NormSlot* slots = w.slots.as<NormSlot>();
-    CU(launch_absmax(w.pval(), w.C(), 0, slots + 0, st));
-    NormArgs na{};
-    na.n = M->n;
-    na.count = 1;
-    na.pool_col = w.pcol();
-    na.pool_val = w.pval();
-    na.slots = slots;
-    na.words = w.words.as<unsigned long long>();
-    na.sticky = w.sticky.as<unsigned>();
-    na.ctl = w.C();
-    CU(launch_norms(na, st));
+    if ((rc = w.init(M->n, st, 0))) return rc;
+    CU(launch_norm_in_place(w.C(), w.slots(), w.words, w.sticky, *M, st));
     Ctl c;
     NormSlot hs[kMaxNorms];
     if ((rc = read_back(w, c, hs))) return rc;
@@ -616,13 +597,12 @@ int psf_product_filter(const psf_csr_t* A, const psf_csr_t* B, int32_t nadd, con
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = prepare(st))) return rc;
     Work w;
-    if ((rc = w.init(n, st, 1))) return rc;
+    if ((rc = w.init(n, st, 0)) || (rc = w.init_products())) return rc;
     w.dense_xover = g_dense_xover.load();
     w.dense_estimate = true;  // one product: the operands' mean row lengths give its expected count
-    CU(cudaMemsetAsync(w.stats.p, 0, sizeof(StepStat), st));
-    if ((rc = validate_inputs(w, {A, B}))) return rc;
-    for (int t = 0; t < nadd; ++t)
-        if (addends[t] && (rc = validate_inputs(w, {addends[t]}))) return rc;
+    std::vector<const psf_csr_t*> inputs{A, B};
+    for (int t = 0; t < nadd; ++t) inputs.push_back(addends[t]);
+    if ((rc = validate_inputs(w, inputs))) return rc;
     const double blen = B && n > 0 ? (double)B->nnz / n : 0.0;
     unsigned long long est = (unsigned long long)n * 8ull + 16;
     for (int t = 0; t < nadd; ++t)
@@ -631,13 +611,19 @@ int psf_product_filter(const psf_csr_t* A, const psf_csr_t* B, int32_t nadd, con
         est += (unsigned long long)B->nnz + 4ull * n;
         est += (unsigned long long)A->nnz * (2ull + (unsigned long long)B->nnz / (unsigned long long)(n > 0 ? n : 1)) * 2ull;
     }
+    // (and what the resident warps' arenas may leave unused: without it a
+    // product of a few thousand short rows overflowed and ran twice)
+    est += 512ull * (unsigned long long)(n < 4 * 7 * num_sms() ? n : 4 * 7 * num_sms());
     RowView va, vb, res;
     if (A) va = view_of(*A);
     unsigned long long cap = est < kMaxPool ? est : kMaxPool;
     psf_result_s* r = nullptr;
+    psf_result_t handle;
+    Ctl c;
+    StepStat ss{};
     for (int attempt = 0;; ++attempt) {
         if ((rc = w.reset_pool(cap))) return rc;
-        CU(cudaMemsetAsync(w.stats.p, 0, sizeof(StepStat), st));
+        if (attempt) CU(cudaMemsetAsync(w.front_stats(), 0, sizeof(StepStat), st));
         // B and the addend matrices are read from pooled copies
         std::vector<AddTerm> add;
         for (int t = 0; t < nadd; ++t) {
@@ -651,13 +637,18 @@ int psf_product_filter(const psf_csr_t* A, const psf_csr_t* B, int32_t nadd, con
             add.push_back(T);
         }
         if (A && (rc = pool_copy(w, *B, 1, &vb))) return rc;
-        if ((rc = run_step(w, A ? &va : nullptr, A ? &vb : nullptr, add, threshold, e_r, maxit, 0, 0, &res,
+        if ((rc = run_step(w, A ? &va : nullptr, A ? &vb : nullptr, add, threshold, e_r, maxit, w.front_stats(), 0, &res,
                            nullptr, blen, A && n > 0 ? (double)A->nnz / n : 0.0)))
             return rc;
-        Ctl c;
-        if ((rc = read_back(w, c, nullptr))) return rc;
-        if ((rc = status_to_code(c.status))) return rc;
+        // (a pool that overflowed leaves empty rows: the scan is harmless)
+        if ((rc = make_result(w, res, &handle, &r))) return rc;
+        if ((rc = read_back(w, c, nullptr, &ss, w.front_stats(), 1)) || (rc = status_to_code(c.status))) {
+            destroy_result(r);
+            return rc;
+        }
         if (c.status & kDevPoolFull) {
+            destroy_result(r);
+            r = nullptr;
             if ((rc = w.clear_sums())) return rc;
             if (attempt > 8) return fail(PSF_ENOMEM, "pool kept overflowing");
             if (cap >= kMaxPool) return fail(PSF_ETOOBIG, "the step needs more than 2^31 - 2^20 pool entries");
@@ -667,18 +658,6 @@ int psf_product_filter(const psf_csr_t* A, const psf_csr_t* B, int32_t nadd, con
             continue;
         }
         break;
-    }
-    psf_result_t handle;
-    if ((rc = make_result(w, res, &handle, &r))) return rc;
-    Ctl c;
-    StepStat ss{};
-    if ((rc = read_back(w, c, nullptr))) {
-        destroy_result(r);
-        return rc;
-    }
-    if (read_stats(w, &ss, w.stats.p, sizeof ss) != PSF_OK) {
-        destroy_result(r);
-        return fail(PSF_ECUDA, "stats read-back");
     }
     if ((rc = finish_result(w, res, r, c.nnz_total))) {
         destroy_result(r);
@@ -722,7 +701,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     const std::vector<double>& a = square ? series->c : series->a;
 
     Work w;
-    if ((rc = w.init(n, st, 16))) return rc;
+    if ((rc = w.init(n, st, submult ? 1 : 10)) || (rc = w.init_products())) return rc;
     if ((rc = validate_inputs(w, {Z}))) return rc;
     w.slot_map = series->kernel;
     w.dense_xover = series->dense_xover >= 0.0 ? series->dense_xover : g_dense_xover.load();
@@ -741,12 +720,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     const double zlen = n > 0 ? (double)Z->nnz / n : 0.0;
     double znnz[kMaxNorms] = {0.0};  // nnz(Z^i) of this evaluation
     znnz[1] = (double)Z->nnz;
-    NormSlot* slots = w.slots.as<NormSlot>();
-    if (n > 0) {
-        const size_t nb = sizeof(unsigned long long) * (size_t)kNormPieces * (size_t)n * 10;
-        CU(w.nwords.alloc(nb, st));
-        CU(cudaMemsetAsync(w.nwords.p, 0, nb, st));
-    }
+    NormSlot* slots = w.slots();
 
     // ---- Alg. 2 step 1: norms ||Z^i||_1, i <= 10 (Eq. 37): exact (the powers
     // Z^2..Z^10 are computed), or ||Z||^i, or ||Z||_1 exact and the others
@@ -774,17 +748,14 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
         if (series->z_need == 0 && zcap < est) zcap = est;
         if (zcap > kMaxPool) zcap = kMaxPool;
         for (int attempt = 0;; ++attempt) {
-            CU(cudaMemsetAsync(slots, 0, sizeof(NormSlot) * kMaxNorms, st));
+            if (attempt) CU(cudaMemsetAsync(slots, 0, kFrontBytes - kFrontSlots, st));
             // the pooled Z and Z^2 .. Z^10, each delimited in the pool by counter
             // snapshots (the marks also give baby steps their powers' ranges)
             if (n > 0) {
                 unsigned long long total = zcap + ps_reserve;
                 if (total > kMaxPool) total = kMaxPool;
                 if ((rc = w.reset_pool(total))) return rc;
-                CU(cudaMemsetAsync(w.stats.p, 0, sizeof(StepStat) * 16, st));
-                if ((rc = mark_pool(w, 0)) || (rc = pool_copy(w, *Z, kSlotZp, &zp)) || (rc = mark_pool(w, 1)))
-                    return rc;
-                CU(launch_absmax(w.pval(), w.C(), 0, slots + 1, st));
+                if ((rc = pool_copy(w, *Z, kSlotZp, &zp, slots + 1))) return rc;  // (and mark[1])
                 // norms by row tiles: matrix 0 is the pooled Z, matrix i-1 is Z^i
                 NormRowsArgs nr{};
                 nr.n = n;
@@ -794,8 +765,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 nr.col = w.pcol();
                 nr.val = w.pval();
                 nr.slots = slots + 1;
-                nr.words = w.nwords.as<unsigned long long>();
-                nr.sticky = w.sticky.as<unsigned>();
+                nr.words = w.nwords;
+                nr.sticky = w.sticky;
                 nr.ctl = w.C();
                 if (chain) {
                     RowView prev = zp;
@@ -804,10 +775,9 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                         double blen = (size_t)(i - 2) < series->len_z.size() ? series->len_z[(size_t)(i - 2)]
                                                                               : zlen * (i - 1) * (i - 1);
                         const bool wz = (size_t)(i - 2) < span_z.size() && span_z[(size_t)(i - 2)] > kBitmapColumns;
-                        if ((rc = run_step(w, &vz, &prev, {}, 0.0, 0.0, 1, i - 2, (size_t)(i - 2), &cur,
-                                           slots + i, blen, zlen, 0, 0ull, 0.0, wz)))
+                        if ((rc = run_step(w, &vz, &prev, {}, 0.0, 0.0, 1, w.front_stats() + (i - 2), (size_t)(i - 2),
+                                           &cur, slots + i, blen, zlen, 0, 0ull, 0.0, wz, 0.0, i)))
                             return rc;
-                        if ((rc = mark_pool(w, i))) return rc;
                         if (i == 2) zsq = cur;
                         nr.rb[i - 1] = cur.rb;
                         nr.re[i - 1] = cur.re;
@@ -819,7 +789,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             }
             Ctl c;
             NormSlot hs[kMaxNorms];
-            if ((rc = read_back(w, c, hs))) return rc;
+            StepStat zs[9];
+            if ((rc = read_back(w, c, hs, zs, w.front_stats(), 9))) return rc;
             if ((rc = status_to_code(c.status))) return rc;
             if (c.status & kDevPoolFull) {
                 if ((rc = w.clear_sums())) return rc;
@@ -834,9 +805,6 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             z_fma = c.fma_total;
             if (z_used > series->z_need) series->z_need = z_used;
             if (chain) {
-                StepStat zs[9];
-                if (read_stats(w, zs, w.stats.p, sizeof zs) != PSF_OK)
-                    return fail(PSF_ECUDA, "stats read-back");
                 series->len_z.assign(9, 0.0);
                 std::vector<unsigned> sz(9, 0u);
                 for (int i = 2; i <= 10; ++i) {
@@ -866,7 +834,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     if (p.q > PSF_MAX_Q) return fail(PSF_ETOOBIG, "q = %d exceeds %d", p.q, PSF_MAX_Q);
     const int N = p.N, q = p.q, b = p.b, g = p.g;
     const int stat_cap = q + b + 4;
-    CU(w.stats.alloc(sizeof(StepStat) * (size_t)stat_cap, st));
+    StepStat* pstat = nullptr;  // the PS phase's step records
     auto coef = [&](int idx) { return (idx < N && idx < (int)a.size()) ? a[(size_t)idx] : 0.0; };
 
     psf_result_s* r = nullptr;
@@ -913,7 +881,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             const bool reuse = attempt == 0 && ps_reserve > 0;
             const unsigned long long used_before = reuse ? z_used : 0ull;
             if (!reuse && (rc = w.reset_pool(cap))) return rc;
-            CU(cudaMemsetAsync(w.stats.p, 0, sizeof(StepStat) * (size_t)stat_cap, st));
+            if ((rc = w.stats_for(stat_cap, attempt > 0, &pstat))) return rc;
             steps.clear();
             int si = 0;
             std::vector<RowView> Zh((size_t)q + 2);
@@ -928,7 +896,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             if (square) {
                 if (reuse) {
                     vm = zsq;
-                } else if ((rc = run_step(w, &vz, &Zh[1], {}, 0.0, 0.0, 1, -1, kSlotW, &vm, nullptr, zlen, zlen))) {
+                } else if ((rc = run_step(w, &vz, &Zh[1], {}, 0.0, 0.0, 1, nullptr, kSlotW, &vm, nullptr, zlen, zlen))) {
                     return rc;
                 }
                 Zh[1] = vm;
@@ -943,7 +911,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 // baby step k + 1 writes row slot k - 1, the slot of the norm phase's Z^(k+1)
                 const int rk = (reuse && !square && k + 1 <= 10 && slot == (size_t)(k - 1)) ? k + 1 : 0;
                 const bool wb = (size_t)(k - 1) < span_baby.size() && span_baby[(size_t)(k - 1)] > kBitmapColumns;
-                if ((rc = run_step(w, &vm, &Zh[(size_t)k], {}, thr, series->e_r, series->maxit, si, slot++,
+                if ((rc = run_step(w, &vm, &Zh[(size_t)k], {}, thr, series->e_r, series->maxit, pstat + si, slot++,
                                    &Zh[(size_t)k + 1], nullptr, blen, pow_len(1), rk, rk ? zfma[rk] : 0ull, 0.0, wb)))
                     return rc;
                 psf_step_info_t s{};
@@ -977,7 +945,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             size_t sslot[2] = {slot, slot + 1};
             int cur = 0;
             if (g == 0) {
-                if ((rc = run_step(w, nullptr, nullptr, block(b - 1), 0.0, 0.0, 1, si, sslot[cur], &S))) return rc;
+                if ((rc = run_step(w, nullptr, nullptr, block(b - 1), 0.0, 0.0, 1, pstat + si, sslot[cur], &S))) return rc;
                 psf_step_info_t s{};
                 s.kind = 2;
                 s.index = 0;
@@ -999,7 +967,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                         T.rd = Zh[(size_t)q].rd;
                         add.push_back(T);
                     }
-                    if ((rc = run_step(w, nullptr, nullptr, add, 0.0, 0.0, 1, si, sslot[nslot], &nxt))) return rc;
+                    if ((rc = run_step(w, nullptr, nullptr, add, 0.0, 0.0, 1, pstat + si, sslot[nslot], &nxt))) return rc;
                     s.kind = 2;
                 } else {
                     double thr = nofilter ? 0.0 : p.sigma[(size_t)i];
@@ -1012,7 +980,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     const bool wg = (size_t)(i - 1) < span_giant.size() && span_giant[(size_t)(i - 1)] > kBitmapColumns;
                     const double fh =
                         (size_t)(i - 1) < series->fma_giant.size() ? series->fma_giant[(size_t)(i - 1)] : 0.0;
-                    if ((rc = run_step(w, &Zh[(size_t)q], &S, add, thr, series->e_r, series->maxit, si, sslot[nslot],
+                    if ((rc = run_step(w, &Zh[(size_t)q], &S, add, thr, series->e_r, series->maxit, pstat + si, sslot[nslot],
                                        &nxt, nullptr, blen, alen, 0, 0ull, olen, wg, fh)))
                         return rc;
                     s.kind = 1;
@@ -1030,7 +998,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 s.index = 1;
                 RowView G = S;
                 const double glen = series->len_odd > 0.0 ? series->len_odd : pow_len(N - 1);
-                if ((rc = run_step(w, &vz, &G, {}, 0.0, 0.0, 1, si, sslot[cur ^ 1], &S, nullptr, glen, zlen)))
+                if ((rc = run_step(w, &vz, &G, {}, 0.0, 0.0, 1, pstat + si, sslot[cur ^ 1], &S, nullptr, glen, zlen)))
                     return rc;
                 steps.push_back(s);
                 ++si;
@@ -1038,7 +1006,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             F = S;
             if ((rc = make_result(w, F, &handle, &r))) return rc;
             Ctl c;
-            if ((rc = read_back(w, c, nullptr))) {
+            std::vector<StepStat> ss(steps.size());
+            if ((rc = read_back(w, c, nullptr, ss.data(), pstat, ss.size()))) {
                 destroy_result(r);
                 return rc;
             }
@@ -1056,13 +1025,6 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 cap = need > 2 * cap ? need : 2 * cap;
                 if (cap > kMaxPool) cap = kMaxPool;
                 continue;
-            }
-            std::vector<StepStat> ss(steps.size());
-            if (!ss.empty()) {
-                if (read_stats(w, ss.data(), w.stats.p, sizeof(StepStat) * ss.size()) != PSF_OK) {
-                    destroy_result(r);
-                    return fail(PSF_ECUDA, "stats read-back");
-                }
             }
             for (size_t i = 0; i < steps.size(); ++i) {
                 steps[i].nnz_pre = (int64_t)ss[i].nnz_pre;
@@ -1460,19 +1422,7 @@ extern "C" int psf_norm1_noalloc(const psf_csr_t* M, void* stream, double* out) 
     // clear what must start at zero, check the input (its outcome is read
     // with the result; the norm kernels never index with a column outside
     // [0, n)), then max |x| and the exact column sums over M's entries
-    CU(launch_norm_scratch_init(ctl, slot, words, sticky, M->n, M->nnz, st));
-    CU(launch_validate(M->n, M->nnz, M->rowptr, M->col, M->val, ctl, st));
-    CU(launch_absmax(M->val, ctl, 0, slot, st));
-    NormArgs na{};
-    na.n = M->n;
-    na.count = 1;
-    na.pool_col = M->col;
-    na.pool_val = M->val;
-    na.slots = slot;
-    na.words = words;
-    na.sticky = sticky;
-    na.ctl = ctl;
-    CU(launch_norms(na, st));
+    CU(launch_norm_in_place(ctl, slot, words, sticky, *M, st));
     int status = 0;
     unsigned long long bits = 0ull;
     CU(cudaMemcpyAsync(&status, &ctl->status, sizeof status, cudaMemcpyDeviceToHost, st));

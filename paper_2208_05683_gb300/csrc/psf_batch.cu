@@ -155,7 +155,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     const psf_series_s* s0 = series[0];
 
     Work w;
-    if ((rc = w.init(n, st, 1))) return rc;
+    if ((rc = w.init(n, st, 10)) || (rc = w.init_products())) return rc;
     w.slot_map = s0->kernel;
     w.chunk_cols = s0->chunk_cols;
     w.chunk_slots = s0->chunk_slots;
@@ -167,11 +167,6 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     CU(d_nnz.alloc(sizeof(int) * (size_t)count, st));
     CU(d_inst.alloc(sizeof(int) * (size_t)(n > 0 ? n : 1), st));
     CU(d_slots.alloc(sizeof(NormSlot) * kMaxNorms * (size_t)count, st));
-    if (n > 0) {
-        const size_t nb = sizeof(unsigned long long) * (size_t)kNormPieces * (size_t)n * 10;
-        CU(w.nwords.alloc(nb, st));
-        CU(cudaMemsetAsync(w.nwords.p, 0, nb, st));
-    }
     std::vector<BatchSrc> src((size_t)count);
     std::vector<int> nnz((size_t)count);
     for (int i = 0; i < count; ++i) {
@@ -193,7 +188,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     {
         Ctl c;
         CU(cudaMemcpyAsync(isband.data(), d_isband.p, (size_t)count, cudaMemcpyDeviceToHost, st));
-        if ((rc = read_back(w, c, nullptr))) return rc;
+        if ((rc = read_back(w, c))) return rc;
         if (c.status & kDevBadInput) return fail(PSF_EINVAL, "a batch input is malformed (row pointers, column order "
                                                             "or range, or non-finite value)");
     }
@@ -247,10 +242,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             if ((rc = w.reset_pool(zcap))) return rc;
             Rows zr;
             if ((rc = w.rows_for(kRowsZ, &zr))) return rc;
-            if ((rc = mark_pool(w, 0))) return rc;
             CU(launch_copy_rows_batch(n, inst, dsrc, zr.rb, zr.re, zr.rd, w.pcol(), w.pval(), w.C(), arena_z, slots + 1,
                                       kMaxNorms, st));
-            if ((rc = mark_pool(w, 1))) return rc;
             const RowView zp = w.pooled(zr);
             // norms by row tiles: matrix 0 is the pooled Z, matrix k-1 is Z^k
             NormRowsArgs nr{};
@@ -263,8 +256,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             nr.slots = slots + 1;
             nr.slot_stride = kMaxNorms;
             nr.inst = inst;
-            nr.words = w.nwords.as<unsigned long long>();
-            nr.sticky = w.sticky.as<unsigned>();
+            nr.words = w.nwords;
+            nr.sticky = w.sticky;
             nr.ctl = w.C();
             if (any_chain) {
                 RowView prev = zp;
@@ -283,8 +276,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                     P.pool_col = w.pcol();
                     P.pool_val = w.pval();
                     P.ctl = w.C();
-                    P.words = w.words.as<unsigned long long>();
-                    P.sticky = w.sticky.as<unsigned>();
+                    P.words = w.words;
+                    P.sticky = w.sticky;
                     P.inst = inst;
                     P.inst_off = d_off.as<int>();
                     P.bstep = d_zstep.as<BatchStep>();
@@ -307,23 +300,19 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                     }
                     P.band = table ? nullptr : d_band;
                     if (any_general || table) CU(launch_product(P, table, st, 0.0, wz));
-                    if (P.band) {
-                        if ((rc = w.take_ticket(&P.ticket, st))) return rc;
-                        CU(launch_band(P, 0.0, st));
-                    }
+                    if (P.band) CU(launch_band(P, 0.0, st));
                     if (g_tune_rec) {
                         CU(cudaEventRecord(t1, st));
                         g_tune_rec->work.push_back(zlen_all * blen);
                         g_tune_rec->ev.emplace_back(t0, t1);
                     }
-                    if ((rc = mark_pool(w, k))) return rc;
                     prev = w.pooled(R);
                 }
                 nr.count = 10;
             }
             CU(launch_norms_rows(nr, st));
             Ctl c;
-            if ((rc = read_back(w, c, nullptr))) return rc;
+            if ((rc = read_back(w, c))) return rc;
             if ((rc = status_to_code(c.status))) return rc;
             if (c.status & kDevPoolFull) {
                 if ((rc = w.clear_sums())) return rc;
@@ -571,8 +560,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         if (g_ps_per_row.load() == 0.0 && cap < est) cap = est;
         if (cap > kMaxPool) cap = kMaxPool;
     }
-    DevBuf d_rowptr, d_bounds, d_tickets;
-    CU(d_tickets.alloc(sizeof(unsigned) * nst, st));
+    DevBuf d_rowptr, d_bounds;
     CU(d_rowptr.alloc(sizeof(int) * ((size_t)n + 1), st));
     CU(d_bounds.alloc(sizeof(int) * ((size_t)count + 1), st));
     std::vector<int> bounds((size_t)count + 1);
@@ -595,8 +583,6 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         auto enqueue = [&](cudaStream_t st) -> int {
         CU(cudaMemsetAsync(d_stat.p, 0, sizeof(StepStat) * nst * (size_t)count, st));
         CU(cudaMemsetAsync(d_dropped.p, 0, sizeof(int) * (size_t)count, st));
-        unsigned* const tickets = d_tickets.as<unsigned>();  // k_band's tile counters, one per stage
-        CU(cudaMemsetAsync(tickets, 0, sizeof(unsigned) * nst, st));
 
         CU(launch_copy_rows_batch(n, inst, dsrc, zr.rb, zr.re, zr.rd, w.pcol(), w.pval(), w.C(), arena_z, nullptr, 0, st));
         const RowView zp = w.pooled(zr);
@@ -645,8 +631,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             P.pool_col = w.pcol();
             P.pool_val = w.pval();
             P.ctl = w.C();
-            P.words = w.words.as<unsigned long long>();
-            P.sticky = w.sticky.as<unsigned>();
+            P.words = w.words;
+            P.sticky = w.sticky;
             P.inst = inst;
             P.inst_off = d_off.as<int>();
             P.bstep = reinterpret_cast<const BatchStep*>(d_tab.as<unsigned char>() + step_off[si]);
@@ -664,8 +650,11 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             }
             const double fma_row = T.work_rows > 0.0 ? T.work_fma / T.work_rows : 8.0 * (T.nadd + 1);
             P.arena = arena_for(fma_row);
-            CU(cudaMemcpyAsync(d_pstart.as<unsigned long long>() + si, &w.C()->pool_used, sizeof(unsigned long long),
-                               cudaMemcpyDeviceToDevice, st));
+            P.start_out = d_pstart.as<unsigned long long>() + si;
+            if (T.any_filter) {
+                P.cslot = d_cslot.as<unsigned long long>();
+                P.ncslot = 2 * count;
+            }
             const bool table = use_table(w.slot_map, fma_row);
             cudaEvent_t e0 = nullptr, e1 = nullptr;
             if (g_prof.on || g_tune_rec) {
@@ -685,7 +674,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             P.band = table ? nullptr : d_band;
             if (any_general || table) CU(launch_product(P, table, st, 0.0, T.wide));
             if (P.band) {
-                P.ticket = tickets + si;
+                if (any_general || table) P.start_out = nullptr;  // (known)
                 CU(launch_band(P, 0.0, st));
             }
             if (g_tune_rec) {
@@ -776,7 +765,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         }
         CU(cudaMemcpyAsync(bounds.data(), d_bounds.p, sizeof(int) * bounds.size(), cudaMemcpyDeviceToHost, st));
         CU(cudaMemcpyAsync(pst.data(), d_stat.p, sizeof(StepStat) * pst.size(), cudaMemcpyDeviceToHost, st));
-        rc = read_back(w, cfin, nullptr);
+        rc = read_back(w, cfin);
         if (exec) cudaGraphExecDestroy(exec);  // the stream has drained
         if (rc) return rc;
         if ((rc = status_to_code(cfin.status))) return rc;

@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(256) k_dense_out(ProductArgs P, const double* 
     }
     arena_close(arena, P.pool_val, lane);
     if (P.cand_col) cand_close(carena, P.cand_x, lane);
+    step_done(P.ctl, P.mark, P.stat ? &P.stat->pool_start : nullptr, P.start_out, P.cslot, P.ncslot);
     my_cand = (unsigned long long)warp_sum((int)my_cand);
     my_absmax = warp_max_u64(my_absmax);
     for (int o = 16; o; o >>= 1) my_fma += __shfl_xor_sync(kFull, my_fma, o);

@@ -42,11 +42,14 @@ struct Ctl {
     unsigned long long cand_cap;
     int cand_over;
     unsigned cand_chunk;  // entries a warp reserves at a time (32..128)
+    unsigned long long pool_mark;  // pool counter at the end of the last launch that reserved
     int dropped;          // set once Algorithm 1 has dropped an entry (baby steps reuse powers until then)
     int pad1;
     unsigned bar_count;  // fields from here on survive a pool reset
     unsigned bar_gen;
     int not_band;  // an input has a row that does not span consecutive columns
+    unsigned done;    // blocks of the running launch that have finished (0 between launches)
+    unsigned ticket;  // k_band's tile counter (0 between launches)
     unsigned long long fma_total;  // algorithmic multiply-adds of all products
     unsigned long long mark[kMaxNorms + 1];  // pool counter snapshots delimiting the norm matrices
 };
@@ -180,7 +183,11 @@ struct ProductArgs {
     const unsigned* bbits;
     // batch: instances whose rows k_band computes (nullptr: none)
     const unsigned char* band;
-    unsigned* ticket;           // k_band's tile counter, 0 at the launch
+    // written by the launch's last block (step_done)
+    int mark;                        // > 0: ctl->mark[mark] <- the pool counter
+    unsigned long long* start_out;   // batch: the pool counter before the step
+    unsigned long long* cslot;       // column-sum maxima that Algorithm 1 starts from 0
+    int ncslot;
 };
 
 // Algorithm 1 passes 2, 3, ... and compaction for every filtered instance of
@@ -587,6 +594,33 @@ __device__ __forceinline__ void clear_sums(unsigned long long* words, unsigned* 
         for (int c = 0; c < kChunks; ++c) words[(size_t)c * n + j] = 0ull;
         sticky[j] = 0u;
     }
+}
+
+// The end of a launch that reserved pool space, by every block once its
+// reservations are done: the last one to finish snapshots the pool counter
+// (where this step's entries begin and end: the next launch knows) and clears
+// what the next launch counts in.  These were 8-byte copies and memsets of
+// their own between the kernels, about 2 us each on the stream.
+__device__ __forceinline__ void step_done(Ctl* ctl, int mark, unsigned long long* start_out,
+                                          unsigned long long* start_out2, unsigned long long* cslot, int ncslot) {
+    __shared__ int last_block;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last_block = atomicAdd(&ctl->done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last_block) return;
+    if (threadIdx.x == 0) {
+        const unsigned long long used = __ldcg(&ctl->pool_used), before = __ldcg(&ctl->pool_mark);
+        if (start_out) *start_out = before;
+        if (start_out2) *start_out2 = before;
+        if (mark > 0) ctl->mark[mark] = used;
+        ctl->pool_mark = used;
+        ctl->done = 0u;
+        ctl->ticket = 0u;
+    }
+    for (int i = threadIdx.x; i < ncslot; i += blockDim.x) cslot[i] = 0ull;
 }
 
 // Column sums of a flat scan: an entry whose column lies outside [0, n)

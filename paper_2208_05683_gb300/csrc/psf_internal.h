@@ -116,19 +116,24 @@ extern Profile g_prof;
 constexpr unsigned long long kMaxPool = (1ull << 31) - (1ull << 20);
 
 // Mailboxes: pinned host buffers mapped into the device's address space,
-// {host, device} pointers, into which k_export writes the control block
-// (offset 0), the norm slots (kMboxSlots) and the step records (kMboxStats)
-// that the host reads back.  A kernel's stores take no copy engine, so these
+// {host, device} pointers, into which k_export writes the control block, the
+// norm slots and the step records that the host reads back.  A kernel's stores take no copy engine, so these
 // reads do not wait behind a large device-to-host copy in flight on another
 // stream (a user copying one result out while the next evaluation runs).
 // Each evaluation's workspace takes one from a process-wide free list and
 // gives it back; they are kept for the life of the process (which must not
 // outlive a cudaDeviceReset).  {nullptr, nullptr} if none could be made: the
 // read-backs then use copies.
-constexpr size_t kMboxBytes = 64 * 1024, kMboxSlots = 4096, kMboxStats = 8192;
-static_assert(sizeof(Ctl) % 4 == 0 && sizeof(Ctl) <= kMboxSlots, "control block in its mailbox part");
-static_assert(sizeof(NormSlot) * kMaxNorms % 4 == 0 && kMboxSlots + sizeof(NormSlot) * kMaxNorms <= kMboxStats,
-              "norm slots in their mailbox part");
+constexpr size_t kMboxBytes = 64 * 1024;
+// The front of a workspace's zeroed block, read back as one piece: control
+// block, norm slots, step records (those of a longer plan have a buffer of
+// their own).
+constexpr size_t kFrontSlots = 256, kFrontStats = 512;
+constexpr int kFrontRecords = 96;  // the norm phase's first 16, then the PS phase's
+constexpr size_t kFrontBytes = (kFrontStats + sizeof(StepStat) * kFrontRecords + 255) & ~(size_t)255;
+static_assert(sizeof(Ctl) % 4 == 0 && sizeof(Ctl) <= kFrontSlots, "control block in its part");
+static_assert(kFrontSlots + sizeof(NormSlot) * kMaxNorms <= kFrontStats, "norm slots in their part");
+static_assert(kFrontBytes <= kMboxBytes / 2, "the front fits a mailbox");
 std::pair<void*, void*> mailbox_take();
 void mailbox_give(std::pair<void*, void*> m);
 
@@ -150,17 +155,22 @@ struct Rows {
 struct Work {
     int n = 0;
     cudaStream_t st = nullptr;
-    DevBuf ctl, stats, slots, words, sticky, pool_col, pool_val, cand_col, cand_x, scan;
-    DevBuf nwords;  // 24-bit-piece column sums of the norm phase (zero between uses)
+    // one block, zeroed with one memset: the front (control block, norm slots,
+    // step records), the column sums of Algorithm 1 (and their sticky counts,
+    // and the norms'), and the norm phase's 24-bit-piece column sums (zero
+    // between uses)
+    DevBuf slab, pool_col, pool_val, cand_col, cand_x, scan, more_stats;
+    unsigned long long* words = nullptr;
+    unsigned* sticky = nullptr;
+    unsigned long long* nwords = nullptr;
+    size_t sums_bytes = 0;  // words and sticky
     DevBuf dense[3];  // the dense-tile path's A, B and C (n^2 doubles each), allocated on first use
     DevBuf bhdr, pool_bits;  // column bitmaps of a product's B rows: n headers, a word per pool entry
     double dense_xover = 1e300;  // dense tiles for a step with at least this many multiply-adds per n^3
     bool dense_estimate = false;  // a step without a recorded count may use the row-length estimate
     unsigned long long cap = 0, ccap = 0, bits_cap = 0;
+    static constexpr size_t kRowsChunk = 8;  // matrices' row arrays allocated at a time
     std::vector<DevBuf*> rows;  // per matrix: n row descriptors, then rb and re (n ints each)
-    DevBuf tickets;              // tile counters of k_band's launches (zero until used)
-    int next_ticket = 0;
-    static constexpr int kTickets = 128;
     bool band = false;           // every input row spans consecutive columns: k_band computes the products
     int slot_map = 0;            // 0 auto (by products per row), 1 table, 2 bitmap, 3 wide window, 4 CTA per row
     int chunk_cols = 0, chunk_slots = 0;
@@ -176,23 +186,45 @@ struct Work {
             mailbox_give(mbox);
         }
     }
-    Ctl* C() const { return ctl.as<Ctl>(); }
-    int init(int n_, cudaStream_t s, int nstats) {
+    char* front() const { return slab.as<char>(); }
+    Ctl* C() const { return slab.as<Ctl>(); }
+    NormSlot* slots() const { return reinterpret_cast<NormSlot*>(front() + kFrontSlots); }
+    StepStat* front_stats() const { return reinterpret_cast<StepStat*>(front() + kFrontStats); }
+    // norms: matrices whose exact norms are taken by row tiles
+    int init(int n_, cudaStream_t s, int norms) {
         n = n_;
         st = s;
         if (!mbox.first) mbox = mailbox_take();
-        CU(ctl.alloc(sizeof(Ctl), st));
-        CU(cudaMemsetAsync(ctl.p, 0, sizeof(Ctl), st));
-        CU(stats.alloc(sizeof(StepStat) * (size_t)(nstats > 0 ? nstats : 1), st));
-        CU(slots.alloc(sizeof(NormSlot) * kMaxNorms, st));
-        CU(cudaMemsetAsync(slots.p, 0, sizeof(NormSlot) * kMaxNorms, st));
-        size_t nn = (size_t)(n > 0 ? n : 1);
-        CU(words.alloc(sizeof(unsigned long long) * kChunks * nn * kMaxNorms, st));
-        CU(cudaMemsetAsync(words.p, 0, sizeof(unsigned long long) * kChunks * nn * kMaxNorms, st));
-        CU(sticky.alloc(sizeof(unsigned) * nn * kMaxNorms, st));
-        CU(cudaMemsetAsync(sticky.p, 0, sizeof(unsigned) * nn * kMaxNorms, st));
-        CU(scan.alloc(sizeof(long long) * scan_scratch_len(n_), st));
-        CU(bhdr.alloc(sizeof(int2) * nn, st));
+        const size_t nn = (size_t)(n > 0 ? n : 1);
+        const size_t b_words = sizeof(unsigned long long) * kChunks * nn;
+        const size_t b_sticky = (sizeof(unsigned) * nn * (size_t)(norms > 1 ? norms : 1) + 7) & ~(size_t)7;
+        const size_t bytes = kFrontBytes + b_words + b_sticky +
+                             sizeof(unsigned long long) * (size_t)kNormPieces * nn * (size_t)norms;
+        CU(slab.alloc(bytes, st));
+        words = reinterpret_cast<unsigned long long*>(front() + kFrontBytes);
+        sticky = reinterpret_cast<unsigned*>(front() + kFrontBytes + b_words);
+        nwords = reinterpret_cast<unsigned long long*>(front() + kFrontBytes + b_words + b_sticky);
+        sums_bytes = b_words + b_sticky;
+        CU(cudaMemsetAsync(slab.p, 0, bytes, st));
+        return PSF_OK;
+    }
+    // scratch of the products' launches
+    int init_products() {
+        CU(scan.alloc(sizeof(long long) * scan_scratch_len(n), st));
+        CU(bhdr.alloc(sizeof(int2) * (size_t)(n > 0 ? n : 1), st));
+        return PSF_OK;
+    }
+    // `count` zeroed step records (not the norm phase's first 16); again: they
+    // were used before
+    int stats_for(int count, bool again, StepStat** out) {
+        if (count <= kFrontRecords - 16) {
+            *out = front_stats() + 16;
+            if (!again) return PSF_OK;
+        } else {
+            if (!again) CU(more_stats.alloc(sizeof(StepStat) * (size_t)count, st));
+            *out = more_stats.as<StepStat>();
+        }
+        CU(cudaMemsetAsync(*out, 0, sizeof(StepStat) * (size_t)count, st));
         return PSF_OK;
     }
     // (re)allocate the entry pool and reset the device control block
@@ -212,19 +244,7 @@ struct Work {
             CU(pool_bits.alloc(sizeof(unsigned) * cap, st));
             bits_cap = cap;
         }
-        Ctl h{};
-        h.pool_cap = cap;
-        h.cand_cap = ccap;
-        h.cand_chunk = cand_chunk();
-        CU(cudaMemcpyAsync(ctl.p, &h, offsetof(Ctl, bar_count), cudaMemcpyHostToDevice, st));
-        return PSF_OK;
-    }
-    // A zero tile counter for one launch of k_band, in stream order on s.
-    int take_ticket(unsigned** out, cudaStream_t s) {
-        if (!tickets.p) CU(tickets.alloc(sizeof(unsigned) * kTickets, s));
-        if (next_ticket == 0) CU(cudaMemsetAsync(tickets.p, 0, sizeof(unsigned) * kTickets, s));
-        *out = tickets.as<unsigned>() + next_ticket;
-        next_ticket = (next_ticket + 1) % kTickets;
+        CU(launch_reset(C(), cap, ccap, cand_chunk(), st));
         return PSF_OK;
     }
     // Entries a warp reserves in a candidate list at a time: up to 128, so
@@ -237,19 +257,18 @@ struct Work {
     // Column-sum accumulators are zero between steps; a phase cut short by a
     // pool overflow can leave some set, so they are cleared before its retry.
     int clear_sums() {
-        size_t nn = (size_t)(n > 0 ? n : 1);
-        CU(cudaMemsetAsync(words.p, 0, sizeof(unsigned long long) * kChunks * nn * kMaxNorms, st));
-        CU(cudaMemsetAsync(sticky.p, 0, sizeof(unsigned) * nn * kMaxNorms, st));
+        CU(cudaMemsetAsync(words, 0, sums_bytes, st));
         return PSF_OK;
     }
     // row arrays of matrix slot i
     int rows_for(size_t i, Rows* out) {
-        while (rows.size() <= i) rows.push_back(new DevBuf());
-        const size_t nn = (size_t)(n > 0 ? n : 1);
-        if (!rows[i]->p) CU(rows[i]->alloc((sizeof(RowDesc) + 2 * sizeof(int)) * nn, st));
-        out->rd = rows[i]->as<RowDesc>();
+        const size_t c = i / kRowsChunk, nn = ((size_t)(n > 0 ? n : 1) + 3) & ~(size_t)3;
+        while (rows.size() <= c) rows.push_back(new DevBuf());
+        const size_t each = (sizeof(RowDesc) + 2 * sizeof(int)) * nn;
+        if (!rows[c]->p) CU(rows[c]->alloc(each * kRowsChunk, st));
+        out->rd = reinterpret_cast<RowDesc*>(rows[c]->as<char>() + each * (i % kRowsChunk));
         out->rb = reinterpret_cast<int*>(out->rd + nn);
-        out->re = out->rb + n;
+        out->re = out->rb + nn;
         return PSF_OK;
     }
     RowView pooled(const Rows& r) const { return RowView{r.rb, r.re, pool_col.as<int>(), pool_val.as<double>(), r.rd}; }
@@ -300,10 +319,10 @@ extern thread_local TuneRecorder* g_tune_rec;
 int lsb_for_bound_host(double x);
 RowView view_of(const psf_csr_t& m);
 int check_csr(const psf_csr_t* m, int n, const char* what);
-int read_back(Work& w, Ctl& c, NormSlot* slots);
+int read_back(Work& w, Ctl& c, NormSlot* slots = nullptr, StepStat* stats = nullptr,
+              const StepStat* dev_stats = nullptr, size_t count = 0);
 int status_to_code(int st);
 unsigned long long arena_for(double row_len);
-int mark_pool(Work& w, int i);
 void destroy_result(psf_result_s* r);
 int prepare(cudaStream_t st);
 // Estimates of ||Z^k||_1, k = 2..10, into norms[2..10] (psf_normest.cu);

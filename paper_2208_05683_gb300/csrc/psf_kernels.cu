@@ -756,6 +756,10 @@ __device__ __forceinline__ void write_desc(const ProductArgs& P, int r, const Ro
     P.out_re[r] = d.re;
     P.out_rd[r] = d;
 }
+// step_done of a product step
+__device__ __forceinline__ void product_done(const ProductArgs& P) {
+    step_done(P.ctl, P.mark, P.stat ? &P.stat->pool_start : nullptr, P.start_out, P.cslot, P.ncslot);
+}
 // The descriptor of the entries written at [base, base + n), one per column
 // that has an entry (read back by a lane of the warp that wrote them).
 __device__ __forceinline__ RowDesc stored_row(const ProductArgs& P, long long base, int n) {
@@ -1063,6 +1067,7 @@ __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W
     // unused end of its candidate chunk as holes
     arena_close(st.arena, P.pool_val, lane);
     if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
+    product_done(P);
     if constexpr (BATCH) return;
     // ---- block totals for the step statistics
     st.cand = (unsigned long long)warp_sum((int)st.cand);
@@ -1590,6 +1595,7 @@ __global__ void __launch_bounds__(kCtaWarps * 32, 7) k_product_cta(const __grid_
     for (int r = blockIdx.x; r < P.n; r += gridDim.x) cta_row(P, add, S, st, r, tid);
     if (wib == 0) arena_close(st.arena, P.pool_val, lane);
     if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
+    product_done(P);
     st.cand = (unsigned long long)warp_sum((int)st.cand);
     st.absmax = warp_max_u64(st.absmax);
     for (int o = 16; o; o >>= 1) st.fma += __shfl_xor_sync(kFull, st.fma, o);
@@ -1818,7 +1824,7 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
     int tile = TEAM ? blockIdx.x : blockIdx.x * kBandWarps + wib;
     while (tile < tiles) {
         int next = 0;
-        if (lead && lane == 0) next = first + (int)atomicAdd(P.ticket, 1u);
+        if (lead && lane == 0) next = first + (int)atomicAdd(&P.ctl->ticket, 1u);
         const int r0 = tile * R;
         // ---- lane i < R: row r0 + i's part of A, and what becomes of it (1:
         // folded here, 2: by the accumulator, 0: done)
@@ -2188,6 +2194,7 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
     }
     if (lead) arena_close(st.arena, P.pool_val, lane);
     if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
+    product_done(P);
     if constexpr (BATCH) return;
     // ---- the step statistics, once per block
     __shared__ unsigned long long blk_written, blk_cand, blk_absmax, blk_fma;
@@ -2278,6 +2285,7 @@ __global__ void __launch_bounds__(256) k_reuse_pass1(ReuseArgs R) {
         if (blk_cand) atomicAdd(&R.stat->ncand, blk_cand);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        R.ctl->cslot[0] = R.ctl->cslot[1] = 0ull;  // (Algorithm 1 starts from 0)
         R.stat->fma = R.fma;
         R.stat->pool_start = R.ctl->mark[R.k - 1];
         R.stat->pool_end = R.ctl->mark[R.k];
@@ -2352,6 +2360,7 @@ __global__ void __launch_bounds__(256) k_reuse_copy_batch(ProductArgs P) {
     }
     arena_close(arena, P.pool_val, lane);
     if (P.cand_col) cand_close(carena, P.cand_x, lane);
+    step_done(P.ctl, 0, nullptr, nullptr, nullptr, 0);
 }
 
 // ---------------------------------------------------------------- k_alg1
@@ -3239,6 +3248,21 @@ __global__ void k_row_bitmaps(int n, RowView B, int2* hdr, unsigned* bits) {
 }
 
 // ---------------------------------------------------------------- plumbing
+// An empty pool of `cap` entries and empty candidate lists (the barrier's and
+// the counters' fields from bar_count on keep their values).
+__global__ void k_reset(Ctl* ctl, unsigned long long cap, unsigned long long cand_cap, unsigned cand_chunk) {
+    if (threadIdx.x) return;
+    ctl->pool_used = ctl->pool_mark = 0ull;
+    ctl->pool_cap = cap;
+    ctl->cslot[0] = ctl->cslot[1] = ctl->nnz_total = 0ull;
+    ctl->status = 0;
+    ctl->cand_cnt[0] = ctl->cand_cnt[1] = ctl->cand_far = 0ull;
+    ctl->cand_cap = cand_cap;
+    ctl->cand_over = 0;
+    ctl->cand_chunk = cand_chunk;
+    ctl->dropped = 0;
+}
+
 // max |x| over the pool entries [mark[i], mark[i+1])
 __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot* slot) {
     const int lane = threadIdx.x & 31;
@@ -3287,9 +3311,9 @@ __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, co
 }
 
 // Exclusive scan of row lengths (re - rb, or a pooled matrix's true entries
-// when rd is given) into rowptr (n + 1 entries), in
-// three launches over tiles of kScanTile rows: tile sums, a scan of the tile
-// sums (one block), and the scan inside each tile plus its tile's offset.
+// when rd is given) into rowptr (n + 1 entries), in two launches over tiles of
+// kScanTile rows: the tile sums and their scan, then the scan inside each tile
+// plus its tile's offset.
 // `sums` holds ceil(n / kScanTile) + 1 values.
 constexpr int kScanTile = 1024;
 
@@ -3318,33 +3342,38 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long* par
     return before + x - v;
 }
 
+// The tile sums; the last block to finish scans them.
 __global__ void __launch_bounds__(kScanTile) k_scan_tile_sums(int n, const int* rb, const int* re, const RowDesc* rd,
-                                                              long long* sums) {
+                                                              long long* sums, Ctl* ctl) {
     __shared__ long long part[32];
+    __shared__ int last_block;
     const long long r = (long long)blockIdx.x * kScanTile + threadIdx.x;
     const long long len = r < n ? (long long)(rd ? rd_nnz(rd[r]) : re[r] - rb[r]) : 0;
     long long total;
     block_excl_scan(len, part, &total);
-    if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(kScanTile) k_scan_tiles(int ntiles, long long* sums, Ctl* ctl) {
-    __shared__ long long part[32];
+    const int ntiles = gridDim.x;
+    if (threadIdx.x == 0) {
+        sums[blockIdx.x] = total;
+        __threadfence();
+        last_block = atomicAdd(&ctl->done, 1u) == (unsigned)ntiles - 1u;
+    }
+    __syncthreads();
+    if (!last_block) return;
     // each thread owns a contiguous run of tiles
     const int per = (ntiles + kScanTile - 1) / kScanTile;
-    const int t0 = threadIdx.x * per, t1 = min(ntiles, t0 + per);
+    const int t0 = min(ntiles, (int)threadIdx.x * per), t1 = min(ntiles, t0 + per);
     long long s = 0;
-    for (int t = t0; t < t1; ++t) s += sums[t];
-    long long total;
+    for (int t = t0; t < t1; ++t) s += __ldcg(sums + t);
     long long run = block_excl_scan(s, part, &total);
     for (int t = t0; t < t1; ++t) {
-        const long long v = sums[t];
+        const long long v = __ldcg(sums + t);
         sums[t] = run;
         run += v;
     }
     if (threadIdx.x == 0) {
         sums[ntiles] = total;
         ctl->nnz_total = (unsigned long long)total;
+        ctl->done = 0u;
     }
 }
 
@@ -3396,11 +3425,13 @@ __global__ void k_gather(int n, RowView src, const int* rowptr, int* col, double
 // slot of round-up(len, 4) entries (rows start 16-byte aligned, like the
 // product kernel's rows).
 __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
-                            RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size) {
+                            RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
+                            NormSlot* absmax) {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     Arena arena;
+    unsigned long long mx = 0ull;
     for (int r = gw; r < n; r += nwarps) {
         int s = rowptr[r], e = rowptr[r + 1];
         const long long base = arena_take(arena, (unsigned long long)((e - s + 3) & ~3), arena_size, ctl, pool_val, lane);
@@ -3413,8 +3444,11 @@ __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const doub
         }
         const int padded = (e - s + 3) & ~3;
         for (int q = lane; q < padded; q += 32) {
+            const double v = q < e - s ? val[s + q] : 0.0;
             pool_col[base + q] = q < e - s ? col[s + q] : 0;
-            pool_val[base + q] = q < e - s ? val[s + q] : 0.0;
+            pool_val[base + q] = v;
+            const unsigned long long b = mag_bits(v);
+            mx = b > mx ? b : mx;
         }
         if (lane == 0) {
             rb[r] = (int)base;
@@ -3423,6 +3457,16 @@ __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const doub
         }
     }
     arena_close(arena, pool_val, lane);
+    if (absmax) {  // max |x| (the fixed point of the norm), one atomic per block
+        __shared__ unsigned long long blk;
+        if (threadIdx.x == 0) blk = 0ull;
+        __syncthreads();
+        mx = warp_max_u64(mx);
+        if (lane == 0 && mx) atomicMax(&blk, mx);
+        __syncthreads();
+        if (threadIdx.x == 0 && blk) atomicMax(&absmax->absmax, blk);
+    }
+    step_done(ctl, 1, nullptr, nullptr, nullptr, 0);
 }
 
 // Reset a caller-provided norm workspace for one matrix of n columns and
@@ -3533,6 +3577,7 @@ __global__ void k_copy_rows_batch(int n, const int* inst, const BatchSrc* src, i
         }
     }
     arena_close(arena, pool_val, lane);
+    step_done(ctl, 1, nullptr, nullptr, nullptr, 0);
 }
 
 // out rows <- the rows of matrix sel[inst[r]] of a table of row descriptors.
@@ -3724,15 +3769,26 @@ static void band_launch(const ProductArgs& P, cudaStream_t st) {
 
 cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
     if (P.n <= 0) return cudaSuccess;
-    const long long warps = (long long)sms_now() * 7 * kBandWarps;
-    const bool team = row_len > 192.0 || (P.n <= warps / kBandWarps && row_len > 64.0);
+    // The tile, measured over n = 256..100000 and rows of 5-600 columns.  TEAM
+    // where a warp per tile leaves the chip idle or a tile is long (us, one
+    // warp / team: n = 1000, 41 x 81 entries a row 43.5 / 29.1; n = 5000,
+    // 101 x 101 210 / 189, 41 x 81 79 / 89; n = 10000, 201 x 201 1039 / 869,
+    // 101 x 101 322 / 362).  Four rows a tile where they make about one round
+    // of the chip's warps or several (one row / four: n = 2000, 31 x 61 36 /
+    // 57; n = 12000 91 / 83; n = 20000, 1.2 rounds, 140 / 169; n = 65536
+    // 408 / 375), and for rows of one 32-column piece, which are mostly
+    // set-up (11 x 11: n = 12000 36 / 29, n = 65536 117 / 83).
+    const double warps = sms_now() * 7.0 * kBandWarps;
+    const double rounds = P.n / (4.0 * warps);  // of tiles of four rows
+    const bool team = row_len > 300.0 || (row_len > 128.0 && P.n <= 5.0 * warps / kBandWarps) ||
+                      (row_len > 80.0 && P.n <= 2.0 * warps / kBandWarps);
     if (P.inst) {
         band_launch<true, false, 4>(P, st);
     } else if (team) {
-        if (P.n >= 2 * warps / kBandWarps * 4) band_launch<false, true, 4>(P, st);
+        if (rounds >= 0.9) band_launch<false, true, 4>(P, st);
         else band_launch<false, true, 1>(P, st);
     } else {
-        if (P.n >= 2 * warps * 4) band_launch<false, false, 4>(P, st);
+        if (rounds >= (row_len <= 32.0 ? 0.35 : 3.0) || (rounds <= 1.0 && rounds >= 0.45)) band_launch<false, false, 4>(P, st);
         else band_launch<false, false, 1>(P, st);
     }
     ++g_launches;
@@ -3750,9 +3806,7 @@ cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bit
 }
 
 cudaError_t launch_alg1(const Alg1Args& A, cudaStream_t st) {
-    cudaError_t err = cudaMemsetAsync(&A.ctl->cslot[0], 0, sizeof(A.ctl->cslot), st);
-    if (err != cudaSuccess) return err;
-    Alg1Args a = A;
+    Alg1Args a = A;  // (cslot is 0: step_done)
     a.budget_ns = barrier_budget_ns();
     void* args[] = {&a};
     ++g_launches;
@@ -3788,14 +3842,7 @@ size_t scan_scratch_len(int n) { return (size_t)((n + kScanTile - 1) / kScanTile
 cudaError_t launch_scan_rows(int n, const int* rb, const int* re, const RowDesc* rd, int* rowptr, Ctl* ctl,
                              long long* sums, cudaStream_t st) {
     const int ntiles = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
-    if (n > 0) {
-        k_scan_tile_sums<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums);
-        ++g_launches;
-    } else {
-        cudaError_t err = cudaMemsetAsync(sums, 0, sizeof(long long), st);
-        if (err != cudaSuccess) return err;
-    }
-    k_scan_tiles<<<1, kScanTile, 0, st>>>(ntiles, sums, ctl);
+    k_scan_tile_sums<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums, ctl);
     ++g_launches;
     k_scan_apply<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums, rowptr);
     ++g_launches;
@@ -3850,14 +3897,14 @@ cudaError_t launch_identity(int n, double alpha, int* rowptr, int* col, double* 
 
 cudaError_t launch_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
                              RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
-                             cudaStream_t st) {
+                             NormSlot* absmax, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     // about four rows per warp: each row is a dependent load pair, so the
     // copy is latency-bound and wants many warps in flight
     long long blocks = ((long long)n + 31) / 32;
     if (blocks > (long long)sms_now() * 8) blocks = (long long)sms_now() * 8;
     k_copy_rows<<<(unsigned)blocks, 256, 0, st>>>(n, rowptr, col, val, rb, re, rd, pool_col, pool_val, ctl,
-                                                  arena_size);
+                                                  arena_size, absmax);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -3872,11 +3919,27 @@ cudaError_t launch_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long lon
     return cudaGetLastError();
 }
 
+cudaError_t launch_norm_in_place(Ctl* ctl, NormSlot* slot, unsigned long long* words, unsigned* sticky,
+                                 const psf_csr_t& M, cudaStream_t st) {
+    cudaError_t err = launch_norm_scratch_init(ctl, slot, words, sticky, M.n, M.nnz, st);
+    if (err == cudaSuccess) err = launch_validate(M.n, M.nnz, M.rowptr, M.col, M.val, ctl, st);
+    if (err == cudaSuccess) err = launch_absmax(M.val, ctl, 0, slot, st);
+    if (err != cudaSuccess) return err;
+    NormArgs na{};
+    na.n = M.n;
+    na.count = 1;
+    na.pool_col = M.col;
+    na.pool_val = M.val;
+    na.slots = slot;
+    na.words = words;
+    na.sticky = sticky;
+    na.ctl = ctl;
+    return launch_norms(na, st);
+}
+
 cudaError_t launch_alg1_batch(const Alg1BatchArgs& A, cudaStream_t st) {
     if (A.ninst > kMaxBatch) return cudaErrorInvalidValue;
-    cudaError_t err = cudaMemsetAsync(A.cslot, 0, sizeof(unsigned long long) * 2 * (size_t)A.ninst, st);
-    if (err != cudaSuccess) return err;
-    Alg1BatchArgs a = A;
+    Alg1BatchArgs a = A;  // (cslot is 0: step_done)
     a.budget_ns = barrier_budget_ns();
     void* args[] = {&a};
     ++g_launches;
@@ -3944,6 +4007,13 @@ cudaError_t launch_reuse_copy_batch(const ProductArgs& P, cudaStream_t st) {
     const long long cap = (long long)num_sms() * 8;
     if (blocks > cap) blocks = cap;
     k_reuse_copy_batch<<<(unsigned)blocks, 256, 0, st>>>(P);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reset(Ctl* ctl, unsigned long long cap, unsigned long long cand_cap, unsigned cand_chunk,
+                         cudaStream_t st) {
+    k_reset<<<1, 32, 0, st>>>(ctl, cap, cand_cap, cand_chunk);
+    ++g_launches;
     return cudaGetLastError();
 }
 

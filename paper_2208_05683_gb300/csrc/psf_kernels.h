@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "../../include/psf.h"
 #include "psf_device.cuh"
 
 namespace psf {
@@ -34,6 +35,9 @@ cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st);
 // column bitmaps of B's rows for the product's symbolic pass
 // (ProductArgs::bhdr, bbits); bits has one word per entry of B's index space
 cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bits, cudaStream_t st);
+// an empty pool (the control block before bar_count)
+cudaError_t launch_reset(Ctl* ctl, unsigned long long cap, unsigned long long cand_cap, unsigned cand_chunk,
+                         cudaStream_t st);
 // bytes (a multiple of 4) of device memory at src to dst, the device address
 // of pinned, mapped host memory, by a kernel on st (k_export)
 cudaError_t launch_export(const void* src, void* dst, size_t bytes, cudaStream_t st);
@@ -51,7 +55,12 @@ cudaError_t launch_gather(int n, const RowView& src, const int* rowptr, int* col
 cudaError_t launch_identity(int n, double alpha, int* rowptr, int* col, double* val, cudaStream_t st);
 cudaError_t launch_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
                              RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
-                             cudaStream_t st);
+                             NormSlot* absmax, cudaStream_t st);
+// exact ||M||_1 of a caller's matrix, its entries read in place, into
+// slot->result: workspace cleared, input checked (ctl->status), max |x|, sums.
+// words: kChunks n, sticky: n
+cudaError_t launch_norm_in_place(Ctl* ctl, NormSlot* slot, unsigned long long* words, unsigned* sticky,
+                                 const psf_csr_t& M, cudaStream_t st);
 cudaError_t launch_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long long* words, unsigned* sticky, int n,
                                      long long nnz, cudaStream_t st);
 // batches (block-diagonal matrix of instances)
