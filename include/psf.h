@@ -441,8 +441,12 @@ PSF_API int psf_plan(const double* coeffs, int64_t m, int32_t s, double tol, uin
  * 1 (default): for products whose A rows average at least 12 entries and
  * whose B rows average at least 32 (each B row is marked many times and has
  * words to share; the giant steps of near-sparse series).  2: for every
- * product.  Results are the same either way; with 0 a call allocates no
- * bitmap words. */
+ * product.  With 1 and 2, a product of rows that span more columns than the
+ * bitmap map covers, but have entries in few of their words, is marked from
+ * lists of those words instead (two words per entry of the entry pool,
+ * allocated by the first such product of a call; without memory for them it
+ * takes the wide bitmap window).  Results are the same either way; with 0 a
+ * call allocates no bitmap words. */
 #define PSF_TUNE_ROW_BITMAPS 8
 PSF_API int psf_tune_set(int32_t key, double value);
 PSF_API int psf_tune_get(int32_t key, double* value);

@@ -179,6 +179,7 @@ int validate_inputs(Work& w, const std::vector<const psf_csr_t*>& ms) {
     int rc = read_back(w, c);
     if (rc) return rc;
     w.band = !c.not_band;
+    w.bandwidth = (int)c.bandwidth;
     return status_to_code(c.status);
 }
 
@@ -193,16 +194,14 @@ unsigned long long arena_for(double row_len) {
 
 // Launch one product step into matrix slot `slot`, with Algorithm 1 when
 // threshold > 0.
-// wide_window: the previous evaluation's rows of this step spanned more
-// columns than one bitmap chunk (kBitmapColumns), so the bitmap map's wide
-// window is used.
+// window: the column window its rows are expected to need (window_for).
 // reuse_k > 0: the step is baby step k and row slot `slot` still holds the
 // norm phase's Z^k; while no entry has been dropped (a device flag), the
 // product is skipped and k_reuse_pass1 does the step on those rows.
 int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddTerm>& add,
              double threshold, double e_r, int maxit, StepStat* stat, size_t slot, RowView* out,
              NormSlot* absmax_slot = nullptr, double blen = 0.0, double alen = 0.0, int reuse_k = 0,
-             unsigned long long reuse_fma = 0, double out_len = 0.0, bool wide_window = false,
+             unsigned long long reuse_fma = 0, double out_len = 0.0, int window = kNarrow,
              double fma_hint = 0.0, int mark = 0) {
     if (add.size() > (size_t)kMaxAdd) return fail(PSF_ETOOBIG, "%zu addend terms (max %d)", add.size(), kMaxAdd);
     Rows R;
@@ -278,7 +277,15 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         // one launch over B); the chunked test settings keep the column marks
         const int bm = g_row_bitmaps.load();
         const bool band = w.band && w.slot_map == 0 && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
-        if (A && !table && !band && bm > 0 && w.bits_cap >= w.cap && w.chunk_cols <= 0 && w.chunk_slots <= 0 &&
+        uint2* const pl = A && !table && !band && bm > 0 && window == kLists && w.slot_map == 0 && w.chunk_cols <= 0 &&
+                                  w.chunk_slots <= 0
+                              ? w.lists()
+                              : nullptr;
+        if (pl) {
+            CU(launch_row_lists(w.n, *B, w.bhdr.as<int2>(), pl, w.st));
+            P.bhdr = w.bhdr.as<int2>();
+            P.blists = pl;
+        } else if (A && !table && !band && bm > 0 && w.bits_cap >= w.cap && w.chunk_cols <= 0 && w.chunk_slots <= 0 &&
             (bm == 2 || (alen >= kBitmapMinA && blen >= kBitmapMinB))) {
             CU(launch_row_bitmaps(w.n, *B, w.bhdr.as<int2>(), w.pool_bits.as<unsigned>(), w.st));
             P.bhdr = w.bhdr.as<int2>();
@@ -286,7 +293,7 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         }
         const bool cta = A && !table && (w.slot_map == 4 || (w.slot_map == 0 && use_cta(w.n, alen, blen)));
         if (band) CU(launch_band(P, A ? alen + blen : 0.0, w.st));
-        else CU(launch_product(P, table, w.st, out_len, wide_window || w.slot_map == 3, cta));
+        else CU(launch_product(P, table, w.st, out_len, window != kNarrow || w.slot_map == 3, cta));
     }
     if (reuse_k > 0) {
         ReuseArgs U{};
@@ -707,13 +714,23 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     w.dense_xover = series->dense_xover >= 0.0 ? series->dense_xover : g_dense_xover.load();
     // the column windows the series' previous evaluation measured (batches on
     // other threads may update them)
-    std::vector<unsigned> span_z, span_baby, span_giant;
+    std::vector<unsigned> span_z, span_baby, span_giant, words_z, words_baby, words_giant;
     {
         std::lock_guard<std::mutex> lock(series->span_mu);
         span_z = series->span_z;
         span_baby = series->span_baby;
         span_giant = series->span_giant;
+        words_z = series->words_z;
+        words_baby = series->words_baby;
+        words_giant = series->words_giant;
     }
+    // the window of a step: by its record, or what e applications of Z reach
+    // from a row with `words` words
+    auto window_of = [&](const std::vector<unsigned>& span, const std::vector<unsigned>& words, size_t i, double e,
+                         double est) {
+        if (i < span.size()) return window_for(span[i], i < words.size() ? (double)words[i] : 0.0);
+        return window_for(std::min((double)n, 2.0 * e * w.bandwidth + 1.0), est);
+    };
     w.chunk_cols = series->chunk_cols;
     w.chunk_slots = series->chunk_slots;
     const RowView vz = view_of(*Z);
@@ -736,6 +753,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     unsigned long long zcap = series->pool_hint;
     if (zcap < series->z_need + series->z_need / 8) zcap = series->z_need + series->z_need / 8;
     unsigned long long z_used = 0, z_fma = 0;
+    double z_words10 = 0.0;  // most words of a row of Z^10
     // Once the series knows what its PS phase needs, the pool holds both
     // phases: the PS phase continues after the powers Z^2..Z^10, whose
     // leading ones double as baby steps while nothing is dropped.
@@ -774,7 +792,9 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                         RowView cur;
                         double blen = (size_t)(i - 2) < series->len_z.size() ? series->len_z[(size_t)(i - 2)]
                                                                               : zlen * (i - 1) * (i - 1);
-                        const bool wz = (size_t)(i - 2) < span_z.size() && span_z[(size_t)(i - 2)] > kBitmapColumns;
+                        // (a first evaluation: entries of about half a square's growth, a word
+                        // or two for each run of them)
+                        const int wz = window_of(span_z, words_z, (size_t)(i - 2), i, 0.35 * zlen * i * i);
                         if ((rc = run_step(w, &vz, &prev, {}, 0.0, 0.0, 1, w.front_stats() + (i - 2), (size_t)(i - 2),
                                            &cur, slots + i, blen, zlen, 0, 0ull, 0.0, wz, 0.0, i)))
                             return rc;
@@ -813,8 +833,12 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     series->len_z[(size_t)(i - 2)] = znnz[i - 1] / n;
                     sz[(size_t)(i - 2)] = zs[i - 2].span_max;
                 }
+                std::vector<unsigned> sw(9, 0u);
+                for (int i = 2; i <= 10; ++i) sw[(size_t)(i - 2)] = zs[i - 2].words_max;
                 std::lock_guard<std::mutex> lock(series->span_mu);
                 series->span_z = sz;
+                series->words_z = sw;
+                z_words10 = sw[8];
             }
             // ||Z||_1 always; Z^2..Z^10 when the chain ran (else estimated above)
             for (int i = 1; i <= (chain || submult ? 10 : 1); ++i) {
@@ -910,7 +934,9 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                                                                          : pow_len(k);
                 // baby step k + 1 writes row slot k - 1, the slot of the norm phase's Z^(k+1)
                 const int rk = (reuse && !square && k + 1 <= 10 && slot == (size_t)(k - 1)) ? k + 1 : 0;
-                const bool wb = (size_t)(k - 1) < span_baby.size() && span_baby[(size_t)(k - 1)] > kBitmapColumns;
+                const double eb = (double)stride * (k + 1);
+                int wb = window_of(span_baby, words_baby, (size_t)(k - 1), eb, z_words10 * eb / 10.0);
+                if (rk && wb == kLists) wb = kWide;  // (mostly skipped: no launch over B for it)
                 if ((rc = run_step(w, &vm, &Zh[(size_t)k], {}, thr, series->e_r, series->maxit, pstat + si, slot++,
                                    &Zh[(size_t)k + 1], nullptr, blen, pow_len(1), rk, rk ? zfma[rk] : 0ull, 0.0, wb)))
                     return rc;
@@ -977,7 +1003,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     const double alen = pow_len(q);
                     const double olen =
                         (size_t)(i - 1) < series->out_giant.size() ? series->out_giant[(size_t)(i - 1)] : 0.0;
-                    const bool wg = (size_t)(i - 1) < span_giant.size() && span_giant[(size_t)(i - 1)] > kBitmapColumns;
+                    const double eg = (double)stride * q * (i + 1);
+                    const int wg = window_of(span_giant, words_giant, (size_t)(i - 1), eg, z_words10 * eg / 10.0);
                     const double fh =
                         (size_t)(i - 1) < series->fma_giant.size() ? series->fma_giant[(size_t)(i - 1)] : 0.0;
                     if ((rc = run_step(w, &Zh[(size_t)q], &S, add, thr, series->e_r, series->maxit, pstat + si, sslot[nslot],
@@ -1041,12 +1068,14 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
             series->fma_giant.assign((size_t)(b > 1 ? b - 1 : 0), 0.0);
             series->out_giant.assign((size_t)(b > 1 ? b - 1 : 0), 0.0);
             std::vector<unsigned> sb((size_t)(q > 1 ? q - 1 : 0), 0u), sg((size_t)(b > 1 ? b - 1 : 0), 0u);
+            std::vector<unsigned> wsb(sb), wsg(sg);
             {
                 double prev_len = pow_len(1);  // Z-hat_(1) = Z or W
                 size_t idx = 0;
                 for (int k = 1; k < q; ++k, ++idx) {
                     series->len_baby[(size_t)(k - 1)] = prev_len;
                     sb[(size_t)(k - 1)] = ss[idx].span_max;
+                    wsb[(size_t)(k - 1)] = ss[idx].words_max;
                     prev_len = (double)steps[idx].nnz_post / n;
                 }
                 double s_len = 0.0;
@@ -1054,6 +1083,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 for (int i = 1; i < b; ++i, ++idx) {
                     series->len_giant[(size_t)(i - 1)] = s_len;
                     sg[(size_t)(i - 1)] = ss[idx].span_max;
+                    wsg[(size_t)(i - 1)] = ss[idx].words_max;
                     series->out_giant[(size_t)(i - 1)] = (double)steps[idx].nnz_pre / n;
                     series->fma_giant[(size_t)(i - 1)] = (double)steps[idx].fma;
                     s_len = (double)steps[idx].nnz_post / n;
@@ -1064,6 +1094,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 std::lock_guard<std::mutex> lock(series->span_mu);
                 series->span_baby = sb;
                 series->span_giant = sg;
+                series->words_baby = wsb;
+                series->words_giant = wsg;
             }
             if ((rc = finish_result(w, F, r, c.nnz_total))) {
                 destroy_result(r);

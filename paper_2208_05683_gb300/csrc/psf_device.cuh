@@ -47,6 +47,7 @@ struct Ctl {
     int pad1;
     unsigned bar_count;  // fields from here on survive a pool reset
     unsigned bar_gen;
+    unsigned bandwidth;  // of the checked inputs: max |column - row|
     int not_band;  // an input has a row that does not span consecutive columns
     unsigned done;    // blocks of the running launch that have finished (0 between launches)
     unsigned ticket;  // k_band's tile counter (0 between launches)
@@ -62,6 +63,8 @@ struct StepStat {
     double eps_f, dropped;
     int iters;
     unsigned span_max;  // widest column window of the product's rows (hi - lo + 1)
+    unsigned words_max; // most 32-column words that one of its rows has entries in
+    unsigned pad;
 };
 
 // Per-matrix norm slot for the exact 1-norm kernel.
@@ -181,6 +184,10 @@ struct ProductArgs {
     // no bitmap)
     const int2* bhdr;
     const unsigned* bbits;
+    // the wide window's form of the same (nullptr: none): bhdr[k].y = words of
+    // row k that hold entries, listed as {column / 32, bitmap} at
+    // blists[B.rb[k]] on, columns ascending
+    const uint2* blists;
     // batch: instances whose rows k_band computes (nullptr: none)
     const unsigned char* band;
     // written by the launch's last block (step_done)

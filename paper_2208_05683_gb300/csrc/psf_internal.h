@@ -40,6 +40,9 @@ struct psf_series_s {
     // is used where it exceeded kBitmapColumns); batches, which may run
     // concurrently on one series, read and write them under span_mu
     std::vector<unsigned> span_z, span_baby, span_giant;
+    // most words of 32 columns that one of a step's rows has entries in (the
+    // list map is used for wide windows of few words)
+    std::vector<unsigned> words_z, words_baby, words_giant;
     std::mutex span_mu;
     int kernel = 0;       // PSF_PARAM_KERNEL
     int chunk_cols = 0;   // PSF_PARAM_CHUNK_COLS
@@ -166,6 +169,9 @@ struct Work {
     size_t sums_bytes = 0;  // words and sticky
     DevBuf dense[3];  // the dense-tile path's A, B and C (n^2 doubles each), allocated on first use
     DevBuf bhdr, pool_bits;  // column bitmaps of a product's B rows: n headers, a word per pool entry
+    DevBuf pool_lists;       // the list map's form: a pair per pool entry, allocated on first use
+    unsigned long long lists_cap = 0;
+    int bandwidth = 0;       // of the checked inputs
     double dense_xover = 1e300;  // dense tiles for a step with at least this many multiply-adds per n^3
     bool dense_estimate = false;  // a step without a recorded count may use the row-length estimate
     unsigned long long cap = 0, ccap = 0, bits_cap = 0;
@@ -247,6 +253,20 @@ struct Work {
         CU(launch_reset(C(), cap, ccap, cand_chunk(), st));
         return PSF_OK;
     }
+    // the lists' memory; null where there is none left (the step then takes the
+    // wide bitmap window, which needs none)
+    uint2* lists() {
+        if (lists_cap < cap) {
+            lists_cap = 0;
+            if (pool_lists.alloc(sizeof(uint2) * cap, st) != cudaSuccess) {
+                pool_lists.p = nullptr;
+                cudaGetLastError();
+                return nullptr;
+            }
+            lists_cap = cap;
+        }
+        return pool_lists.as<uint2>();
+    }
     // Entries a warp reserves in a candidate list at a time: up to 128, so
     // that about 12k warps' unused chunk ends take at most a quarter of it.
     unsigned cand_chunk() const {
@@ -306,6 +326,22 @@ inline bool use_table(int slot_map, double work_per_row) {
 inline bool use_cta(int n, double alen, double blen) {
     (void)alen;
     return n > 0 && n <= 7 * num_sms() && blen >= 16.0;
+}
+
+// A step's column window: the bitmap map's own, its wide one, or the list map
+// (wide, and its rows have entries in few words).  span, words: the widest
+// row's columns and the most words of a row, in the previous evaluation or as
+// far as this one can tell (words 0: unknown).  The line lies at the narrow
+// window's edge because the two are level there: on a 512 x 512 grid (tol
+// 1e-12) a product of rows spanning 4097 columns takes 740 us in the narrow
+// window, and one of 5121 takes 846 with the list map and 1155 in the wide
+// window; then 6145: 900 / 1303, 10241: 1519 / 2277, and the giant steps
+// S_1..S_5 4.1 / 3.9, 5.7 / 9.0, 8.0 / 12.5, 11.3 / 17.4, 16.1 / 37.8 ms (the
+// last ones exceed the wide window's 16384 columns).
+enum Window { kNarrow = 0, kWide = 1, kLists = 2 };
+inline int window_for(double span, double words) {
+    if (!(span > kBitmapColumns)) return kNarrow;
+    return words > 0.0 && words <= kListMapWords ? kLists : kWide;
 }
 
 // Recorder of product launches for psf_autotune (set on the calling thread

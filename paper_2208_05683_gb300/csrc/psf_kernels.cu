@@ -13,6 +13,7 @@
 //  k_band         the same step where rows span consecutive columns: outputs
 //                 folded in registers.
 //  k_row_bitmaps  column bitmaps of B's rows for the symbolic pass.
+//  k_row_lists    the same as lists of the words in use, for the list map.
 //  k_reuse_pass1  a baby step equal to a power of the norm phase: the first
 //                 pass of Algorithm 1 on that power's rows.
 //  k_reuse_copy_batch  the same for the instances of a batch: those rows
@@ -69,6 +70,21 @@ constexpr int kBmBits = kBmWords * 32;
 // at 5 blocks per SM instead of 7.
 constexpr int kBmWordsBig = 512;
 static_assert(kBmBits == kBitmapColumns, "the host's notion of the bitmap window");
+// The list map, for rows that span yet more columns but have entries in few
+// of their 32-column words (on a grid of side M a row of radius r has 2r + 1
+// runs of at most 2r + 1 columns, M apart): a byte per word of a 32768-column
+// window says which of up to kListIds words in use it is; prefix and bitmap
+// are kept for those alone.  B rows come as lists of their words, so marking
+// one costs its words, not its columns, and the map of a row with more
+// entries than slots serves all its column chunks.  Bound by instructions
+// issued (the last giant step of exp on a 512 x 512 grid: 6.6 G warp
+// instructions at 40 % of the issue slots, FP64 pipe 53 %); 160 ids leave six
+// blocks an SM their shared memory (192: five).  That step took
+// 37.8 ms with 16384-column bitmaps and takes 16.1; the evaluation 104 -> 64.
+constexpr int kListWords = 1024;
+constexpr int kListIds = kListMapWords;
+constexpr unsigned kNoId = 0xffu;
+static_assert(kListIds < (int)kNoId, "an id fits a byte");
 // Accumulator slots; with 7 bitmap blocks of 4 warps per SM shared memory is
 // full.  The bitmap map keeps a segment's a_rk in the last 32 slots, so a row
 // has kAccCap - 32 of them; its WIDE instantiation, for steps whose rows are
@@ -105,6 +121,20 @@ struct ProdSmem<false, W> {
     unsigned short colbuf[kAccCap];
 };
 
+template <>
+struct ProdSmem<false, kListWords> {
+    static constexpr int kCols = kListWords * 32;
+    static constexpr int kWarps = 4;
+    static constexpr int kBlocksPerSm = 6;
+    uint2 pm[kListIds];  // by id: set bits before the word, bitmap
+    double acc[kAccCap];
+    int kb[32];
+    int kl[32];
+    unsigned short colbuf[kAccCap];
+    unsigned short word[kListIds];  // id -> window word
+    unsigned char id[kListWords];   // window word -> id (kNoId: no entry)
+};
+
 template <bool TAB, int W = kBmWords>
 size_t prod_smem_bytes() {
     return sizeof(ProdSmem<TAB, W>) * ProdSmem<TAB, W>::kWarps + sizeof(AddTerm) * kMaxAdd;
@@ -128,6 +158,11 @@ __device__ __forceinline__ int slot_lookup(const ProdSmem<true>& S, int o) { ret
 template <int W>
 __device__ __forceinline__ int slot_lookup(const ProdSmem<false, W>& S, int o) {
     const uint2 e = S.pm[o >> 5];
+    return (int)e.x + __popc(e.y << (~o & 31)) - 1;
+}
+
+__device__ __forceinline__ int slot_lookup(const ProdSmem<false, kListWords>& S, int o) {
+    const uint2 e = S.pm[S.id[o >> 5]];
     return (int)e.x + __popc(e.y << (~o & 31)) - 1;
 }
 
@@ -415,7 +450,7 @@ __device__ __forceinline__ void build_map(const ProductArgs& P, const AddTerm* a
 }
 
 // number of marked columns in [0, wlen)
-__device__ __forceinline__ int count_marks(int wlen, int lane, const ProdSmem<true>& S) {
+__device__ __forceinline__ int count_marks(int wlen, int lane, const ProdSmem<true>& S, int& /*words*/) {
     int total = 0;
     for (int i0 = 0; i0 < wlen; i0 += 32) {
         int i = i0 + lane;
@@ -423,11 +458,17 @@ __device__ __forceinline__ int count_marks(int wlen, int lane, const ProdSmem<tr
     }
     return total;
 }
+// (the upper half: words with a mark, for the map's choice)
 template <int W>
-__device__ __forceinline__ int count_marks(int wlen, int lane, const ProdSmem<false, W>& S) {
+__device__ __forceinline__ int count_marks(int wlen, int lane, const ProdSmem<false, W>& S, int& words) {
     int s = 0;
-    for (int w = lane; w < ((wlen + 31) >> 5); w += 32) s += __popc(S.pm[w].y);
-    return warp_sum(s);
+    for (int w = lane; w < ((wlen + 31) >> 5); w += 32) {
+        const unsigned b = S.pm[w].y;
+        s += __popc(b) + (b ? 1 << 16 : 0);
+    }
+    s = warp_sum(s);
+    words += s >> 16;
+    return s & 0xffff;
 }
 
 // Number the marked columns of [0, wlen) in ascending order and fill
@@ -728,6 +769,164 @@ __device__ __forceinline__ void accumulate_segment(const ProductArgs& P, int seg
     }
 }
 
+// ---- the list map
+__device__ __forceinline__ void clear_map(int wlen, int lane, ProdSmem<false, kListWords>& S) {
+    unsigned* id4 = reinterpret_cast<unsigned*>(S.id);
+    for (int i = lane; i < (wlen + 127) >> 7; i += 32) id4[i] = 0xffffffffu;
+}
+// OR `bits` into window word w for the active lanes, whose words are
+// distinct; nid: words in use so far (past kListIds: the map is full, and the
+// mark is dropped).
+__device__ __forceinline__ void list_or(ProdSmem<false, kListWords>& S, bool active, int w, unsigned bits, int& nid) {
+    const unsigned i = active ? S.id[w] : 0u;
+    const bool fresh = active && i == kNoId;
+    const unsigned m = __ballot_sync(kFull, fresh);
+    if (fresh) {
+        const int j = nid + __popc(m & lanemask_lt());
+        if (j < kListIds) {
+            S.id[w] = (unsigned char)j;
+            S.word[j] = (unsigned short)w;
+            S.pm[j] = make_uint2(0u, bits);
+        }
+    } else if (active) {
+        S.pm[i].y |= bits;
+    }
+    nid += __popc(m);
+    __syncwarp();
+}
+// The columns of [c0, cend) among the row [s, e) (ascending), 32 at a time:
+// the lanes of one word form a run, whose bits a segmented OR collects.
+__device__ __forceinline__ void list_mark_row(const int* __restrict__ col, int s, int e, int c0, int cend, int lane,
+                                              ProdSmem<false, kListWords>& S, int& nid) {
+    for (int q0 = s; q0 < e; q0 += 32) {
+        const int q = q0 + lane;
+        const int c = q < e ? col[q] : INT_MAX;
+        const bool in = c >= c0 && c < cend;
+        const int w = in ? (c - c0) >> 5 : -1 - lane;
+        unsigned v = in ? 1u << ((c - c0) & 31) : 0u;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned v2 = __shfl_down_sync(kFull, v, d);
+            const int w2 = __shfl_down_sync(kFull, w, d);
+            if (lane + d < 32 && w2 == w) v |= v2;
+        }
+        const int wp = __shfl_up_sync(kFull, w, 1);
+        list_or(S, in && (lane == 0 || wp != w), w, v, nid);
+    }
+}
+// Mark every output column of row r in [c0, cend), c0 a multiple of 32;
+// returns the words in use (more than kListIds: the window is too wide).
+__device__ __forceinline__ int list_build(const ProductArgs& P, const AddTerm* add, int nadd, int r, int c0, int cend,
+                                          int pa0, int pa1, int lane, ProdSmem<false, kListWords>& S, int ab, int ae) {
+    int nid = 0;
+    clear_map(cend - c0, lane, S);
+    __syncwarp();
+    for (int t = 0; t < nadd; ++t) {
+        if (!add[t].rd) {
+            list_or(S, lane == 0 && r >= c0 && r < cend, (r - c0) >> 5, 1u << ((r - c0) & 31), nid);
+        } else {
+            list_mark_row(P.pool_col, __shfl_sync(kFull, ab, t), __shfl_sync(kFull, ae, t), c0, cend, lane, S, nid);
+        }
+    }
+    const int wb = c0 >> 5;
+    const unsigned nw = (unsigned)((cend - c0 + 31) >> 5);
+    for (int seg = pa0; seg < pa1 && nid <= kListIds; seg += 32) {
+        const int cnt = min(32, pa1 - seg);
+        if (lane < cnt) {
+            const int k = P.A.col[seg + lane];
+            S.kb[lane] = P.B.rb[k];
+            S.kl[lane] = P.bhdr[k].y;
+        }
+        __syncwarp();
+        // four B rows' first words are loaded before any is marked
+        for (int i0 = 0; i0 < cnt; i0 += 4) {
+            uint2 t[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                t[j] = make_uint2(0xffffffffu, 0u);
+                if (i0 + j < cnt && lane < S.kl[i0 + j]) t[j] = P.blists[S.kb[i0 + j] + lane];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (i0 + j >= cnt) break;
+                const int m = S.kl[i0 + j];
+                const unsigned w = t[j].x - (unsigned)wb;
+                list_or(S, lane < m && w < nw, (int)w, t[j].y, nid);
+                for (int l0 = 32; l0 < m; l0 += 32) {
+                    uint2 x = make_uint2(0xffffffffu, 0u);
+                    if (l0 + lane < m) x = P.blists[S.kb[i0 + j] + l0 + lane];
+                    const unsigned w2 = x.x - (unsigned)wb;
+                    list_or(S, l0 + lane < m && w2 < nw, (int)w2, x.y, nid);
+                }
+            }
+        }
+        __syncwarp();
+    }
+    return nid;
+}
+// The same for the widest window from c0 on that the map holds (cend is cut,
+// to a multiple of 32); returns the columns marked (ids: the words in use).
+__device__ __forceinline__ int list_chunk(const ProductArgs& P, const AddTerm* add, int nadd, int r, int c0, int& cend,
+                                          int pa0, int pa1, int lane, ProdSmem<false, kListWords>& S, int ab, int ae,
+                                          int& words, int& ids) {
+    for (;;) {
+        const int nid = list_build(P, add, nadd, r, c0, cend, pa0, pa1, lane, S, ab, ae);
+        if (nid <= kListIds) {
+            int s = 0;
+            for (int i = lane; i < nid; i += 32) s += __popc(S.pm[i].y);
+            words += nid;
+            ids = nid;
+            return warp_sum(s);
+        }
+        words = max(words, kListIds + 1);
+        cend = c0 + max(32, ((cend - c0) / 2) & ~31);
+    }
+}
+// Number the columns from window word `from` on in ascending order and fill
+// colbuf, whole words of them while they fit `cap` slots; returns their count, *cut: the offset of the
+// first word without slots (wlen if all fit).
+__device__ __forceinline__ int assign_slots(int wlen, int cap, int lane, ProdSmem<false, kListWords>& S, int* cut,
+                                            int from, int ids) {
+    const int nw = (wlen + 31) >> 5, per = (nw - from + 31) >> 5;
+    const int b = min(nw, from + lane * per), e = min(nw, b + per);
+    int s = 0;
+    for (int w = b; w < e; ++w) {
+        const unsigned i = S.id[w];
+        if (i != kNoId) s += __popc(S.pm[i].y);
+    }
+    int run = warp_excl_scan(s, lane);
+    const int total = __shfl_sync(kFull, run + s, 31);
+    int cw = nw;  // first word that does not fit
+    int cs = total;
+    for (int w = b; w < e; ++w) {
+        const unsigned i = S.id[w];
+        if (i == kNoId) continue;
+        const unsigned bits = S.pm[i].y;
+        S.pm[i].x = (unsigned)run;
+        if (run + __popc(bits) > cap && cw == nw) {
+            cw = w;
+            cs = run;
+        }
+        run += __popc(bits);
+    }
+    int cutoff = wlen, cnt = total;
+    if (total > cap) {
+        const int w = warp_min(cw);
+        cnt = warp_min(cw == w ? cs : INT_MAX);
+        cutoff = w * 32;
+    }
+    __syncwarp();
+    // the words in use, one a turn: lane l takes bit l
+    for (int i = 0; i < ids; ++i) {
+        const uint2 p = S.pm[i];
+        const int o = S.word[i] * 32 + lane;
+        if ((p.y >> lane & 1u) && o >= from * 32 && o < cutoff) S.colbuf[p.x + __popc(p.y & lanemask_lt())] = (unsigned short)o;
+    }
+    __syncwarp();
+    *cut = cutoff;
+    return cnt;
+}
+
 // Statistics of one row of a batched step, added to its instance's record:
 // multiply-adds (per-lane partial counts), Algorithm 1 candidates (per lane),
 // entries written and the largest |x| (per lane).
@@ -770,7 +969,8 @@ __device__ __forceinline__ RowDesc stored_row(const ProductArgs& P, long long ba
 // Per-warp state of the product kernel across the rows a warp processes.
 struct RowState {
     unsigned long long written = 0ull, cand = 0ull, absmax = 0ull, fma = 0ull;
-    int span = 0;  // widest column window of this warp's rows
+    int span = 0;   // widest column window of this warp's rows
+    int words = 0;  // most words that one of them has entries in
     Arena arena;
     CandArena carena;
 };
@@ -828,7 +1028,8 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     int lo = INT_MAX, hi = -1;
     bool fixed = false;
     int fixed_span = 0;
-    if constexpr (!TAB) {
+    constexpr bool LIST = !TAB && W == kListWords;
+    if constexpr (!TAB && !LIST) {
         int w0 = 0, w1 = P.n;
         if constexpr (BATCH) {
             w1 = -1;
@@ -893,19 +1094,28 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     // ---- exact entry count of the row, reserve it in the pool
     long long total = 0;
     bool reuse = false;
-    if (hi - lo + 1 <= kCols) {
+    int words = 0, ids = 0;
+    if constexpr (LIST) {
+        for (long long c0 = lo; c0 <= hi;) {
+            int cend = (int)min((long long)hi + 1, c0 + kCols);
+            total += list_chunk(P, add, nadd, r, (int)c0, cend, pa0, pa1, lane, S, ab, ae, words, ids);
+            reuse = c0 == lo && cend == hi + 1;
+            c0 = cend;
+        }
+    } else if (hi - lo + 1 <= kCols) {
         build_map<TAB, (!BATCH || W == kBmWords), !BATCH>(P, add, nadd, tmask, r, lo, hi + 1, pa0, pa1, true, lane, S,
                                                    !WIDE, ab, ae, a_holes, fixed ? &my_fma : nullptr);
-        total = count_marks(hi - lo + 1, lane, S);
+        total = count_marks(hi - lo + 1, lane, S, words);
         reuse = true;
     } else {
         for (long long c0 = lo; c0 <= hi; c0 += kCols) {
             int cend = (int)min((long long)hi + 1, c0 + kCols);
             build_map<TAB, false, !BATCH>(P, add, nadd, tmask, r, (int)c0, cend, pa0, pa1, false, lane, S, !WIDE, ab,
                                           ae);
-            total += count_marks(cend - (int)c0, lane, S);
+            total += count_marks(cend - (int)c0, lane, S, words);
         }
     }
+    st.words = max(st.words, words);
     const long long base = arena_take(arena, (unsigned long long)((total + 3) & ~3LL), P.arena, P.ctl, P.pool_val, lane);
     if (base < 0) {
         if (lane == 0) write_desc(P, r, RowDesc{0, 0, 0, 0});
@@ -926,14 +1136,30 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
     const bool single = reuse && total <= slots;
     int written = 0;
     int c0 = lo;
+    // the map's columns are [m0, mend): a chunk's, but the list map's serves
+    // every chunk of slots inside them
+    int m0 = lo, mend = LIST && reuse ? hi + 1 : lo;
     while (c0 <= hi) {
         int cend = (int)min((long long)hi + 1, (long long)c0 + kCols);
-        if (!reuse)
+        if constexpr (LIST) {
+            if (c0 >= mend) {
+                int w = 0;
+                list_chunk(P, add, nadd, r, c0, cend, pa0, pa1, lane, S, ab, ae, w, ids);
+                m0 = c0;
+                mend = cend;
+            }
+            cend = mend;
+        } else if (!reuse) {
             build_map<TAB, false, !BATCH>(P, add, nadd, tmask, r, c0, cend, pa0, pa1, false, lane, S, !WIDE, ab, ae);
+        }
+        if constexpr (!LIST) m0 = c0;
         reuse = false;
-        int cut;
-        const int cnt = assign_slots(cend - c0, slots, lane, S, &cut);
-        const int c1 = c0 + cut;
+        int cut, cnt;
+        if constexpr (LIST)
+            cnt = assign_slots(cend - m0, slots, lane, S, &cut, (c0 - m0) >> 5, ids);
+        else
+            cnt = assign_slots(cend - m0, slots, lane, S, &cut);
+        const int c1 = m0 + cut;
         for (int i = lane; i < cnt; i += 32) S.acc[i] = 0.0;
         __syncwarp();
 
@@ -945,7 +1171,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
             const double alpha = BATCH ? P.alpha_tab[(size_t)t * P.ninst + r_inst] : T.alpha;
             if (!T.rd) {
                 if (lane == 0 && r >= c0 && r < c1) {
-                    int i = slot_lookup(S, r - c0);
+                    int i = slot_lookup(S, r - m0);
                     S.acc[i] = __fma_rn(alpha, 1.0, S.acc[i]);
                 }
             } else {
@@ -953,7 +1179,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
                 for (int q = s + lane; q < e; q += 32) {
                     int c = P.pool_col[q];
                     if (c >= c0 && c < c1) {
-                        int i = slot_lookup(S, c - c0);
+                        int i = slot_lookup(S, c - m0);
                         S.acc[i] = __fma_rn(alpha, P.pool_val[q], S.acc[i]);
                     }
                 }
@@ -965,7 +1191,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
         for (int seg = pa0; seg < pa1; seg += 32) {
             const int cnt_seg = min(32, pa1 - seg);
             load_segment<TAB>(P, seg, cnt_seg, single, c0, c1, lane, S, !wide_row, false);
-            accumulate_segment<WIDE>(P, seg, cnt_seg, c0, lane, S, wide_row);
+            accumulate_segment<WIDE>(P, seg, cnt_seg, m0, lane, S, wide_row);
         }
 
         // ---- write back the nonzero entries in column order; the entries
@@ -987,7 +1213,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
             int c = 0;
             if (i < cnt) {
                 x = S.acc[i];
-                c = c0 + (int)S.colbuf[i];
+                c = m0 + (int)S.colbuf[i];
             }
             unsigned long long xb = mag_bits(x);
             bool nz = i < cnt && xb != 0ull;
@@ -1039,12 +1265,12 @@ __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W
     const int nadd = P.nadd;
     for (int t = threadIdx.x; t < nadd; t += blockDim.x) add[t] = P.add[t];
     __shared__ unsigned long long blk_written, blk_cand, blk_absmax, blk_fma, blk_arena;
-    __shared__ int blk_span;
+    __shared__ int blk_span, blk_words;
     if (threadIdx.x == 0) {
         // the block's warps take their first pool arenas with one atomic: at
         // the launch every warp wants one at once, on the same counter
         blk_arena = atomicAdd(&P.ctl->pool_used, (unsigned long long)kWarps * P.arena);
-        blk_span = 0;
+        blk_span = blk_words = 0;
         blk_fma = 0ull;
         blk_written = 0ull;
         blk_cand = 0ull;
@@ -1079,12 +1305,14 @@ __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W
         atomicAdd(&blk_cand, st.cand);
         atomicMax(&blk_absmax, st.absmax);
         atomicMax(&blk_span, st.span);
+        atomicMax(&blk_words, st.words);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         if (blk_fma) atomicAdd(&P.ctl->fma_total, blk_fma);
         if (P.stat) {
             if (blk_span > 0) atomicMax(&P.stat->span_max, (unsigned)blk_span);
+            if (blk_words > 0) atomicMax(&P.stat->words_max, (unsigned)blk_words);
             if (blk_fma) atomicAdd(&P.stat->fma, blk_fma);
             if (blk_written) atomicAdd(&P.stat->nnz_pre, blk_written);
             if (blk_cand) atomicAdd(&P.stat->ncand, blk_cand);
@@ -3247,6 +3475,54 @@ __global__ void k_row_bitmaps(int n, RowView B, int2* hdr, unsigned* bits) {
     }
 }
 
+// ---------------------------------------------------------------- k_row_lists
+// The words of every row of B that hold entries, as {column / 32, bitmap} at
+// the row's own positions of `lists`, columns ascending; hdr[r].y = how many
+// (never more than the row's entries).  One warp per row; a 32-entry piece's
+// last run of columns may go on in the next piece and is carried over.
+__global__ void k_row_lists(int n, RowView B, int2* hdr, uint2* lists) {
+    const int lane = threadIdx.x & 31;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
+        const int s = B.rb[r], e = B.re[r];
+        int m = 0;               // words written
+        int cw = -1;             // the carried run's word
+        unsigned cb = 0u;        // and bits
+        for (int q0 = s; q0 < e; q0 += 32) {
+            const int q = q0 + lane;
+            const bool in = q < e;
+            const int c = in ? B.col[q] : 0;
+            const int w = in ? c >> 5 : -2 - lane;
+            unsigned v = in ? 1u << (c & 31) : 0u;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned v2 = __shfl_down_sync(kFull, v, d);
+                const int w2 = __shfl_down_sync(kFull, w, d);
+                if (lane + d < 32 && w2 == w) v |= v2;
+            }
+            const int wp = __shfl_up_sync(kFull, w, 1);
+            const unsigned lead = __ballot_sync(kFull, in && (lane == 0 || wp != w));
+            const bool joins = __shfl_sync(kFull, w, 0) == cw;  // the first run continues the carried one
+            if (joins) {
+                if (lane == 0) v |= cb;
+            } else if (cw >= 0) {
+                if (lane == 0) lists[s + m] = make_uint2((unsigned)cw, cb);
+                ++m;
+            }
+            const int ll = 31 - __clz(lead);  // the last run's first lane: carried
+            if ((lead >> lane & 1u) && lane != ll)
+                lists[s + m + __popc(lead & lanemask_lt())] = make_uint2((unsigned)w, v);
+            m += __popc(lead) - 1;
+            cw = __shfl_sync(kFull, w, ll);
+            cb = __shfl_sync(kFull, v, ll);
+        }
+        if (lane == 0) {
+            if (cw >= 0) lists[s + m] = make_uint2((unsigned)cw, cb);
+            hdr[r] = make_int2(0, cw >= 0 ? m + 1 : 0);
+        }
+    }
+}
+
 // ---------------------------------------------------------------- plumbing
 // An empty pool of `cap` entries and empty candidate lists (the barrier's and
 // the counters' fields from bar_count on keep their values).
@@ -3283,12 +3559,13 @@ __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot
 __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, const double* val,
                            Ctl* ctl) {
     int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r > n) return;
     bool bad = false;
-    if (r == 0 && rowptr[0] != 0) bad = true;
-    if (r == n) {
-        if (rowptr[n] != nnz) bad = true;
+    int bw = 0;
+    if (r > n) {
+    } else if (r == n) {
+        if (rowptr[n] != nnz || (n == 0 && rowptr[0] != 0)) bad = true;
     } else {
+        if (r == 0 && rowptr[0] != 0) bad = true;
         int s = rowptr[r], e = rowptr[r + 1];
         if (s > e || s < 0 || e > nnz) {
             bad = true;
@@ -3305,9 +3582,12 @@ __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, co
                 prev = c;
             }
             if (e > s && prev - col[s] != e - s - 1) ctl->not_band = 1;
+            if (e > s && !bad) bw = max(prev - r, r - col[s]);
         }
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
+    bw = warp_max(bw);
+    if ((threadIdx.x & 31) == 0 && bw > 0) atomicMax(&ctl->bandwidth, (unsigned)bw);
 }
 
 // Exclusive scan of row lengths (re - rb, or a pooled matrix's true entries
@@ -3670,15 +3950,17 @@ cudaError_t kernels_init() {
     int sms = 0;
     err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
-    const void* prods[7] = {(const void*)k_product<true, false, false>, (const void*)k_product<false, false, false>,
+    const void* prods[8] = {(const void*)k_product<false, false, true, kListWords>,
+                            (const void*)k_product<true, false, false>, (const void*)k_product<false, false, false>,
                             (const void*)k_product<true, true, false>, (const void*)k_product<false, true, false>,
                             (const void*)k_product<false, false, true>,
                             (const void*)k_product<false, false, true, kBmWordsBig>,
                             (const void*)k_product<false, true, false, kBmWordsBig>};
-    const int psmem[7] = {(int)prod_smem_bytes<true>(), (int)prod_smem_bytes<false>(), (int)prod_smem_bytes<true>(),
+    const int psmem[8] = {(int)prod_smem_bytes<false, kListWords>(),
+                          (int)prod_smem_bytes<true>(), (int)prod_smem_bytes<false>(), (int)prod_smem_bytes<true>(),
                           (int)prod_smem_bytes<false>(), (int)prod_smem_bytes<false>(),
                           (int)prod_smem_bytes<false, kBmWordsBig>(), (int)prod_smem_bytes<false, kBmWordsBig>()};
-    for (int i = 0; i < 7; ++i) {
+    for (int i = 0; i < 8; ++i) {
         err = cudaFuncSetAttribute(prods[i], cudaFuncAttributeMaxDynamicSharedMemorySize, psmem[i]);
         if (err != cudaSuccess) return err;
     }
@@ -3748,6 +4030,7 @@ cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, do
         return wide_window ? prod_launch<false, true, false, kBmWordsBig>(P, st) : prod_launch<false, true, false>(P, st);
     }
     if (table) return prod_launch<true, false, false>(P, st);
+    if (P.blists) return prod_launch<false, false, true, kListWords>(P, st);
     // rows expected to span more columns than the bitmap covers: the wide
     // window (with every accumulator slot, as WIDE)
     if (wide_window) return prod_launch<false, false, true, kBmWordsBig>(P, st);
@@ -3791,6 +4074,16 @@ cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
         if (rounds >= (row_len <= 32.0 ? 0.35 : 3.0) || (rounds <= 1.0 && rounds >= 0.45)) band_launch<false, false, 4>(P, st);
         else band_launch<false, false, 1>(P, st);
     }
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_row_lists(int n, const RowView& B, int2* hdr, uint2* lists, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    long long blocks = ((long long)n + 7) / 8;
+    const long long cap = (long long)sms_now() * 8;
+    if (blocks > cap) blocks = cap;
+    k_row_lists<<<(unsigned)blocks, 256, 0, st>>>(n, B, hdr, lists);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -38,6 +38,11 @@ cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bit
 // an empty pool (the control block before bar_count)
 cudaError_t launch_reset(Ctl* ctl, unsigned long long cap, unsigned long long cand_cap, unsigned cand_chunk,
                          cudaStream_t st);
+// the same as lists of words (ProductArgs::bhdr, blists) for the list map, the
+// wide window's form for rows with entries in at most kListMapWords words of
+// 32 columns; lists: a pair per entry of B's index space
+constexpr int kListMapWords = 160;
+cudaError_t launch_row_lists(int n, const RowView& B, int2* hdr, uint2* lists, cudaStream_t st);
 // bytes (a multiple of 4) of device memory at src to dst, the device address
 // of pinned, mapped host memory, by a kernel on st (k_export)
 cudaError_t launch_export(const void* src, void* dst, size_t bytes, cudaStream_t st);
