@@ -299,6 +299,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                         CU(cudaEventRecord(t0, st));
                     }
                     P.band = table ? nullptr : d_band;
+                    P.pair = P.band && any_general;
                     if (any_general || table) CU(launch_product(P, table, st, 0.0, wz));
                     if (P.band) CU(launch_band(P, 0.0, st));
                     if (g_tune_rec) {
@@ -672,11 +673,9 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 P.bbits = w.pool_bits.as<unsigned>();
             }
             P.band = table ? nullptr : d_band;
+            P.pair = P.band && any_general;
             if (any_general || table) CU(launch_product(P, table, st, 0.0, T.wide));
-            if (P.band) {
-                if (any_general || table) P.start_out = nullptr;  // (known)
-                CU(launch_band(P, 0.0, st));
-            }
+            if (P.band) CU(launch_band(P, 0.0, st));
             if (g_tune_rec) {
                 CU(cudaEventRecord(e1, st));
                 g_tune_rec->work.push_back(fma_row);

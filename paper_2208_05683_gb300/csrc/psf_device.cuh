@@ -190,6 +190,10 @@ struct ProductArgs {
     const uint2* blists;
     // batch: instances whose rows k_band computes (nullptr: none)
     const unsigned char* band;
+    // batch: k_product and k_band share the step.  k_band starts as k_product's
+    // blocks leave their SMs and waits for its end in its own last lines, and
+    // only k_band ends the step (step_done)
+    int pair;
     // written by the launch's last block (step_done)
     int mark;                        // > 0: ctl->mark[mark] <- the pool counter
     unsigned long long* start_out;   // batch: the pool counter before the step

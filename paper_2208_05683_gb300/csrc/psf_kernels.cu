@@ -1253,6 +1253,8 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
 template <bool TAB, bool BATCH, bool WIDE, int W = kBmWords>
 __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W>::kBlocksPerSm)
     k_product(const __grid_constant__ ProductArgs P) {
+    if constexpr (BATCH)
+        if (P.pair) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // a baby step whose product equals an already computed power (no entry
     // dropped so far) is done by k_reuse_pass1 instead (same value in all blocks)
     if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
@@ -1293,8 +1295,11 @@ __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W
     // unused end of its candidate chunk as holes
     arena_close(st.arena, P.pool_val, lane);
     if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
+    if constexpr (BATCH) {
+        if (!P.pair) product_done(P);
+        return;
+    }
     product_done(P);
-    if constexpr (BATCH) return;
     // ---- block totals for the step statistics
     st.cand = (unsigned long long)warp_sum((int)st.cand);
     st.absmax = warp_max_u64(st.absmax);
@@ -2422,6 +2427,8 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
     }
     if (lead) arena_close(st.arena, P.pool_val, lane);
     if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
+    if constexpr (BATCH)
+        if (P.pair) asm volatile("griddepcontrol.wait;" ::: "memory");
     product_done(P);
     if constexpr (BATCH) return;
     // ---- the step statistics, once per block
@@ -3967,7 +3974,8 @@ cudaError_t kernels_init() {
     err = cudaFuncSetAttribute((const void*)k_product_cta, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)cta_smem_bytes());
     if (err != cudaSuccess) return err;
-    const void* bands[10] = {
+    const void* bands[12] = {
+        (const void*)k_band<true, false, 1, false>,  (const void*)k_band<true, false, 1, true>,
         (const void*)k_band<false, false, 1, false>, (const void*)k_band<false, false, 4, false>,
         (const void*)k_band<false, true, 1, false>,  (const void*)k_band<false, true, 4, false>,
         (const void*)k_band<true, false, 4, false>,  (const void*)k_band<false, false, 1, true>,
@@ -4039,15 +4047,33 @@ cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, do
     return prod_launch<false, false, false>(P, st);
 }
 
+// In a batch with instances of both kinds the step is two launches, k_product
+// and k_band, neither of which reads what the other writes.  k_band is
+// launched programmatically: its blocks take the SMs that k_product's leave
+// (each kernel's warps end at different times, a quarter of them idle on
+// average), and it waits for k_product's end before it ends the step itself.
+// 128 instances of 64-4096 rows: 17.6 -> 17.1 ms a call, 27: 5.9 -> 5.3 ms.
+// (One launch that hands rows of both kinds to the same warps or SMs was
+// slower, 19.4-23.3 ms: the two codes together outgrow an SM's instruction
+// cache.)
 template <bool BATCH, bool TEAM, int R>
-static void band_launch(const ProductArgs& P, cudaStream_t st) {
+static cudaError_t band_launch(const ProductArgs& P, cudaStream_t st) {
     const long long cap = (long long)sms_now() * 7, tiles = ((long long)P.n + R - 1) / R;
     const long long blocks = TEAM ? tiles : (tiles + kBandWarps - 1) / kBandWarps;
-    const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)(blocks < cap ? blocks : cap));
+    c.blockDim = dim3(kBandWarps * 32);
+    c.dynamicSmemBytes = band_smem_bytes();
+    c.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = P.pair ? 1 : 0;
+    ++g_launches;
     // (a batch's rows may be filtered when candidate lists are given)
-    const bool filt = P.cand_col != nullptr;
-    if (filt) k_band<BATCH, TEAM, R, true><<<grid, kBandWarps * 32, band_smem_bytes(), st>>>(P);
-    else k_band<BATCH, TEAM, R, false><<<grid, kBandWarps * 32, band_smem_bytes(), st>>>(P);
+    return P.cand_col ? cudaLaunchKernelEx(&c, k_band<BATCH, TEAM, R, true>, P)
+                      : cudaLaunchKernelEx(&c, k_band<BATCH, TEAM, R, false>, P);
 }
 
 cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
@@ -4060,22 +4086,18 @@ cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
     // of the chip's warps or several (one row / four: n = 2000, 31 x 61 36 /
     // 57; n = 12000 91 / 83; n = 20000, 1.2 rounds, 140 / 169; n = 65536
     // 408 / 375), and for rows of one 32-column piece, which are mostly
-    // set-up (11 x 11: n = 12000 36 / 29, n = 65536 117 / 83).
+    // set-up (11 x 11: n = 12000 36 / 29, n = 65536 117 / 83).  A batch: one
+    // row below one round (a call of 4 instances, 2000 rows at most: 2.22 ms
+    // with four, 1.61 with one); its rows' lengths differ too much for more.
     const double warps = sms_now() * 7.0 * kBandWarps;
     const double rounds = P.n / (4.0 * warps);  // of tiles of four rows
     const bool team = row_len > 300.0 || (row_len > 128.0 && P.n <= 5.0 * warps / kBandWarps) ||
                       (row_len > 80.0 && P.n <= 2.0 * warps / kBandWarps);
-    if (P.inst) {
-        band_launch<true, false, 4>(P, st);
-    } else if (team) {
-        if (rounds >= 0.9) band_launch<false, true, 4>(P, st);
-        else band_launch<false, true, 1>(P, st);
-    } else {
-        if (rounds >= (row_len <= 32.0 ? 0.35 : 3.0) || (rounds <= 1.0 && rounds >= 0.45)) band_launch<false, false, 4>(P, st);
-        else band_launch<false, false, 1>(P, st);
-    }
-    ++g_launches;
-    return cudaGetLastError();
+    if (P.inst) return rounds >= 1.0 ? band_launch<true, false, 4>(P, st) : band_launch<true, false, 1>(P, st);
+    if (team) return rounds >= 0.9 ? band_launch<false, true, 4>(P, st) : band_launch<false, true, 1>(P, st);
+    if (rounds >= (row_len <= 32.0 ? 0.35 : 3.0) || (rounds <= 1.0 && rounds >= 0.45))
+        return band_launch<false, false, 4>(P, st);
+    return band_launch<false, false, 1>(P, st);
 }
 
 cudaError_t launch_row_lists(int n, const RowView& B, int2* hdr, uint2* lists, cudaStream_t st) {
