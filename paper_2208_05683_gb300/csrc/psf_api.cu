@@ -1334,6 +1334,24 @@ int psf_result_csr(psf_result_t r, psf_csr_t* view) {
 int psf_result_copy(psf_result_t r, int32_t* rowptr, int32_t* col, double* val, void* stream) {
     if (!r) return fail(PSF_EINVAL, "null result");
     cudaStream_t st = (cudaStream_t)stream;
+    // into arrays of the current device (the result's too): one kernel
+    int dev = 0;
+    CU(cudaGetDevice(&dev));
+    auto here = [dev](const void* p) {
+        if (!p) return true;
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return at.type == cudaMemoryTypeDevice && at.device == dev && ((uintptr_t)p & 3) == 0;
+    };
+    if (here(r->rowptr) && here(rowptr) && here(col) && here(val)) {
+        int rc = prepare(st);
+        if (rc) return rc;
+        CU(launch_copy_result(r->n, r->nnz, r->rowptr, r->col, r->val, rowptr, col, val, st));
+        return PSF_OK;
+    }
     // cudaMemcpyDefault: the destination may be device or host memory
     if (rowptr) CU(cudaMemcpyAsync(rowptr, r->rowptr, sizeof(int) * ((size_t)r->n + 1), cudaMemcpyDefault, st));
     if (col && r->nnz) CU(cudaMemcpyAsync(col, r->col, sizeof(int) * (size_t)r->nnz, cudaMemcpyDefault, st));

@@ -27,6 +27,7 @@
 //                 allocation-free variant).
 //  k_export       small device records written into pinned, device-mapped
 //                 host memory (the host's read-backs take no copy engine).
+//  k_copy_result  a result's arrays into the caller's.
 //  k_absmax, k_validate*, k_copy_rows*, k_scan_*, k_gather*, k_identity,
 //  k_inst_table, k_compose_rows, k_bounds: plumbing.
 #include <atomic>
@@ -3482,6 +3483,58 @@ __global__ void k_row_bitmaps(int n, RowView B, int2* hdr, unsigned* bits) {
     }
 }
 
+// ---------------------------------------------------------------- k_copy_result
+// A result's arrays into the caller's, in one launch instead of three copies:
+// each copy cost about 5 us of the host's time and 2 us on the stream, more
+// than the bytes of a small result (a batch of 128 hands over 384 arrays).
+// 16 bytes a thread and access, four in flight, where source and destination
+// are aligned alike; the arrays of a batch's results start anywhere and go by
+// words.
+// A batch call of 128 instances 17.05 -> 16.25 ms, one banded product
+// (n = 30001, 4 MB of result) 281 -> 259 us.
+struct CopyArgs {
+    const unsigned* src[3];
+    unsigned* dst[3];
+    long long words[3];
+};
+__global__ void __launch_bounds__(256) k_copy_result(const __grid_constant__ CopyArgs C) {
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        const unsigned* __restrict__ s = C.src[a];
+        unsigned* __restrict__ d = C.dst[a];
+        const long long n = C.words[a];
+        const long long head = ((16 - ((unsigned long long)d & 15)) & 15) >> 2;
+        if ((((unsigned long long)s ^ (unsigned long long)d) & 15) == 0 && n > head) {
+            const long long q = (n - head) >> 2;  // 16-byte pieces
+            const uint4* __restrict__ s4 = reinterpret_cast<const uint4*>(s + head);
+            uint4* __restrict__ d4 = reinterpret_cast<uint4*>(d + head);
+            long long i = t0;
+            for (; i + 3 * step < q; i += 4 * step) {
+                const uint4 x0 = s4[i], x1 = s4[i + step], x2 = s4[i + 2 * step], x3 = s4[i + 3 * step];
+                d4[i] = x0;
+                d4[i + step] = x1;
+                d4[i + 2 * step] = x2;
+                d4[i + 3 * step] = x3;
+            }
+            for (; i < q; i += step) d4[i] = s4[i];
+            if (t0 < head) d[t0] = s[t0];
+            const long long tail = head + 4 * q + t0;
+            if (tail < n) d[tail] = s[tail];
+        } else {
+            long long i = t0;
+            for (; i + 3 * step < n; i += 4 * step) {
+                const unsigned x0 = s[i], x1 = s[i + step], x2 = s[i + 2 * step], x3 = s[i + 3 * step];
+                d[i] = x0;
+                d[i + step] = x1;
+                d[i + 2 * step] = x2;
+                d[i + 3 * step] = x3;
+            }
+            for (; i < n; i += step) d[i] = s[i];
+        }
+    }
+}
+
 // ---------------------------------------------------------------- k_row_lists
 // The words of every row of B that hold entries, as {column / 32, bitmap} at
 // the row's own positions of `lists`, columns ascending; hdr[r].y = how many
@@ -4098,6 +4151,28 @@ cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
     if (rounds >= (row_len <= 32.0 ? 0.35 : 3.0) || (rounds <= 1.0 && rounds >= 0.45))
         return band_launch<false, false, 4>(P, st);
     return band_launch<false, false, 1>(P, st);
+}
+
+cudaError_t launch_copy_result(int n, long long nnz, const int* rowptr, const int* col, const double* val,
+                               int* d_rowptr, int* d_col, double* d_val, cudaStream_t st) {
+    CopyArgs C{};
+    const void* src[3] = {rowptr, col, val};
+    void* dst[3] = {d_rowptr, d_col, d_val};
+    const long long words[3] = {(long long)n + 1, nnz, 2 * nnz};
+    long long most = 0;
+    for (int a = 0; a < 3; ++a) {
+        C.src[a] = static_cast<const unsigned*>(src[a]);
+        C.dst[a] = static_cast<unsigned*>(dst[a]);
+        C.words[a] = dst[a] ? words[a] : 0;
+        most = most > C.words[a] ? most : C.words[a];
+    }
+    if (most == 0) return cudaSuccess;
+    long long blocks = (most + 1023) / 1024;
+    const long long cap = (long long)sms_now() * 8;
+    if (blocks > cap) blocks = cap;
+    k_copy_result<<<(unsigned)blocks, 256, 0, st>>>(C);
+    ++g_launches;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_row_lists(int n, const RowView& B, int2* hdr, uint2* lists, cudaStream_t st) {

@@ -43,6 +43,11 @@ cudaError_t launch_reset(Ctl* ctl, unsigned long long cap, unsigned long long ca
 // 32 columns; lists: a pair per entry of B's index space
 constexpr int kListMapWords = 160;
 cudaError_t launch_row_lists(int n, const RowView& B, int2* hdr, uint2* lists, cudaStream_t st);
+// a result's three arrays (n + 1 ints, nnz ints, nnz doubles; a null
+// destination is skipped) by one kernel; all pointers are 4-byte aligned
+// memory of the current device
+cudaError_t launch_copy_result(int n, long long nnz, const int* rowptr, const int* col, const double* val,
+                               int* d_rowptr, int* d_col, double* d_val, cudaStream_t st);
 // bytes (a multiple of 4) of device memory at src to dst, the device address
 // of pinned, mapped host memory, by a kernel on st (k_export)
 cudaError_t launch_export(const void* src, void* dst, size_t bytes, cudaStream_t st);
