@@ -344,7 +344,8 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         a.cand_col = P.cand_col;
         a.cand_x = P.cand_x;
         a.far_shift = g_far_shift.load(std::memory_order_relaxed);
-        CU(launch_alg1(a, w.st));
+        const double len = out_len > 0.0 ? out_len : alen > 0.0 ? alen + blen : (double)add.size() * w.n;
+        CU(launch_alg1(a, len * w.n, w.st));
     }
     *out = w.pooled(R);
     return PSF_OK;

@@ -46,7 +46,7 @@ struct Ctl {
     int dropped;          // set once Algorithm 1 has dropped an entry (baby steps reuse powers until then)
     int pad1;
     unsigned bar_count;  // fields from here on survive a pool reset
-    unsigned bar_gen;
+    unsigned pad4;
     unsigned bandwidth;  // of the checked inputs: max |column - row|
     int not_band;  // an input has a row that does not span consecutive columns
     unsigned done;    // blocks of the running launch that have finished (0 between launches)
@@ -712,34 +712,38 @@ __device__ __forceinline__ unsigned long long far_split(double eps_g, int shift)
 // Grid-wide barrier for cooperative launches, with a bounded wait: after
 // `budget_ns` it records kDevTimeout and returns false (a budget of 0 gives
 // up at once unless the barrier is already complete: a test of that path).
+// One atomic per block: the first block adds 2^31 less the others' ones, so
+// the counter's top bit flips when all have arrived and its low bits come
+// back to where they were, whatever the next launch's grid; the waiting
+// blocks poll that bit.
 __device__ __forceinline__ bool grid_barrier(Ctl* ctl, unsigned long long budget_ns) {
     __syncthreads();
     __shared__ int ok;
     if (threadIdx.x == 0) {
         ok = 1;
-        volatile unsigned* gen = &ctl->bar_gen;
-        unsigned g = *gen;
         __threadfence();
-        unsigned arrived = atomicAdd(&ctl->bar_count, 1u);
-        if (arrived == gridDim.x - 1) {
-            atomicExch(&ctl->bar_count, 0u);
-            __threadfence();
-            atomicAdd(&ctl->bar_gen, 1u);
-        } else {
-            unsigned long long t0 = global_ns();
-            while (*gen == g) {
+        const unsigned old = atomicAdd(&ctl->bar_count, blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1) : 1u);
+        const volatile unsigned* const now = &ctl->bar_count;
+        if (((old ^ *now) >> 31) == 0u) {
+            const unsigned long long t0 = global_ns();
+            while (((old ^ *now) >> 31) == 0u) {
                 if (budget_ns == 0ull || global_ns() - t0 > budget_ns) {
                     atomicOr(&ctl->status, kDevTimeout);
                     ok = 0;
                     break;
                 }
-                __nanosleep(64);
             }
         }
         __threadfence();
     }
     __syncthreads();
     return ok != 0;
+}
+
+// The same for a launch of one cluster: the hardware's barrier, which orders
+// global memory among the cluster's blocks.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 }  // namespace psf

@@ -2604,10 +2604,33 @@ __global__ void __launch_bounds__(256) k_reuse_copy_batch(ProductArgs P) {
 // launch.  On entry the column sums of pass 1 (entries |x| <= eps_g) are in
 // the chunk words and both cslot words are 0.  Every block evaluates the same
 // scalar recurrence from the same global values, so all blocks take the same
-// decisions without further communication.
+// decisions without further communication.  Bound by the latency of a pass
+// (finalize: eight words a column; the list; a barrier after each), not by
+// bytes or instructions, up to a few hundred thousand candidates: with the
+// barrier's one atomic per block (it was two, and sleeps between polls)
+// cos of banded N(0, 1), n = 1000, w = 8, took 1153 us before and 1048 after.
 constexpr int kAlg1Threads = 1024;  // one block per SM: few grid-barrier arrivals
 constexpr int kAlg1BlocksPerSm = 1;
+// Small steps run as one cluster of 16 blocks: the passes of a step are two
+// barriers each, and the cluster's cost less than the grid's, which is most
+// of the time while the candidates are few.  Measured as whole evaluations
+// (us, grid / cluster): 1D n = 256 445 / 430, n = 2000 (50 k entries a step)
+// 520 / 505, 16 x 16 grid (51 k) 910 / 853, banded n = 1000 (74 k) 675 / 655;
+// n = 2000 (148 k) 744 / 769, 32 x 32 grid (318 k) 996 / 995, 48 x 48 (808 k)
+// 1188 / 1279: the line lies at 100 k entries.
+constexpr int kClusterColumns = 4096;
+constexpr double kClusterEntries = 1e5;
 
+template <bool CLUSTER>
+__device__ __forceinline__ bool alg1_barrier(const Alg1Args& A) {
+    if constexpr (CLUSTER) {
+        cluster_barrier();
+        return true;
+    }
+    return grid_barrier(A.ctl, A.budget_ns);
+}
+
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Args A) {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2668,7 +2691,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
                 }
             }
         }
-        if (!grid_barrier(A.ctl, A.budget_ns)) {
+        if (!alg1_barrier<CLUSTER>(A)) {
             alive = false;
             break;
         }
@@ -2760,7 +2783,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
                     }
                 }
             }
-            if (!grid_barrier(A.ctl, A.budget_ns)) {
+            if (!alg1_barrier<CLUSTER>(A)) {
                 alive = false;
                 break;
             }
@@ -2786,7 +2809,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
                 }
             }
         }
-        if (!grid_barrier(A.ctl, A.budget_ns)) {
+        if (!alg1_barrier<CLUSTER>(A)) {
             alive = false;
             break;
         }
@@ -2805,7 +2828,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
         // once all blocks reach the first barrier.
         const unsigned long long fb = (unsigned long long)__double_as_longlong(eps_f);
         const int sx = it & 1, sc = (it - 1) & 1;
-        if (!grid_barrier(A.ctl, A.budget_ns)) return;
+        if (!alg1_barrier<CLUSTER>(A)) return;
         if (gt == 0) A.ctl->cslot[sc] = 0ull;
         unsigned long long mx = 0ull;
         for (unsigned long long q = p0 + (unsigned long long)gt; q < p1; q += (unsigned long long)nthreads) {
@@ -2814,13 +2837,13 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
         }
         mx = warp_max_u64(mx);
         if (lane == 0 && mx) atomicMax(&A.ctl->cslot[sx], mx);
-        if (!grid_barrier(A.ctl, A.budget_ns)) return;
+        if (!alg1_barrier<CLUSTER>(A)) return;
         const int lsb = lsb_for_bound(__ldcg(&A.ctl->cslot[sx]));
         for (unsigned long long q = p0 + (unsigned long long)gt; q < p1; q += (unsigned long long)nthreads) {
             const unsigned long long xb = mag_bits(__ldcg(A.val + q));
             if (xb != 0ull && xb <= fb) exact_add_checked(A.words, A.sticky, A.col[q], A.n, xb, lsb, A.ctl);
         }
-        if (!grid_barrier(A.ctl, A.budget_ns)) return;
+        if (!alg1_barrier<CLUSTER>(A)) return;
         unsigned long long local = 0ull;
         for (int j = gt; j < A.n; j += nthreads) {
             const double s = chunk_round(A.words + j, n, A.sticky + j, lsb, true);
@@ -2829,7 +2852,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
         }
         local = warp_max_u64(local);
         if (lane == 0 && local) atomicMax(&A.ctl->cslot[sc], local);
-        if (!grid_barrier(A.ctl, A.budget_ns)) return;
+        if (!alg1_barrier<CLUSTER>(A)) return;
         c = __longlong_as_double((long long)__ldcg(&A.ctl->cslot[sc]));
     }
     if (!(c > 0.0)) {
@@ -3975,7 +3998,7 @@ __global__ void k_identity(int n, double alpha, int* rowptr, int* col, double* v
 // Launch configuration, per device (set up once by kernels_init, guarded by
 // a mutex; a device's entry is published through `ready`).
 struct DevCfg {
-    int sms = 0, alg1_blocks = 0, alg1b_blocks = 0, norm_blocks = 0;
+    int sms = 0, alg1_blocks = 0, alg1_cluster = 0, alg1b_blocks = 0, norm_blocks = 0;
     std::atomic<bool> ready{false};
 };
 constexpr int kMaxDevices = 64;
@@ -4042,9 +4065,27 @@ cudaError_t kernels_init() {
                                (int)norms_rows_smem_bytes());
     if (err != cudaSuccess) return err;
     int per = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_alg1, kAlg1Threads, 0);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_alg1<false>, kAlg1Threads, 0);
     if (err != cudaSuccess) return err;
     c.alg1_blocks = sms * (per < kAlg1BlocksPerSm ? per : kAlg1BlocksPerSm);
+    // one cluster of 16 blocks where the device takes it (8 is what every
+    // device does)
+    c.alg1_cluster = 8;
+    if (cudaFuncSetAttribute((const void*)k_alg1<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaLaunchConfig_t q{};
+        q.gridDim = dim3(16);
+        q.blockDim = dim3(kAlg1Threads);
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 16;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        q.attrs = &at;
+        q.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_alg1<true>, &q) == cudaSuccess && clusters > 0)
+            c.alg1_cluster = 16;
+    }
+    cudaGetLastError();
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_alg1_batch, kAlg1Threads, 0);
     if (err != cudaSuccess) return err;
     c.alg1b_blocks = sms * (per < 4 ? per : 4);
@@ -4195,12 +4236,25 @@ cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bit
     return cudaGetLastError();
 }
 
-cudaError_t launch_alg1(const Alg1Args& A, cudaStream_t st) {
+cudaError_t launch_alg1(const Alg1Args& A, double entries, cudaStream_t st) {
     Alg1Args a = A;  // (cslot is 0: step_done)
     a.budget_ns = barrier_budget_ns();
-    void* args[] = {&a};
     ++g_launches;
-    return cudaLaunchCooperativeKernel((const void*)k_alg1, dim3(dcfg().alg1_blocks), dim3(kAlg1Threads), args,
+    if (dcfg().alg1_cluster > 0 && a.budget_ns > 0 && A.n <= kClusterColumns && entries <= kClusterEntries) {
+        cudaLaunchConfig_t c{};
+        c.gridDim = dim3((unsigned)dcfg().alg1_cluster);
+        c.blockDim = dim3(kAlg1Threads);
+        c.stream = st;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = c.gridDim.x;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        c.attrs = &at;
+        c.numAttrs = 1;
+        return cudaLaunchKernelEx(&c, k_alg1<true>, a);
+    }
+    void* args[] = {&a};
+    return cudaLaunchCooperativeKernel((const void*)k_alg1<false>, dim3(dcfg().alg1_blocks), dim3(kAlg1Threads), args,
                                        0, st);
 }
 

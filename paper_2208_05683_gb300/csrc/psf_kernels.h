@@ -51,7 +51,8 @@ cudaError_t launch_copy_result(int n, long long nnz, const int* rowptr, const in
 // bytes (a multiple of 4) of device memory at src to dst, the device address
 // of pinned, mapped host memory, by a kernel on st (k_export)
 cudaError_t launch_export(const void* src, void* dst, size_t bytes, cudaStream_t st);
-cudaError_t launch_alg1(const Alg1Args& A, cudaStream_t st);
+// entries: about how many the step's rows hold
+cudaError_t launch_alg1(const Alg1Args& A, double entries, cudaStream_t st);
 cudaError_t launch_norms(const NormArgs& A, cudaStream_t st);
 cudaError_t launch_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot* slot, cudaStream_t st);
 cudaError_t launch_validate(int n, int nnz, const int* rowptr, const int* col, const double* val, Ctl* ctl,
