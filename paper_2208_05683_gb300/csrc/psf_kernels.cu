@@ -33,11 +33,45 @@
 #include <atomic>
 #include <climits>
 #include <mutex>
+#include <utility>
 
 #include "psf_device.cuh"
 #include "psf_kernels.h"
 
 namespace psf {
+
+// Programmatic launches.  The kernels of a call follow one another on a stream,
+// and most of a small call is the time between them: a kernel's blocks are
+// scheduled only when the last one has drained.  Launched programmatically
+// (launch_pdl) a kernel is brought onto the SMs while the one before it runs;
+// it starts by waiting for that one's end (all of its blocks, and what they
+// wrote) and then lets the next one come.  Every kernel here does so first of
+// all, so that whatever ran two launches earlier has ended too.  A launch
+// that is no such kernel's neighbour behaves as an ordinary one.
+// Measured on whole calls (us, ordinary / programmatic): norm1 of a 37 x 29 grid
+// 46.5 / 38.3, one banded product of 30001 rows 259 / 246, exp of the 1D
+// Laplacian, n = 256, 511 / 430, cos of banded N(0, 1), n = 1000, 1084 / 1014,
+// banded n = 65536 3843 / 3778.
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter() {
+    pdl_wait();
+    pdl_release();
+}
+template <class... Params, class... Args>
+static cudaError_t launch_pdl(void (*k)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, std::forward<Args>(args)...);
+}
 
 // ---------------------------------------------------------------- k_product
 // Compact-accumulator kernel: one warp computes one output row, with no
@@ -1254,8 +1288,7 @@ __device__ __forceinline__ void product_row(const ProductArgs& P, const AddTerm*
 template <bool TAB, bool BATCH, bool WIDE, int W = kBmWords>
 __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W>::kBlocksPerSm)
     k_product(const __grid_constant__ ProductArgs P) {
-    if constexpr (BATCH)
-        if (P.pair) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_enter();
     // a baby step whose product equals an already computed power (no entry
     // dropped so far) is done by k_reuse_pass1 instead (same value in all blocks)
     if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
@@ -1818,6 +1851,7 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
 }
 
 __global__ void __launch_bounds__(kCtaWarps * 32, 7) k_product_cta(const __grid_constant__ ProductArgs P) {
+    pdl_enter();
     if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AddTerm* add = reinterpret_cast<AddTerm*>(smem_raw);
@@ -2026,6 +2060,9 @@ __device__ __forceinline__ void band_desc(const ProductArgs& P, int r, long long
 
 template <bool BATCH, bool TEAM, int R, bool FILT>
 __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_constant__ ProductArgs P) {
+    // (a batch's k_band works beside k_product and waits for it at its end)
+    if (BATCH && P.pair) pdl_release();
+    else pdl_enter();
     if (P.skip_unless && __ldcg(P.skip_unless) == 0) return;
     using Stage = BandStage<R, TEAM>;
     constexpr int N = Stage::N;
@@ -2429,7 +2466,7 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
     if (lead) arena_close(st.arena, P.pool_val, lane);
     if (P.cand_col) cand_close(st.carena, P.cand_x, lane);
     if constexpr (BATCH)
-        if (P.pair) asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (P.pair) pdl_wait();
     product_done(P);
     if constexpr (BATCH) return;
     // ---- the step statistics, once per block
@@ -2476,6 +2513,7 @@ size_t band_smem_bytes() { return sizeof(AddTerm) * kMaxAdd + sizeof(BandMap) * 
 // product kernel then runs instead).
 
 __global__ void __launch_bounds__(256) k_reuse_pass1(ReuseArgs R) {
+    pdl_enter();
     if (__ldcg(&R.ctl->dropped) != 0) return;
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -2539,6 +2577,7 @@ __global__ void __launch_bounds__(256) k_reuse_pass1(ReuseArgs R) {
 // product's multiply-add count (the B row lengths summed over row r of A).
 // The product kernel skips these rows.
 __global__ void __launch_bounds__(256) k_reuse_copy_batch(ProductArgs P) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -2632,6 +2671,7 @@ __device__ __forceinline__ bool alg1_barrier(const Alg1Args& A) {
 
 template <bool CLUSTER>
 __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Args A) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -2893,6 +2933,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1(Alg1Arg
 constexpr int kMaxBatch = 1024;  // instances of one batched launch
 
 __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1_batch(Alg1BatchArgs A) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -3207,6 +3248,7 @@ __global__ void __launch_bounds__(kAlg1Threads, kAlg1BlocksPerSm) k_alg1_batch(A
 constexpr int kNormThreads = 256;
 
 __global__ void __launch_bounds__(kNormThreads) k_norms(NormArgs A) {
+    pdl_enter();
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthreads = gridDim.x * blockDim.x;
     const size_t n = (size_t)A.n;
@@ -3310,6 +3352,7 @@ static_assert(kNormTile <= 255, "shared 24-bit pieces of a tile must not overflo
 size_t norms_rows_smem_bytes() { return sizeof(unsigned) * (size_t)(kNormPieces + 1) * kNormWin; }
 
 __global__ void __launch_bounds__(kNormRowsThreads) k_norms_rows(NormRowsArgs A) {
+    pdl_enter();
     extern __shared__ unsigned nsm[];  // [kNormPieces][kNormWin] pieces, then [kNormWin] sticky counts
     __shared__ int s_lo[kNormRowsThreads / 32], s_hi[kNormRowsThreads / 32];
     if (__ldcg(&A.ctl->status) & kDevPoolFull) return;  // discarded phase
@@ -3416,6 +3459,7 @@ __global__ void __launch_bounds__(kNormRowsThreads) k_norms_rows(NormRowsArgs A)
 
 __global__ void k_norms_finish(int n, int count, NormSlot* slots, unsigned long long* words, unsigned* sticky,
                                const Ctl* ctl, const int* inst, int slot_stride) {
+    pdl_enter();
     if (__ldcg(&ctl->status) & kDevPoolFull) return;
     // one thread per (matrix, column); the column count is padded to whole
     // warps so that a warp's columns belong to one matrix and it reduces
@@ -3461,6 +3505,7 @@ __global__ void k_norms_finish(int n, int count, NormSlot* slots, unsigned long 
 // queue behind a large device-to-host copy that another stream has in
 // flight (a result being copied out while the next evaluation runs).
 __global__ void k_export(const unsigned* src, unsigned* dst, int nwords) {
+    pdl_enter();
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) dst[i] = __ldcg(src + i);
 }
 
@@ -3472,6 +3517,7 @@ __global__ void k_export(const unsigned* src, unsigned* dst, int nwords) {
 // per row: each 32-entry piece ORs runs of lanes with the same word (the
 // columns ascend) and the first lane of a run adds it to the word.
 __global__ void k_row_bitmaps(int n, RowView B, int2* hdr, unsigned* bits) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
@@ -3521,6 +3567,7 @@ struct CopyArgs {
     long long words[3];
 };
 __global__ void __launch_bounds__(256) k_copy_result(const __grid_constant__ CopyArgs C) {
+    pdl_enter();
     const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
 #pragma unroll 1
     for (int a = 0; a < 3; ++a) {
@@ -3564,6 +3611,7 @@ __global__ void __launch_bounds__(256) k_copy_result(const __grid_constant__ Cop
 // (never more than the row's entries).  One warp per row; a 32-entry piece's
 // last run of columns may go on in the next piece and is carried over.
 __global__ void k_row_lists(int n, RowView B, int2* hdr, uint2* lists) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
@@ -3610,6 +3658,7 @@ __global__ void k_row_lists(int n, RowView B, int2* hdr, uint2* lists) {
 // An empty pool of `cap` entries and empty candidate lists (the barrier's and
 // the counters' fields from bar_count on keep their values).
 __global__ void k_reset(Ctl* ctl, unsigned long long cap, unsigned long long cand_cap, unsigned cand_chunk) {
+    pdl_enter();
     if (threadIdx.x) return;
     ctl->pool_used = ctl->pool_mark = 0ull;
     ctl->pool_cap = cap;
@@ -3624,6 +3673,7 @@ __global__ void k_reset(Ctl* ctl, unsigned long long cap, unsigned long long can
 
 // max |x| over the pool entries [mark[i], mark[i+1])
 __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot* slot) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const unsigned long long cap = ctl->pool_cap;  // counters may run past it on overflow
     const unsigned long long p0 = min(__ldcg(&ctl->mark[i]), cap), p1 = min(__ldcg(&ctl->mark[i + 1]), cap);
@@ -3641,6 +3691,7 @@ __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot
 // columns in range and strictly increasing per row, values finite.
 __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, const double* val,
                            Ctl* ctl) {
+    pdl_enter();
     int r = blockIdx.x * blockDim.x + threadIdx.x;
     bool bad = false;
     int bw = 0;
@@ -3708,6 +3759,7 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long* par
 // The tile sums; the last block to finish scans them.
 __global__ void __launch_bounds__(kScanTile) k_scan_tile_sums(int n, const int* rb, const int* re, const RowDesc* rd,
                                                               long long* sums, Ctl* ctl) {
+    pdl_enter();
     __shared__ long long part[32];
     __shared__ int last_block;
     const long long r = (long long)blockIdx.x * kScanTile + threadIdx.x;
@@ -3742,6 +3794,7 @@ __global__ void __launch_bounds__(kScanTile) k_scan_tile_sums(int n, const int* 
 
 __global__ void __launch_bounds__(kScanTile) k_scan_apply(int n, const int* rb, const int* re, const RowDesc* rd,
                                                            const long long* sums, int* rowptr) {
+    pdl_enter();
     __shared__ long long part[32];
     const long long r = (long long)blockIdx.x * kScanTile + threadIdx.x;
     const long long len = r < n ? (long long)(rd ? rd_nnz(rd[r]) : re[r] - rb[r]) : 0;
@@ -3778,6 +3831,7 @@ __device__ __forceinline__ void gather_row(const RowView& src, int r, long long 
 }
 
 __global__ void k_gather(int n, RowView src, const int* rowptr, int* col, double* val) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -3790,6 +3844,7 @@ __global__ void k_gather(int n, RowView src, const int* rowptr, int* col, double
 __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const double* val, int* rb, int* re,
                             RowDesc* rd, int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size,
                             NormSlot* absmax) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -3837,6 +3892,7 @@ __global__ void k_copy_rows(int n, const int* rowptr, const int* col, const doub
 // column-sum words, and let the matrix's entries [0, nnz) be norm matrix 0.
 __global__ void k_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long long* words, unsigned* sticky, int n,
                                     long long nnz) {
+    pdl_enter();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nt = (long long)gridDim.x * blockDim.x;
     for (long long i = t; i < (long long)kChunks * n; i += nt) words[i] = 0ull;
@@ -3856,6 +3912,7 @@ __global__ void k_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long long
 // ---- batches: the instance of every row (binary search over the row
 // offsets off[0..ninst], off[ninst] = n)
 __global__ void k_inst_table(int n, int ninst, const int* off, int* inst) {
+    pdl_enter();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     int lo = 0, hi = ninst - 1;  // largest i with off[i] <= r
@@ -3870,6 +3927,7 @@ __global__ void k_inst_table(int n, int ninst, const int* off, int* inst) {
 // Check every input of a batch like k_validate: thread per global row.
 __global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, const int* nnz, Ctl* ctl,
                                  unsigned char* band) {
+    pdl_enter();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int i = inst[r];
@@ -3903,6 +3961,7 @@ __global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, co
 __global__ void k_copy_rows_batch(int n, const int* inst, const BatchSrc* src, int* rb, int* re, RowDesc* rd,
                                   int* pool_col, double* pool_val, Ctl* ctl, unsigned long long arena_size, NormSlot* absmax,
                                   int stride) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -3949,6 +4008,7 @@ struct RowTable {
 };
 __global__ void k_compose_rows(int n, const int* inst, const int* sel, RowTable T, int* out_rb, int* out_re,
                                RowDesc* out_rd) {
+    pdl_enter();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const RowDesc d = T.rd[sel[inst[r]]][r];
@@ -3963,6 +4023,7 @@ __global__ void k_compose_rows(int n, const int* inst, const int* sel, RowTable 
 // columns.
 __global__ void k_gather_batch(int n, int ninst, const int* inst, const int* off, RowView src, const int* rowptr,
                                int* out_rp, int* col, double* val) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
     const int gw = gt >> 5;
@@ -3980,11 +4041,13 @@ __global__ void k_gather_batch(int n, int ninst, const int* inst, const int* off
 
 // bounds[i] = rowptr[off[i]], i = 0..ninst
 __global__ void k_bounds(int ninst, const int* off, const int* rowptr, int* bounds) {
+    pdl_enter();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i <= ninst) bounds[i] = rowptr[off[i]];
 }
 
 __global__ void k_identity(int n, double alpha, int* rowptr, int* col, double* val) {
+    pdl_enter();
     int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < n) {
         rowptr[r] = r;
@@ -4109,6 +4172,10 @@ static cudaError_t prod_launch(const ProductArgs& P, cudaStream_t st) {
     long long blocks = ((long long)P.n + kWarps - 1) / kWarps;
     const long long cap = (long long)sms_now() * ProdSmem<TAB, W>::kBlocksPerSm;
     if (blocks > cap) blocks = cap;
+    // (an ordinary launch: one wave of blocks that fill shared memory must find
+    // every SM free.  Brought in while a kernel without shared memory runs,
+    // some SMs take fewer of them and the rest make a second wave: cos on a
+    // 101 x 97 grid, squared, 2.64 -> 2.87 ms, exp on 128 x 128 3.61 -> 3.72)
     k_product<TAB, BATCH, WIDE, W><<<(unsigned)blocks, kWarps * 32, prod_smem_bytes<TAB, W>(), st>>>(P);
     ++g_launches;
     return cudaGetLastError();
@@ -4118,7 +4185,7 @@ static cudaError_t cta_launch(const ProductArgs& P, cudaStream_t st) {
     long long blocks = P.n;
     const long long cap = (long long)sms_now() * 7;
     if (blocks > cap) blocks = cap;
-    k_product_cta<<<(unsigned)blocks, kCtaWarps * 32, cta_smem_bytes(), st>>>(P);
+    launch_pdl(k_product_cta, (unsigned)blocks, kCtaWarps * 32, cta_smem_bytes(), st, P);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4154,20 +4221,11 @@ template <bool BATCH, bool TEAM, int R>
 static cudaError_t band_launch(const ProductArgs& P, cudaStream_t st) {
     const long long cap = (long long)sms_now() * 7, tiles = ((long long)P.n + R - 1) / R;
     const long long blocks = TEAM ? tiles : (tiles + kBandWarps - 1) / kBandWarps;
-    cudaLaunchConfig_t c{};
-    c.gridDim = dim3((unsigned)(blocks < cap ? blocks : cap));
-    c.blockDim = dim3(kBandWarps * 32);
-    c.dynamicSmemBytes = band_smem_bytes();
-    c.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &at;
-    c.numAttrs = P.pair ? 1 : 0;
+    const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
     ++g_launches;
     // (a batch's rows may be filtered when candidate lists are given)
-    return P.cand_col ? cudaLaunchKernelEx(&c, k_band<BATCH, TEAM, R, true>, P)
-                      : cudaLaunchKernelEx(&c, k_band<BATCH, TEAM, R, false>, P);
+    return launch_pdl(P.cand_col ? k_band<BATCH, TEAM, R, true> : k_band<BATCH, TEAM, R, false>, grid, kBandWarps * 32,
+                      band_smem_bytes(), st, P);
 }
 
 cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
@@ -4211,7 +4269,7 @@ cudaError_t launch_copy_result(int n, long long nnz, const int* rowptr, const in
     long long blocks = (most + 1023) / 1024;
     const long long cap = (long long)sms_now() * 8;
     if (blocks > cap) blocks = cap;
-    k_copy_result<<<(unsigned)blocks, 256, 0, st>>>(C);
+    launch_pdl(k_copy_result, (unsigned)blocks, 256, 0, st, C);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4221,7 +4279,7 @@ cudaError_t launch_row_lists(int n, const RowView& B, int2* hdr, uint2* lists, c
     long long blocks = ((long long)n + 7) / 8;
     const long long cap = (long long)sms_now() * 8;
     if (blocks > cap) blocks = cap;
-    k_row_lists<<<(unsigned)blocks, 256, 0, st>>>(n, B, hdr, lists);
+    launch_pdl(k_row_lists, (unsigned)blocks, 256, 0, st, n, B, hdr, lists);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4231,7 +4289,7 @@ cudaError_t launch_row_bitmaps(int n, const RowView& B, int2* hdr, unsigned* bit
     long long blocks = ((long long)n + 7) / 8;
     const long long cap = (long long)sms_now() * 8;
     if (blocks > cap) blocks = cap;
-    k_row_bitmaps<<<(unsigned)blocks, 256, 0, st>>>(n, B, hdr, bits);
+    launch_pdl(k_row_bitmaps, (unsigned)blocks, 256, 0, st, n, B, hdr, bits);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4245,12 +4303,14 @@ cudaError_t launch_alg1(const Alg1Args& A, double entries, cudaStream_t st) {
         c.gridDim = dim3((unsigned)dcfg().alg1_cluster);
         c.blockDim = dim3(kAlg1Threads);
         c.stream = st;
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = c.gridDim.x;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        c.attrs = &at;
-        c.numAttrs = 1;
+        cudaLaunchAttribute at[2]{};
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = c.gridDim.x;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        c.attrs = at;
+        c.numAttrs = 2;
         return cudaLaunchKernelEx(&c, k_alg1<true>, a);
     }
     void* args[] = {&a};
@@ -4268,7 +4328,7 @@ cudaError_t launch_norms(const NormArgs& A, cudaStream_t st) {
 }
 
 cudaError_t launch_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot* slot, cudaStream_t st) {
-    k_absmax<<<sms_now() * 4, 256, 0, st>>>(pool_val, ctl, i, slot);
+    launch_pdl(k_absmax, sms_now() * 4, 256, 0, st, pool_val, ctl, i, slot);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4276,7 +4336,7 @@ cudaError_t launch_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlo
 cudaError_t launch_validate(int n, int nnz, const int* rowptr, const int* col, const double* val, Ctl* ctl,
                             cudaStream_t st) {
     int blocks = (n + 1 + 255) / 256;
-    k_validate<<<blocks, 256, 0, st>>>(n, nnz, rowptr, col, val, ctl);
+    launch_pdl(k_validate, blocks, 256, 0, st, n, nnz, rowptr, col, val, ctl);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4286,9 +4346,9 @@ size_t scan_scratch_len(int n) { return (size_t)((n + kScanTile - 1) / kScanTile
 cudaError_t launch_scan_rows(int n, const int* rb, const int* re, const RowDesc* rd, int* rowptr, Ctl* ctl,
                              long long* sums, cudaStream_t st) {
     const int ntiles = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
-    k_scan_tile_sums<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums, ctl);
+    launch_pdl(k_scan_tile_sums, ntiles, kScanTile, 0, st, n, rb, re, rd, sums, ctl);
     ++g_launches;
-    k_scan_apply<<<ntiles, kScanTile, 0, st>>>(n, rb, re, rd, sums, rowptr);
+    launch_pdl(k_scan_apply, ntiles, kScanTile, 0, st, n, rb, re, rd, sums, rowptr);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4298,7 +4358,7 @@ cudaError_t launch_gather(int n, const RowView& src, const int* rowptr, int* col
     if (n <= 0) return cudaSuccess;
     int blocks = (n + 7) / 8;
     if (blocks > sms_now() * 16) blocks = sms_now() * 16;
-    k_gather<<<blocks, 256, 0, st>>>(n, src, rowptr, col, val);
+    launch_pdl(k_gather, blocks, 256, 0, st, n, src, rowptr, col, val);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4334,7 +4394,7 @@ cudaError_t launch_fp64_probe(int iters, double* out, cudaStream_t st) {
 }
 
 cudaError_t launch_identity(int n, double alpha, int* rowptr, int* col, double* val, cudaStream_t st) {
-    k_identity<<<(n + 1 + 255) / 256, 256, 0, st>>>(n, alpha, rowptr, col, val);
+    launch_pdl(k_identity, (n + 1 + 255) / 256, 256, 0, st, n, alpha, rowptr, col, val);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4347,7 +4407,7 @@ cudaError_t launch_copy_rows(int n, const int* rowptr, const int* col, const dou
     // copy is latency-bound and wants many warps in flight
     long long blocks = ((long long)n + 31) / 32;
     if (blocks > (long long)sms_now() * 8) blocks = (long long)sms_now() * 8;
-    k_copy_rows<<<(unsigned)blocks, 256, 0, st>>>(n, rowptr, col, val, rb, re, rd, pool_col, pool_val, ctl,
+    launch_pdl(k_copy_rows, (unsigned)blocks, 256, 0, st, n, rowptr, col, val, rb, re, rd, pool_col, pool_val, ctl,
                                                   arena_size, absmax);
     ++g_launches;
     return cudaGetLastError();
@@ -4358,7 +4418,7 @@ cudaError_t launch_norm_scratch_init(Ctl* ctl, NormSlot* slot, unsigned long lon
     int blocks = (int)(((long long)kChunks * n + 255) / 256);
     if (blocks < 1) blocks = 1;
     if (blocks > sms_now() * 4) blocks = sms_now() * 4;
-    k_norm_scratch_init<<<blocks, 256, 0, st>>>(ctl, slot, words, sticky, n, nnz);
+    launch_pdl(k_norm_scratch_init, blocks, 256, 0, st, ctl, slot, words, sticky, n, nnz);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4393,7 +4453,7 @@ cudaError_t launch_alg1_batch(const Alg1BatchArgs& A, cudaStream_t st) {
 
 cudaError_t launch_inst_table(int n, int ninst, const int* off, int* inst, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_inst_table<<<(n + 255) / 256, 256, 0, st>>>(n, ninst, off, inst);
+    launch_pdl(k_inst_table, (n + 255) / 256, 256, 0, st, n, ninst, off, inst);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4401,7 +4461,7 @@ cudaError_t launch_inst_table(int n, int ninst, const int* off, int* inst, cudaS
 cudaError_t launch_validate_batch(int n, const int* inst, const BatchSrc* src, const int* nnz, Ctl* ctl,
                                   unsigned char* band, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    k_validate_batch<<<(n + 255) / 256, 256, 0, st>>>(n, inst, src, nnz, ctl, band);
+    launch_pdl(k_validate_batch, (n + 255) / 256, 256, 0, st, n, inst, src, nnz, ctl, band);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4412,7 +4472,7 @@ cudaError_t launch_copy_rows_batch(int n, const int* inst, const BatchSrc* src, 
     if (n <= 0) return cudaSuccess;
     int blocks = (n + 7) / 8;
     if (blocks > sms_now() * 8) blocks = sms_now() * 8;
-    k_copy_rows_batch<<<blocks, 256, 0, st>>>(n, inst, src, rb, re, rd, pool_col, pool_val, ctl, arena_size, absmax,
+    launch_pdl(k_copy_rows_batch, blocks, 256, 0, st, n, inst, src, rb, re, rd, pool_col, pool_val, ctl, arena_size, absmax,
                                               stride);
     ++g_launches;
     return cudaGetLastError();
@@ -4424,7 +4484,7 @@ cudaError_t launch_compose_rows(int n, const int* inst, const int* sel, const Ro
     if (count > kMaxAdd + 2) return cudaErrorInvalidValue;
     RowTable T{};
     for (int k = 0; k < count; ++k) T.rd[k] = rds[k];
-    k_compose_rows<<<(n + 255) / 256, 256, 0, st>>>(n, inst, sel, T, out_rb, out_re, out_rd);
+    launch_pdl(k_compose_rows, (n + 255) / 256, 256, 0, st, n, inst, sel, T, out_rb, out_re, out_rd);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4434,13 +4494,13 @@ cudaError_t launch_gather_batch(int n, int ninst, const int* inst, const int* of
     int blocks = (n + 7) / 8;
     if (blocks < 1) blocks = 1;
     if (blocks > sms_now() * 16) blocks = sms_now() * 16;
-    k_gather_batch<<<blocks, 256, 0, st>>>(n, ninst, inst, off, src, rowptr, out_rp, col, val);
+    launch_pdl(k_gather_batch, blocks, 256, 0, st, n, ninst, inst, off, src, rowptr, out_rp, col, val);
     ++g_launches;
     return cudaGetLastError();
 }
 
 cudaError_t launch_bounds(int ninst, const int* off, const int* rowptr, int* bounds, cudaStream_t st) {
-    k_bounds<<<(ninst + 1 + 255) / 256, 256, 0, st>>>(ninst, off, rowptr, bounds);
+    launch_pdl(k_bounds, (ninst + 1 + 255) / 256, 256, 0, st, ninst, off, rowptr, bounds);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4450,19 +4510,19 @@ cudaError_t launch_reuse_copy_batch(const ProductArgs& P, cudaStream_t st) {
     long long blocks = ((long long)P.n + 7) / 8;
     const long long cap = (long long)num_sms() * 8;
     if (blocks > cap) blocks = cap;
-    k_reuse_copy_batch<<<(unsigned)blocks, 256, 0, st>>>(P);
+    launch_pdl(k_reuse_copy_batch, (unsigned)blocks, 256, 0, st, P);
     return cudaGetLastError();
 }
 
 cudaError_t launch_reset(Ctl* ctl, unsigned long long cap, unsigned long long cand_cap, unsigned cand_chunk,
                          cudaStream_t st) {
-    k_reset<<<1, 32, 0, st>>>(ctl, cap, cand_cap, cand_chunk);
+    launch_pdl(k_reset, 1, 32, 0, st, ctl, cap, cand_cap, cand_chunk);
     ++g_launches;
     return cudaGetLastError();
 }
 
 cudaError_t launch_export(const void* src, void* dst, size_t bytes, cudaStream_t st) {
-    k_export<<<1, 256, 0, st>>>(static_cast<const unsigned*>(src), static_cast<unsigned*>(dst), (int)(bytes / 4));
+    launch_pdl(k_export, 1, 256, 0, st, static_cast<const unsigned*>(src), static_cast<unsigned*>(dst), (int)(bytes / 4));
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4471,7 +4531,7 @@ cudaError_t launch_reuse_pass1(const ReuseArgs& R, cudaStream_t st) {
     if (R.n <= 0) return cudaSuccess;
     int blocks = (R.n + 7) / 8;
     if (blocks > sms_now() * 8) blocks = sms_now() * 8;
-    k_reuse_pass1<<<blocks, 256, 0, st>>>(R);
+    launch_pdl(k_reuse_pass1, blocks, 256, 0, st, R);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -4479,14 +4539,14 @@ cudaError_t launch_reuse_pass1(const ReuseArgs& R, cudaStream_t st) {
 cudaError_t launch_norms_rows(const NormRowsArgs& A, cudaStream_t st) {
     if (A.n <= 0 || A.count <= 0) return cudaSuccess;
     dim3 grid((unsigned)((A.n + kNormTile - 1) / kNormTile), (unsigned)A.count);
-    k_norms_rows<<<grid, kNormRowsThreads, norms_rows_smem_bytes(), st>>>(A);
+    launch_pdl(k_norms_rows, grid, kNormRowsThreads, norms_rows_smem_bytes(), st, A);
     ++g_launches;
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     const long long total = (long long)A.count * (((long long)A.n + 31) & ~31LL);
     long long blocks = (total + 255) / 256;  // one (matrix, column) per thread
     if (blocks > 65535LL * 64) blocks = 65535LL * 64;
-    k_norms_finish<<<(unsigned)blocks, 256, 0, st>>>(A.n, A.count, A.slots, A.words, A.sticky, A.ctl, A.inst,
+    launch_pdl(k_norms_finish, (unsigned)blocks, 256, 0, st, A.n, A.count, A.slots, A.words, A.sticky, A.ctl, A.inst,
                                                      A.slot_stride);
     ++g_launches;
     return cudaGetLastError();
