@@ -276,7 +276,8 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         // the bitmap map marks B rows from their column bitmaps (built here,
         // one launch over B); the chunked test settings keep the column marks
         const int bm = g_row_bitmaps.load();
-        const bool band = w.band && w.slot_map == 0 && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
+        // (the tuner's run without the table map takes the form that evaluations would)
+        const bool band = w.band && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
         uint2* const pl = A && !table && !band && bm > 0 && window == kLists && w.slot_map == 0 && w.chunk_cols <= 0 &&
                                   w.chunk_slots <= 0
                               ? w.lists()

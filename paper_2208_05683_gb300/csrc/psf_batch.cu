@@ -58,8 +58,13 @@ struct BatchStorage {
     }
 };
 
-// Pool sizing learnt from earlier batches (entries per row of the batch).
+// Pool sizing learnt from earlier batches (entries per row of the batch, of at
+// least one round of the chip's warps: a launch's warps each reserve a whole
+// arena, so a batch of a few hundred rows has far more entries reserved per
+// row than a large one will, and taught every worker of a server to allocate
+// pools of tens of GB).
 std::atomic<double> g_z_per_row{0.0}, g_ps_per_row{0.0};
+double pool_rows(int n) { return std::max((double)n, 28.0 * num_sms()); }
 
 void raise_to(std::atomic<double>& a, double v) {
     double cur = a.load();
@@ -197,7 +202,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     bool any_band = false, any_general = false;
     for (int i = 0; i < count; ++i) (isband[(size_t)i] ? any_band : any_general) = true;
     const unsigned char* d_band = nullptr;
-    if (any_band && w.slot_map == 0 && w.chunk_cols <= 0 && w.chunk_slots <= 0) d_band = d_isband.as<unsigned char>();
+    // (the tuner's run without the table map takes the form that evaluations would)
+    if (any_band && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) && w.chunk_cols <= 0 && w.chunk_slots <= 0) d_band = d_isband.as<unsigned char>();
     else any_general = true;
     const double zlen_all = n > 0 ? (double)nnz_tot / n : 0.0;
     const unsigned long long arena_z = arena_for(zlen_all > 0.0 ? zlen_all : 1.0);
@@ -231,7 +237,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         CU(d_zstep.alloc(sizeof(BatchStep) * (size_t)count, st));
         CU(cudaMemcpyAsync(d_zstep.p, zstep.data(), sizeof(BatchStep) * zstep.size(), cudaMemcpyHostToDevice, st));
         CU(d_zstat.alloc(sizeof(StepStat) * 9 * (size_t)count, st));
-        unsigned long long zcap = (unsigned long long)(g_z_per_row.load() * 1.25 * n) + 4096ull;
+        unsigned long long zcap = (unsigned long long)(g_z_per_row.load() * 1.25 * pool_rows(n)) + 4096ull;
         unsigned long long est = (unsigned long long)nnz_tot * (any_chain ? 128ull : 2ull) + (unsigned long long)n * 8ull +
                                  4096ull * 64ull;
         if (g_z_per_row.load() == 0.0 && zcap < est) zcap = est;
@@ -324,7 +330,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 if (zcap > kMaxPool) zcap = kMaxPool;
                 continue;
             }
-            if (n > 0) raise_to(g_z_per_row, (double)c.pool_used / n);
+            if (n > 0) raise_to(g_z_per_row, (double)c.pool_used / pool_rows(n));
             break;
         }
         std::vector<NormSlot> hs(kMaxNorms * (size_t)count);
@@ -554,7 +560,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     }
 
     // ---- PS phase in one pool
-    unsigned long long cap = (unsigned long long)(g_ps_per_row.load() * 1.25 * n) + 4096ull;
+    unsigned long long cap = (unsigned long long)(g_ps_per_row.load() * 1.25 * pool_rows(n)) + 4096ull;
     {
         unsigned long long est = (unsigned long long)nnz_tot * 64ull + (unsigned long long)n * 64ull + 4096ull * 64ull;
         for (int i = 0; i < count; ++i) est += (unsigned long long)(4.0 * ip[(size_t)i].znnz[10]);
@@ -777,7 +783,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             if (cap > kMaxPool) cap = kMaxPool;
             continue;
         }
-        if (n > 0) raise_to(g_ps_per_row, (double)cfin.pool_used / n);
+        if (n > 0) raise_to(g_ps_per_row, (double)cfin.pool_used / pool_rows(n));
         break;
     }
     const unsigned long long nnz_out = cfin.nnz_total;

@@ -1305,7 +1305,8 @@ __global__ void __launch_bounds__(ProdSmem<TAB, W>::kWarps * 32, ProdSmem<TAB, W
     if (threadIdx.x == 0) {
         // the block's warps take their first pool arenas with one atomic: at
         // the launch every warp wants one at once, on the same counter
-        blk_arena = atomicAdd(&P.ctl->pool_used, (unsigned long long)kWarps * P.arena);
+        // (beside k_band a warp takes its first with its first row: it may have none)
+        blk_arena = BATCH && P.pair ? ~0ull >> 1 : atomicAdd(&P.ctl->pool_used, (unsigned long long)kWarps * P.arena);
         blk_span = blk_words = 0;
         blk_fma = 0ull;
         blk_written = 0ull;
