@@ -203,8 +203,16 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     for (int i = 0; i < count; ++i) (isband[(size_t)i] ? any_band : any_general) = true;
     const unsigned char* d_band = nullptr;
     // (the tuner's run without the table map takes the form that evaluations would)
-    if (any_band && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) && w.chunk_cols <= 0 && w.chunk_slots <= 0) d_band = d_isband.as<unsigned char>();
-    else any_general = true;
+    // from two rounds of the chip's warps on: with fewer rows the second launch
+    // of every stage costs more than the banded rows' fold saves (us a call,
+    // one launch / two: 8 instances of 64-980 rows 1870 / 2050, 14 of 64-4096
+    // 3720 / 3780, 27 of 64-3906 5240 / 5040, 54 of 64-1283 7850 / 7000, 128 of
+    // 64-4096 18000 / 16500)
+    if (any_band && n >= 56 * num_sms() && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) &&
+        w.chunk_cols <= 0 && w.chunk_slots <= 0)
+        d_band = d_isband.as<unsigned char>();
+    else
+        any_general = true;
     const double zlen_all = n > 0 ? (double)nnz_tot / n : 0.0;
     const unsigned long long arena_z = arena_for(zlen_all > 0.0 ? zlen_all : 1.0);
 
