@@ -278,8 +278,10 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         const int bm = g_row_bitmaps.load();
         // (the tuner's run without the table map takes the form that evaluations would)
         const bool band = w.band && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
-        uint2* const pl = A && !table && !band && bm > 0 && window == kLists && w.slot_map == 0 && w.chunk_cols <= 0 &&
-                                  w.chunk_slots <= 0
+        // (one row per block reads bitmaps only: such a step gets no lists)
+        const bool cta = A && !table && (w.slot_map == 4 || (w.slot_map == 0 && use_cta(w.n, alen, blen)));
+        uint2* const pl = A && !table && !band && !cta && bm > 0 && window == kLists && w.slot_map == 0 &&
+                                  w.chunk_cols <= 0 && w.chunk_slots <= 0
                               ? w.lists()
                               : nullptr;
         if (pl) {
@@ -292,7 +294,6 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
             P.bhdr = w.bhdr.as<int2>();
             P.bbits = w.pool_bits.as<unsigned>();
         }
-        const bool cta = A && !table && (w.slot_map == 4 || (w.slot_map == 0 && use_cta(w.n, alen, blen)));
         if (band) CU(launch_band(P, A ? alen + blen : 0.0, w.st));
         else CU(launch_product(P, table, w.st, out_len, window != kNarrow || w.slot_map == 3, cta));
     }
@@ -726,11 +727,12 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
         words_baby = series->words_baby;
         words_giant = series->words_giant;
     }
-    // the window of a step: by its record, or what e applications of Z reach
+    // the window of a step: by its record (of a matrix that may have been a
+    // larger one: no row spans more than n), or what e applications of Z reach
     // from a row with `words` words
     auto window_of = [&](const std::vector<unsigned>& span, const std::vector<unsigned>& words, size_t i, double e,
                          double est) {
-        if (i < span.size()) return window_for(span[i], i < words.size() ? (double)words[i] : 0.0);
+        if (i < span.size()) return window_for(std::min((double)n, (double)span[i]), i < words.size() ? (double)words[i] : 0.0);
         return window_for(std::min((double)n, 2.0 * e * w.bandwidth + 1.0), est);
     };
     w.chunk_cols = series->chunk_cols;

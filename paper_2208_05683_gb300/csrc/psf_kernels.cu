@@ -1642,7 +1642,7 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
             S.kb[wib][lane] = b;
             S.kl[wib][lane] = e - b;
             int h = 0;
-            if (P.bhdr) {
+            if (P.bbits) {  // (the headers of lists are not a bitmap's)
                 const int2 bh = P.bhdr[k];
                 h = bh.y > 0 ? ((bh.x - (lo >> 5)) << 16) | bh.y : 0;
             }
@@ -4221,7 +4221,7 @@ static cudaError_t cta_launch(const ProductArgs& P, cudaStream_t st) {
 cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, double out_len, bool wide_window,
                            bool cta) {
     if (P.n <= 0) return cudaSuccess;
-    if (cta && !table && !P.inst && P.chunk_cols <= 0 && P.chunk_slots <= 0) return cta_launch(P, st);
+    if (cta && !table && !P.inst && !P.blists && P.chunk_cols <= 0 && P.chunk_slots <= 0) return cta_launch(P, st);
     if (P.inst) {
         if (table) return prod_launch<true, true, false>(P, st);
         return wide_window ? prod_launch<false, true, false, kBmWordsBig>(P, st) : prod_launch<false, true, false>(P, st);
