@@ -568,7 +568,7 @@ int psf_norm1(const psf_csr_t* M, void* stream, double* out) {
         return PSF_OK;
     }
     // M's entries are read in place; its check's outcome comes with the norm
-    // (the norm kernels never index with a column outside [0, n)), so there is
+    // (the norm kernels read nothing of a matrix that failed it), so there is
     // one synchronisation
     Work w;
     if ((rc = w.init(M->n, st, 0))) return rc;
@@ -1474,8 +1474,8 @@ extern "C" int psf_norm1_noalloc(const psf_csr_t* M, void* stream, double* out) 
     unsigned* sticky = reinterpret_cast<unsigned*>(base + kNaSticky);
     unsigned long long* words = reinterpret_cast<unsigned long long*>(base + kNaWords);
     // clear what must start at zero, check the input (its outcome is read
-    // with the result; the norm kernels never index with a column outside
-    // [0, n)), then max |x| and the exact column sums over M's entries
+    // with the result; the norm kernels read nothing of a matrix that failed
+    // it), then max |x| and the exact column sums over M's entries
     CU(launch_norm_in_place(ctl, slot, words, sticky, *M, st));
     int status = 0;
     unsigned long long bits = 0ull;

@@ -3253,9 +3253,10 @@ __global__ void __launch_bounds__(kNormThreads) k_norms(NormArgs A) {
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthreads = gridDim.x * blockDim.x;
     const size_t n = (size_t)A.n;
-    // a phase whose pool overflowed is discarded (all blocks read the same
-    // status, set by an earlier launch)
-    if (__ldcg(&A.ctl->status) & kDevPoolFull) return;
+    // a phase whose pool overflowed is discarded, and a caller's matrix that
+    // failed its check is not read: only the check has bounded its entry count
+    // (all blocks read the same status, set by an earlier launch)
+    if (__ldcg(&A.ctl->status) & (kDevPoolFull | kDevBadInput)) return;
     // every |x| of every matrix into per-column fixed-point sums: streaming
     // passes over the matrices' pool ranges
     for (int mi = 0; mi < A.count; ++mi) {
@@ -3702,6 +3703,7 @@ __global__ void k_reset(Ctl* ctl, unsigned long long cap, unsigned long long can
 // max |x| over the pool entries [mark[i], mark[i+1])
 __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot* slot) {
     pdl_enter();
+    if (__ldcg(&ctl->status) & kDevBadInput) return;  // (as k_norms)
     const int lane = threadIdx.x & 31;
     const unsigned long long cap = ctl->pool_cap;  // counters may run past it on overflow
     const unsigned long long p0 = min(__ldcg(&ctl->mark[i]), cap), p1 = min(__ldcg(&ctl->mark[i + 1]), cap);
