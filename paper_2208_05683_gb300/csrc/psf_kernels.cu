@@ -237,7 +237,7 @@ __device__ __forceinline__ void load_segment(const ProductArgs& P, int seg, int 
 }
 
 // ---- symbolic pass, table map: plain flag stores, four pieces per step
-__device__ __forceinline__ void mark_row(const int* __restrict__ col, int s, int e, int c0, int cend, int lane,
+__device__ __forceinline__ void mark_row(const int* col, int s, int e, int c0, int cend, int lane,
                                          ProdSmem<true>& S) {
     for (int q0 = s; q0 < e; q0 += 128) {
         int cs[4];
@@ -264,7 +264,7 @@ __device__ __forceinline__ void clear_map(int wlen, int lane, ProdSmem<true>& S)
 // load_segment has already clipped it to that range (or, for a row that
 // takes one chunk, the range spans every B column of the row).
 template <bool CHK, int W>
-__device__ __forceinline__ void mark_row(const int* __restrict__ col, int s, int e, int c0, int cend, int lane,
+__device__ __forceinline__ void mark_row(const int* col, int s, int e, int c0, int cend, int lane,
                                          ProdSmem<false, W>& S) {
     const int m = (e - s + 31) >> 5;
     const int q0 = s + lane * m, q1 = min(e, q0 + m);
@@ -293,7 +293,7 @@ __device__ __forceinline__ void mark_row(const int* __restrict__ col, int s, int
 // before either row's columns are ORed in, so the second row's loads do not
 // wait for the first row's marking.  The rows are clipped to the window.
 template <int W>
-__device__ __forceinline__ void mark_row_pair(const int* __restrict__ col, int sa, int ea, int sb, int eb, int c0,
+__device__ __forceinline__ void mark_row_pair(const int* col, int sa, int ea, int sb, int eb, int c0,
                                               int lane, ProdSmem<false, W>& S) {
     const int ma = (ea - sa + 31) >> 5, mb = (eb - sb + 31) >> 5;
     int qa = sa + lane * ma, qb = sb + lane * mb;
@@ -338,7 +338,7 @@ __device__ __forceinline__ void mark_row_pair(const int* __restrict__ col, int s
 // so the rows' column loads are in flight together instead of one row after
 // the other.  The rows are clipped to [c0, cend) (see mark_row).
 template <int W>
-__device__ __forceinline__ void mark_rows_short(const int* __restrict__ col, int cnt, int c0, int cend, int lane,
+__device__ __forceinline__ void mark_rows_short(const int* col, int cnt, int c0, int cend, int lane,
                                                 ProdSmem<false, W>& S, bool active = true) {
     if (lane >= cnt || !active) return;
     const int s = S.kb[lane], e = s + S.kl[lane];
@@ -385,7 +385,7 @@ __device__ __forceinline__ void mark_from_bitmaps(const ProductArgs& P, int pa0,
 #pragma unroll
     for (int u = 0; u < R; ++u) reg[u] = 0u;
     int* kwn = reinterpret_cast<int*>(S.colbuf);  // free until the slots are assigned
-    const unsigned* __restrict__ bits = P.bbits;
+    const unsigned* bits = P.bbits;
     for (int seg = pa0; seg < pa1; seg += 32) {
         const int cnt = min(32, pa1 - seg);
         load_segment<false>(P, seg, cnt, true, c0, cend, lane, S, store_a, a_holes, fma, kwn);
@@ -597,7 +597,7 @@ struct Chunk {
 };
 
 template <bool TAB, int W>
-__device__ __forceinline__ void chunk_load(const int* __restrict__ bcol, const double* __restrict__ bval,
+__device__ __forceinline__ void chunk_load(const int* bcol, const double* bval,
                                            const ProdSmem<TAB, W>& S, int kk, int off, int lane, Chunk& ch) {
     const int len = S.kl[kk];
     const int* rc = bcol + S.kb[kk] + lane;
@@ -652,8 +652,8 @@ __device__ __forceinline__ void chunk_fold(ProdSmem<TAB, W>& S, const Chunk& ch,
 template <bool WIDE>
 __device__ __forceinline__ void accumulate_segment(const ProductArgs& P, int /*seg*/, int cnt, int c0, int lane,
                                                    ProdSmem<true>& S, bool /*wide_row*/) {
-    const int* __restrict__ bcol = P.B.col;
-    const double* __restrict__ bval = P.B.val;
+    const int* bcol = P.B.col;
+    const double* bval = P.B.val;
     int k0 = 0, o0 = 0;
     while (k0 < cnt && S.kl[k0] == 0) ++k0;
     if (k0 >= cnt) return;
@@ -688,7 +688,7 @@ __device__ __forceinline__ void accumulate_segment(const ProductArgs& P, int /*s
 // One 32-lane piece of short B row kk (at most 32 entries): column -1 where
 // there is none.
 template <int W>
-__device__ __forceinline__ void short_load(const int* __restrict__ bcol, const double* __restrict__ bval,
+__device__ __forceinline__ void short_load(const int* bcol, const double* bval,
                                            const ProdSmem<false, W>& S, int cnt, int kk, int lane, int& c, double& v) {
     c = -1;
     v = 0.0;
@@ -709,8 +709,8 @@ __device__ __forceinline__ void short_fold(ProdSmem<false, W>& S, int c, double 
 template <bool WIDE, int W>
 __device__ __forceinline__ void accumulate_segment(const ProductArgs& P, int seg, int cnt, int c0, int lane,
                                                    ProdSmem<false, W>& S, bool wide_row) {
-    const int* __restrict__ bcol = P.B.col;
-    const double* __restrict__ bval = P.B.val;
+    const int* bcol = P.B.col;
+    const double* bval = P.B.val;
     const double* ka = ka_of(S);
     // a_rk of row kk: kept in the accumulator's last slots, or (WIDE, or a
     // row that takes every slot) read from A's row (the same address in
@@ -758,8 +758,8 @@ __device__ __forceinline__ void accumulate_segment(const ProductArgs& P, int seg
             }
         } else {
             // whole 128-entry chunks: four full pieces, no per-lane tests
-            const int* __restrict__ rc = bcol + S.kb[kk] + lane;
-            const double* __restrict__ rv = bval + S.kb[kk] + lane;
+            const int* rc = bcol + S.kb[kk] + lane;
+            const double* rv = bval + S.kb[kk] + lane;
             int off = 0;
             for (; off + 128 <= len; off += 128) {
                 int j[4];
@@ -831,7 +831,7 @@ __device__ __forceinline__ void list_or(ProdSmem<false, kListWords>& S, bool act
 }
 // The columns of [c0, cend) among the row [s, e) (ascending), 32 at a time:
 // the lanes of one word form a run, whose bits a segmented OR collects.
-__device__ __forceinline__ void list_mark_row(const int* __restrict__ col, int s, int e, int c0, int cend, int lane,
+__device__ __forceinline__ void list_mark_row(const int* col, int s, int e, int c0, int cend, int lane,
                                               ProdSmem<false, kListWords>& S, int& nid) {
     for (int q0 = s; q0 < e; q0 += 32) {
         const int q = q0 + lane;
@@ -1758,8 +1758,8 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
         __syncthreads();
     }
     // ---- the B rows, k ascending, a block barrier after each
-    const int* __restrict__ bcol = P.B.col;
-    const double* __restrict__ bval = P.B.val;
+    const int* bcol = P.B.col;
+    const double* bval = P.B.val;
     for (int seg = pa0; seg < pa1; seg += 32) {
         const int cnt = min(32, pa1 - seg);
         __syncthreads();  // every thread is done with the last segment (its last rows may be empty)
@@ -1775,8 +1775,8 @@ __device__ __forceinline__ void cta_row(const ProductArgs& P, const AddTerm* add
             const int len = S.kl[0][kk];
             if (len == 0) continue;
             const double a = S.ka[kk];
-            const int* __restrict__ rc = bcol + S.kb[0][kk];
-            const double* __restrict__ rv = bval + S.kb[0][kk];
+            const int* rc = bcol + S.kb[0][kk];
+            const double* rv = bval + S.kb[0][kk];
             int off = tid;
             for (; off + 3 * kT < len; off += 4 * kT) {
                 int j[4];
@@ -1922,7 +1922,7 @@ struct BandStage {  // terms k of the tile's rows
 // acc[r][u] = fma(a[r], x[u], acc[r][u]) for the rows [R0, R1] and the pieces
 // [U0, U1], the columns this lane has (in[u])
 template <int R, int U0, int U1, int R0, int R1>
-__device__ __forceinline__ void fold_rows(const double* __restrict__ a, const double (&x)[2], const bool (&in)[2],
+__device__ __forceinline__ void fold_rows(const double* a, const double (&x)[2], const bool (&in)[2],
                                           double (&acc)[R][2]) {
 #pragma unroll
     for (int r = R0; r <= R1; ++r) {
@@ -1938,7 +1938,7 @@ __device__ __forceinline__ void fold_rows(const double* __restrict__ a, const do
 // part (a chain with every lane predicated off measured the time of a full
 // one).
 template <int R, int U0, int U1>
-__device__ __forceinline__ void fold_term(int rows, const double* __restrict__ a, const double (&x)[2],
+__device__ __forceinline__ void fold_term(int rows, const double* a, const double (&x)[2],
                                           const bool (&in)[2], double (&acc)[R][2]) {
     if constexpr (R == 1) {
         fold_rows<R, U0, U1, 0, 0>(a, x, in, acc);
@@ -1969,7 +1969,7 @@ __device__ __forceinline__ void fold_term(int rows, const double* __restrict__ a
 // The columns gmin + lane + 32 u <= gmax of a group over the staged terms
 // [0, nt) in order, the pieces that B row k meets.
 template <int R, bool TEAM>
-__device__ __forceinline__ void fold_group(const BandStage<R, TEAM>& G, int nt, const double* __restrict__ val,
+__device__ __forceinline__ void fold_group(const BandStage<R, TEAM>& G, int nt, const double* val,
                                            int gmin, int gmax, int lane, double (&acc)[R][2]) {
     const double* const v = val + gmin + lane;
 #pragma unroll 1
@@ -3600,14 +3600,14 @@ __global__ void __launch_bounds__(256) k_copy_result(const __grid_constant__ Cop
     const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
 #pragma unroll 1
     for (int a = 0; a < 3; ++a) {
-        const unsigned* __restrict__ s = C.src[a];
-        unsigned* __restrict__ d = C.dst[a];
+        const unsigned* s = C.src[a];
+        unsigned* d = C.dst[a];
         const long long n = C.words[a];
         const long long head = ((16 - ((unsigned long long)d & 15)) & 15) >> 2;
         if ((((unsigned long long)s ^ (unsigned long long)d) & 15) == 0 && n > head) {
             const long long q = (n - head) >> 2;  // 16-byte pieces
-            const uint4* __restrict__ s4 = reinterpret_cast<const uint4*>(s + head);
-            uint4* __restrict__ d4 = reinterpret_cast<uint4*>(d + head);
+            const uint4* s4 = reinterpret_cast<const uint4*>(s + head);
+            uint4* d4 = reinterpret_cast<uint4*>(d + head);
             long long i = t0;
             for (; i + 3 * step < q; i += 4 * step) {
                 const uint4 x0 = s4[i], x1 = s4[i + step], x2 = s4[i + 2 * step], x3 = s4[i + 3 * step];
