@@ -860,6 +860,9 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     if (make_plan(a, tol_g, poly, submult, series->s, norms, p, stride))
         return fail(PSF_ENOTCONV, "no truncation length within %zu coefficients (Eq. 34)", a.size());
     if (p.q > PSF_MAX_Q) return fail(PSF_ETOOBIG, "q = %d exceeds %d", p.q, PSF_MAX_Q);
+    // (no banded products of this phase, nor the norm phase's, whose rows may keep holes)
+    const bool holes = p.bound <= kHoleBound;
+    if (!holes) w.band = false;
     const int N = p.N, q = p.q, b = p.b, g = p.g;
     const int stat_cap = q + b + 4;
     StepStat* pstat = nullptr;  // the PS phase's step records
@@ -906,7 +909,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
         for (int attempt = 0;; ++attempt) {
             // attempt 0 continues in the norm phase's pool when it reserved
             // room; a retry after an overflow starts from an empty pool
-            const bool reuse = attempt == 0 && ps_reserve > 0;
+            const bool reuse = attempt == 0 && ps_reserve > 0 && holes;
             const unsigned long long used_before = reuse ? z_used : 0ull;
             if (!reuse && (rc = w.reset_pool(cap))) return rc;
             if ((rc = w.stats_for(stat_cap, attempt > 0, &pstat))) return rc;

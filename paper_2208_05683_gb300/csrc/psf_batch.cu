@@ -377,6 +377,15 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         }
     }
 
+    // no holes where a product's operand may overflow (kHoleBound): no banded
+    // products in this phase, and no rows of the norm phase's
+    auto holes = [&](int i) { return ip[(size_t)i].trivial || ip[(size_t)i].p.bound <= kHoleBound; };
+    for (int i = 0; i < count; ++i)
+        if (!holes(i)) {
+            d_band = nullptr;
+            any_general = true;
+        }
+
     // ---- the norm phase's powers stay in their pool for the baby steps: while
     // an instance has dropped no entry, its baby step k is its Z^k
     bool keep_powers = false;
@@ -475,7 +484,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 if (D.index <= p.q) {
                     const double thr = nofilter ? 0.0 : p.zeta[(size_t)D.index];
                     B = step_of(kBatchProduct, thr, S->e_r, S->maxit);
-                    if (keep_powers && chain[(size_t)i] && D.index <= 10 && !P.sq) {
+                    if (keep_powers && holes(i) && chain[(size_t)i] && D.index <= 10 && !P.sq) {
                         B.reuse = 1;
                         T.any_reuse = true;
                         T.reuse_rows += ni;

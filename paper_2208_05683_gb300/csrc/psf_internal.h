@@ -344,6 +344,15 @@ inline int window_for(double span, double words) {
     return words > 0.0 && words <= kListMapWords ? kLists : kWide;
 }
 
+// A row may keep holes (stored zeros: k_band, filter_row) where no operand of
+// a product can have overflowed: the fold takes a hole as an entry, and
+// 0 * inf would put a NaN where an entry that is not there gives nothing.
+// By the norms' bounds (Plan::bound), with room for norms that are estimates
+// (their error grows with the power: 2^323 to the largest double).  Past it a
+// plan's thresholds are 0 wherever an operand is infinite, so the filter
+// leaves no holes either.
+constexpr double kHoleBound = 0x1p700;
+
 // Recorder of product launches for psf_autotune (set on the calling thread
 // only): each launch's work per row and its event pair.
 struct TuneRecorder {

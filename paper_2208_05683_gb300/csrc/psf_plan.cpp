@@ -95,6 +95,7 @@ int make_plan(const std::vector<double>& a, double tol, bool poly, bool submult,
     p.zeta.assign((size_t)q + 2, 0.0);
     p.sigma.assign((size_t)b + 1, 0.0);
     p.d.assign((size_t)q + 2, 0.0);
+    p.bound = 0.0;
     if (N < 2) return 0;
 
     auto coef = [&](int idx) { return (idx < N && idx < M) ? a[(size_t)idx] : 0.0; };
@@ -111,6 +112,12 @@ int make_plan(const std::vector<double>& a, double tol, bool poly, bool submult,
     // Eq. (26)
     nS[0] = nB[(size_t)b - 1];
     for (int i = 1; i < b; ++i) nS[(size_t)i] = nB[(size_t)(b - 1 - i)] + z[(size_t)q] * nS[(size_t)i - 1];
+
+    // the operands: the powers up to q, and S_0 .. S_{b-2}
+    for (int k = 1; k <= q; ++k)
+        if (!(z[(size_t)k] <= p.bound)) p.bound = std::isnan(z[(size_t)k]) ? INFINITY : z[(size_t)k];
+    for (int i = 0; i + 1 < b; ++i)
+        if (!(nS[(size_t)i] <= p.bound)) p.bound = std::isnan(nS[(size_t)i]) ? INFINITY : nS[(size_t)i];
 
     // Eq. (21): beta_{i,k} = sum_{l=k}^{q-1} |a_{iq+l}| z_{l-k}
     auto beta = [&](int i, int k) {

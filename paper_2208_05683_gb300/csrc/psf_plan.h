@@ -14,6 +14,7 @@ struct Plan {
     std::vector<double> zeta;   // index k = 2..q
     std::vector<double> sigma;  // index j = 1+g..b-1
     std::vector<double> d;      // d_k (Eq. 24)
+    double bound = 0.0;         // no entry of a product's operand in the scheme is larger (inf: unknown)
 };
 
 // Returns 0 on success, 1 if no truncation length exists within the supplied
