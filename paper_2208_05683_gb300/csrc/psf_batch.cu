@@ -206,8 +206,8 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     // from two rounds of the chip's warps on: with fewer rows the second launch
     // of every stage costs more than the banded rows' fold saves (us a call,
     // one launch / two: 8 instances of 64-980 rows 1870 / 2050, 14 of 64-4096
-    // 3720 / 3780, 27 of 64-3906 5240 / 5040, 54 of 64-1283 7850 / 7000, 128 of
-    // 64-4096 18000 / 16500)
+    // 3720 / 3780, 20 of 64-4096 3980 / 3760, 54 of 64-1283 6230 / 6260, 27 of
+    // 64-3906 5060 / 4790, 54 of 64-4096 8730 / 8040, 128 of 64-4096 17600 / 15800)
     if (any_band && n >= 56 * num_sms() && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) &&
         w.chunk_cols <= 0 && w.chunk_slots <= 0)
         d_band = d_isband.as<unsigned char>();

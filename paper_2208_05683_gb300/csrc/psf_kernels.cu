@@ -4243,7 +4243,7 @@ cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, do
 // launched programmatically: its blocks take the SMs that k_product's leave
 // (each kernel's warps end at different times, a quarter of them idle on
 // average), and it waits for k_product's end before it ends the step itself.
-// 128 instances of 64-4096 rows: 17.6 -> 17.1 ms a call, 27: 5.9 -> 5.3 ms.
+// 128 instances of 64-4096 rows: 17.6 -> 15.8 ms a call, 27: 5.1 -> 4.8 ms.
 // (One launch that hands rows of both kinds to the same warps or SMs was
 // slower, 19.4-23.3 ms: the two codes together outgrow an SM's instruction
 // cache.)
@@ -4268,14 +4268,19 @@ cudaError_t launch_band(const ProductArgs& P, double row_len, cudaStream_t st) {
     // of the chip's warps or several (one row / four: n = 2000, 31 x 61 36 /
     // 57; n = 12000 91 / 83; n = 20000, 1.2 rounds, 140 / 169; n = 65536
     // 408 / 375), and for rows of one 32-column piece, which are mostly
-    // set-up (11 x 11: n = 12000 36 / 29, n = 65536 117 / 83).  A batch: one
-    // row below one round (a call of 4 instances, 2000 rows at most: 2.22 ms
-    // with four, 1.61 with one); its rows' lengths differ too much for more.
+    // set-up (11 x 11: n = 12000 36 / 29, n = 65536 117 / 83).  A batch: four
+    // rows from three rounds on where every instance is banded (ms a call, one
+    // row / four: 25.6 k rows 5.07 / 5.62, 80 k 7.22 / 7.12, 131 k 13.1 / 12.8,
+    // 320 k 26.2 / 24.5), one where k_product shares the step: the tiles then
+    // take what SMs its rows leave, and the batch's tile of four rows spills
+    // most (one row / four, rows of which banded: 26 k, 13 k 6.26 / 6.95; 26 k,
+    // 18 k 4.79 / 4.94; 56 k, 35 k 12.7 / 13.8; 111 k, 83 k 15.8 / 16.3; 268 k,
+    // 185 k 42.5 / 43.1).
     const double warps = sms_now() * 7.0 * kBandWarps;
     const double rounds = P.n / (4.0 * warps);  // of tiles of four rows
     const bool team = row_len > 300.0 || (row_len > 128.0 && P.n <= 5.0 * warps / kBandWarps) ||
                       (row_len > 80.0 && P.n <= 2.0 * warps / kBandWarps);
-    if (P.inst) return rounds >= 1.0 ? band_launch<true, false, 4>(P, st) : band_launch<true, false, 1>(P, st);
+    if (P.inst) return !P.pair && rounds >= 3.0 ? band_launch<true, false, 4>(P, st) : band_launch<true, false, 1>(P, st);
     if (team) return rounds >= 0.9 ? band_launch<false, true, 4>(P, st) : band_launch<false, true, 1>(P, st);
     if (rounds >= (row_len <= 32.0 ? 0.35 : 3.0) || (rounds <= 1.0 && rounds >= 0.45))
         return band_launch<false, false, 4>(P, st);
