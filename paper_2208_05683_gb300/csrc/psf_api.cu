@@ -171,16 +171,27 @@ int status_to_code(int st) {
 
 // Validate input matrices on the device and wait for the outcome: nothing
 // indexes with an input's columns before this returns PSF_OK.  Notes whether
-// every row of every input so far spans consecutive columns (w.band).
-int validate_inputs(Work& w, const std::vector<const psf_csr_t*>& ms) {
+// every row of every input spans consecutive columns and those of A B do too,
+// up to a few (w.band); series: and of sums of their powers.
+int validate_inputs(Work& w, const std::vector<const psf_csr_t*>& ms, const psf_csr_t* A, const psf_csr_t* B,
+                    bool series) {
     for (const psf_csr_t* m : ms)
         if (m) CU(launch_validate(m->n, m->nnz, m->rowptr, m->col, m->val, w.C(), w.st));
     Ctl c;
     int rc = read_back(w, c);
     if (rc) return rc;
+    if ((rc = status_to_code(c.status))) return rc;
     w.band = !c.not_band;
     w.bandwidth = (int)c.bandwidth;
-    return status_to_code(c.status);
+    if (w.band && c.apart) {
+        w.band = A != nullptr;  // (sums alone: their terms' places are not looked at)
+        if (A) {
+            CU(launch_count_apart(*A, *B, series, w.C(), w.st));
+            if ((rc = read_back(w, c))) return rc;
+            w.band = mostly_runs(c.apart_rows, w.n);
+        }
+    }
+    return PSF_OK;
 }
 
 
@@ -198,11 +209,12 @@ unsigned long long arena_for(double row_len) {
 // reuse_k > 0: the step is baby step k and row slot `slot` still holds the
 // norm phase's Z^k; while no entry has been dropped (a device flag), the
 // product is skipped and k_reuse_pass1 does the step on those rows.
+// general: a step of a band whose rows are mostly in pieces (not k_band's).
 int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddTerm>& add,
              double threshold, double e_r, int maxit, StepStat* stat, size_t slot, RowView* out,
              NormSlot* absmax_slot = nullptr, double blen = 0.0, double alen = 0.0, int reuse_k = 0,
              unsigned long long reuse_fma = 0, double out_len = 0.0, int window = kNarrow,
-             double fma_hint = 0.0, int mark = 0) {
+             double fma_hint = 0.0, int mark = 0, bool general = false) {
     if (add.size() > (size_t)kMaxAdd) return fail(PSF_ETOOBIG, "%zu addend terms (max %d)", add.size(), kMaxAdd);
     Rows R;
     int rc = w.rows_for(slot, &R);
@@ -277,7 +289,7 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
         // one launch over B); the chunked test settings keep the column marks
         const int bm = g_row_bitmaps.load();
         // (the tuner's run without the table map takes the form that evaluations would)
-        const bool band = w.band && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
+        const bool band = w.band && !general && (w.slot_map == 0 || (g_tune_rec && w.slot_map == 2)) && w.chunk_cols <= 0 && w.chunk_slots <= 0 && !table;
         // (one row per block reads bitmaps only: such a step gets no lists)
         const bool cta = A && !table && (w.slot_map == 4 || (w.slot_map == 0 && use_cta(w.n, alen, blen)));
         uint2* const pl = A && !table && !band && !cta && bm > 0 && window == kLists && w.slot_map == 0 &&
@@ -612,7 +624,7 @@ int psf_product_filter(const psf_csr_t* A, const psf_csr_t* B, int32_t nadd, con
     w.dense_estimate = true;  // one product: the operands' mean row lengths give its expected count
     std::vector<const psf_csr_t*> inputs{A, B};
     for (int t = 0; t < nadd; ++t) inputs.push_back(addends[t]);
-    if ((rc = validate_inputs(w, inputs))) return rc;
+    if ((rc = validate_inputs(w, inputs, A, B, false))) return rc;
     const double blen = B && n > 0 ? (double)B->nnz / n : 0.0;
     unsigned long long est = (unsigned long long)n * 8ull + 16;
     for (int t = 0; t < nadd; ++t)
@@ -712,7 +724,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
 
     Work w;
     if ((rc = w.init(n, st, submult ? 1 : 10)) || (rc = w.init_products())) return rc;
-    if ((rc = validate_inputs(w, {Z}))) return rc;
+    if ((rc = validate_inputs(w, {Z}, Z, Z, true))) return rc;
     w.slot_map = series->kernel;
     w.dense_xover = series->dense_xover >= 0.0 ? series->dense_xover : g_dense_xover.load();
     // the column windows the series' previous evaluation measured (batches on
@@ -734,6 +746,19 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                          double est) {
         if (i < span.size()) return window_for(std::min((double)n, (double)span[i]), i < words.size() ? (double)words[i] : 0.0);
         return window_for(std::min((double)n, 2.0 * e * w.bandwidth + 1.0), est);
+    };
+    // steps of a band of this size that k_band left to the accumulator
+    if (series->general_n != n) {
+        series->general_z.clear();
+        series->general_baby.clear();
+        series->general_giant.clear();
+        series->general_n = n;
+    }
+    auto general_of = [](const std::vector<char>& v, size_t i) { return i < v.size() && v[i]; };
+    // (a step that k_product took for that reason stays with it)
+    auto note_general = [&](std::vector<char>& v, size_t i, const StepStat& rec) {
+        if (v.size() <= i) v.resize(i + 1, 0);
+        if (!mostly_runs(rec.general, n)) v[i] = 1;
     };
     w.chunk_cols = series->chunk_cols;
     w.chunk_slots = series->chunk_slots;
@@ -800,7 +825,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                         // or two for each run of them)
                         const int wz = window_of(span_z, words_z, (size_t)(i - 2), i, 0.35 * zlen * i * i);
                         if ((rc = run_step(w, &vz, &prev, {}, 0.0, 0.0, 1, w.front_stats() + (i - 2), (size_t)(i - 2),
-                                           &cur, slots + i, blen, zlen, 0, 0ull, 0.0, wz, 0.0, i)))
+                                           &cur, slots + i, blen, zlen, 0, 0ull, 0.0, wz, 0.0, i,
+                                           general_of(series->general_z, (size_t)(i - 2)))))
                             return rc;
                         if (i == 2) zsq = cur;
                         nr.rb[i - 1] = cur.rb;
@@ -836,6 +862,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     zfma[i] = zs[i - 2].fma;
                     series->len_z[(size_t)(i - 2)] = znnz[i - 1] / n;
                     sz[(size_t)(i - 2)] = zs[i - 2].span_max;
+                    note_general(series->general_z, (size_t)(i - 2), zs[i - 2]);
                 }
                 std::vector<unsigned> sw(9, 0u);
                 for (int i = 2; i <= 10; ++i) sw[(size_t)(i - 2)] = zs[i - 2].words_max;
@@ -945,7 +972,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                 int wb = window_of(span_baby, words_baby, (size_t)(k - 1), eb, z_words10 * eb / 10.0);
                 if (rk && wb == kLists) wb = kWide;  // (mostly skipped: no launch over B for it)
                 if ((rc = run_step(w, &vm, &Zh[(size_t)k], {}, thr, series->e_r, series->maxit, pstat + si, slot++,
-                                   &Zh[(size_t)k + 1], nullptr, blen, pow_len(1), rk, rk ? zfma[rk] : 0ull, 0.0, wb)))
+                                   &Zh[(size_t)k + 1], nullptr, blen, pow_len(1), rk, rk ? zfma[rk] : 0ull, 0.0, wb, 0.0, 0,
+                                   general_of(series->general_baby, (size_t)(k - 1)))))
                     return rc;
                 psf_step_info_t s{};
                 s.kind = 0;
@@ -1015,7 +1043,8 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     const double fh =
                         (size_t)(i - 1) < series->fma_giant.size() ? series->fma_giant[(size_t)(i - 1)] : 0.0;
                     if ((rc = run_step(w, &Zh[(size_t)q], &S, add, thr, series->e_r, series->maxit, pstat + si, sslot[nslot],
-                                       &nxt, nullptr, blen, alen, 0, 0ull, olen, wg, fh)))
+                                       &nxt, nullptr, blen, alen, 0, 0ull, olen, wg, fh, 0,
+                                       general_of(series->general_giant, (size_t)(i - 1)))))
                         return rc;
                     s.kind = 1;
                     s.threshold = thr;
@@ -1083,6 +1112,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     series->len_baby[(size_t)(k - 1)] = prev_len;
                     sb[(size_t)(k - 1)] = ss[idx].span_max;
                     wsb[(size_t)(k - 1)] = ss[idx].words_max;
+                    note_general(series->general_baby, (size_t)(k - 1), ss[idx]);
                     prev_len = (double)steps[idx].nnz_post / n;
                 }
                 double s_len = 0.0;
@@ -1091,6 +1121,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     series->len_giant[(size_t)(i - 1)] = s_len;
                     sg[(size_t)(i - 1)] = ss[idx].span_max;
                     wsg[(size_t)(i - 1)] = ss[idx].words_max;
+                    note_general(series->general_giant, (size_t)(i - 1), ss[idx]);
                     series->out_giant[(size_t)(i - 1)] = (double)steps[idx].nnz_pre / n;
                     series->fma_giant[(size_t)(i - 1)] = (double)steps[idx].fma;
                     s_len = (double)steps[idx].nnz_post / n;

@@ -196,6 +196,19 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         if ((rc = read_back(w, c))) return rc;
         if (c.status & kDevBadInput) return fail(PSF_EINVAL, "a batch input is malformed (row pointers, column order "
                                                             "or range, or non-finite value)");
+        if (c.apart) {
+            // runs of columns whose products are not
+            DevBuf d_apart;
+            std::vector<unsigned> apart((size_t)count);
+            CU(d_apart.alloc(sizeof(unsigned) * (size_t)count, st));
+            CU(cudaMemsetAsync(d_apart.p, 0, sizeof(unsigned) * (size_t)count, st));
+            CU(launch_count_apart_batch(n, inst, dsrc, d_apart.as<unsigned>(), st));
+            CU(cudaMemcpyAsync(apart.data(), d_apart.p, sizeof(unsigned) * (size_t)count, cudaMemcpyDeviceToHost, st));
+            CU(cudaStreamSynchronize(st));
+            for (int i = 0; i < count; ++i)
+                if (!mostly_runs(apart[(size_t)i], Zs[i].n)) isband[(size_t)i] = 0;
+            CU(cudaMemcpyAsync(d_isband.p, isband.data(), (size_t)count, cudaMemcpyHostToDevice, st));
+        }
     }
     // the instances whose rows k_band computes (the chunked and forced slot maps
     // are for tests of the accumulator)

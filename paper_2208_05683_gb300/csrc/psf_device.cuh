@@ -49,6 +49,8 @@ struct Ctl {
     unsigned pad4;
     unsigned bandwidth;  // of the checked inputs: max |column - row|
     int not_band;  // an input has a row that does not span consecutive columns
+    int apart;     // ... a row that does not meet the one before it, or far from the diagonal
+    unsigned apart_rows;  // rows that k_count_apart counted
     unsigned done;    // blocks of the running launch that have finished (0 between launches)
     unsigned ticket;  // k_band's tile counter (0 between launches)
     unsigned long long fma_total;  // algorithmic multiply-adds of all products
@@ -64,7 +66,7 @@ struct StepStat {
     int iters;
     unsigned span_max;  // widest column window of the product's rows (hi - lo + 1)
     unsigned words_max; // most 32-column words that one of its rows has entries in
-    unsigned pad;
+    unsigned general;   // rows that k_band left to the accumulator
 };
 
 // Per-matrix norm slot for the exact 1-norm kernel.

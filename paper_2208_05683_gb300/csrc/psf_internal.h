@@ -44,6 +44,10 @@ struct psf_series_s {
     // list map is used for wide windows of few words)
     std::vector<unsigned> words_z, words_baby, words_giant;
     std::mutex span_mu;
+    // steps whose rows k_band mostly left to the accumulator (the filter cuts
+    // a band to pieces), on matrices of general_n rows: k_product takes them
+    std::vector<char> general_z, general_baby, general_giant;
+    int general_n = -1;
     int kernel = 0;       // PSF_PARAM_KERNEL
     int chunk_cols = 0;   // PSF_PARAM_CHUNK_COLS
     int chunk_slots = 0;  // PSF_PARAM_CHUNK_SLOTS
@@ -177,7 +181,7 @@ struct Work {
     unsigned long long cap = 0, ccap = 0, bits_cap = 0;
     static constexpr size_t kRowsChunk = 8;  // matrices' row arrays allocated at a time
     std::vector<DevBuf*> rows;  // per matrix: n row descriptors, then rb and re (n ints each)
-    bool band = false;           // every input row spans consecutive columns: k_band computes the products
+    bool band = false;           // input rows are runs of columns whose products are runs: k_band computes them
     int slot_map = 0;            // 0 auto (by products per row), 1 table, 2 bitmap, 3 wide window, 4 CTA per row
     int chunk_cols = 0, chunk_slots = 0;
 
@@ -327,6 +331,13 @@ inline bool use_cta(int n, double alen, double blen) {
     (void)alen;
     return n > 0 && n <= 7 * num_sms() && blen >= 16.0;
 }
+
+// k_band against k_product: more than one row in kGeneralShare that it would
+// leave to the accumulator (its narrow map, three or more warps of a shared
+// tile waiting) and k_product, with its windows, row bitmaps and the row per
+// block, takes the step
+constexpr unsigned kGeneralShare = 8;
+inline bool mostly_runs(unsigned long long general, int n) { return general * kGeneralShare <= (unsigned long long)n; }
 
 // A step's column window: the bitmap map's own, its wide one, or the list map
 // (wide, and its rows have entries in few words).  span, words: the widest

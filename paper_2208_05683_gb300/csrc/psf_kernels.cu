@@ -2079,8 +2079,10 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
     __shared__ long long s_base;
     __shared__ int s_lo[R], s_hi[R], s_nnz[R], s_ok;
     __shared__ unsigned s_sum[R];
+    __shared__ int s_late;  // the block's rows left to the accumulator
     const int nadd = P.nadd;
     for (int t = threadIdx.x; t < nadd; t += blockDim.x) add[t] = P.add[t];
+    if (threadIdx.x == 0) s_late = 0;
     __syncthreads();
     auto sync = [] {
         if constexpr (TEAM) __syncthreads();
@@ -2447,6 +2449,7 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
         }
         if (late) {
             sync();
+            if (!BATCH && lead && lane == 0) atomicAdd(&s_late, __popc(late));
             if (lead)
                 while (late) {
                     const int i = __ffs(late) - 1;
@@ -2494,6 +2497,7 @@ __global__ void __launch_bounds__(kBandWarps * 32, 7) k_band(const __grid_consta
         if (blk_fma) atomicAdd(&P.ctl->fma_total, blk_fma);
         if (P.stat) {
             if (blk_span > 0) atomicMax(&P.stat->span_max, (unsigned)blk_span);
+            if (s_late > 0) atomicAdd(&P.stat->general, (unsigned)s_late);
             if (blk_fma) atomicAdd(&P.stat->fma, blk_fma);
             if (blk_written) atomicAdd(&P.stat->nnz_pre, blk_written);
             if (blk_cand) atomicAdd(&P.stat->ncand, blk_cand);
@@ -3717,6 +3721,48 @@ __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot
     if (lane == 0 && mx) atomicMax(&slot->absmax, mx);
 }
 
+// Where the rows of B are runs of consecutive columns, a row of A B is one too
+// if the B rows that it takes meet one another (share a column, or lie side by
+// side), and a sum of powers of Z is if they lie about the diagonal.  Bands do;
+// runs at unrelated places (permuted blocks, gathers) don't, and k_band would
+// leave every row of their products to the accumulator's narrow map.
+// Row r of length len, columns [first, last], is further from the diagonal
+// than it is long.
+__device__ __forceinline__ bool far_from_diagonal(int r, int first, int last, int len) {
+    return max(first - r, r - last) > len + 1;
+}
+// Row k of a checked matrix (0 < k < n) does not meet row k - 1.
+__device__ __forceinline__ bool row_apart(const int* rowptr, const int* col, int k) {
+    const int s0 = rowptr[k - 1], s = rowptr[k], e = rowptr[k + 1];
+    return s0 < s && s < e && (col[s] - 1 > col[s - 1] || col[e - 1] + 1 < col[s0]);
+}
+// Row r of A takes rows of B that do not meet, or (series) is far from the diagonal.
+__device__ __forceinline__ bool row_falls_apart(const int* a_rp, const int* a_col, const int* b_rp, const int* b_col,
+                                                int r, bool series) {
+    const int s = a_rp[r], e = a_rp[r + 1];
+    if (s >= e) return false;
+    if (series && far_from_diagonal(r, a_col[s], a_col[e - 1], e - s)) return true;
+    for (int q = s + 1; q < e; ++q)
+        if (row_apart(b_rp, b_col, a_col[q])) return true;
+    return false;
+}
+// How many rows do (a second look, after k_validate or k_validate_batch has
+// seen a row apart or far from the diagonal: about 10 us that bands don't pay).
+__global__ void k_count_apart(int n, const int* a_rp, const int* a_col, const int* b_rp, const int* b_col, int series,
+                              Ctl* ctl) {
+    pdl_enter();
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = warp_sum(r < n && row_falls_apart(a_rp, a_col, b_rp, b_col, r, series != 0) ? 1 : 0);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&ctl->apart_rows, (unsigned)c);
+}
+__global__ void k_count_apart_batch(int n, const int* inst, const BatchSrc* src, unsigned* count) {
+    pdl_enter();
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n) return;
+    const BatchSrc S = src[inst[r]];
+    if (row_falls_apart(S.rowptr, S.col, S.rowptr, S.col, r - S.off, true)) atomicAdd(count + inst[r], 1u);
+}
+
 // Check a canonical CSR input: row pointers non-decreasing from 0 to nnz,
 // columns in range and strictly increasing per row, values finite.
 __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, const double* val,
@@ -3746,7 +3792,13 @@ __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, co
                 prev = c;
             }
             if (e > s && prev - col[s] != e - s - 1) ctl->not_band = 1;
-            if (e > s && !bad) bw = max(prev - r, r - col[s]);
+            if (e > s && !bad) {
+                bw = max(prev - r, r - col[s]);
+                bool apart = far_from_diagonal(r, col[s], prev, e - s);
+                const int s0 = r > 0 ? rowptr[r - 1] : s;  // (the row before may not have passed)
+                if (s0 >= 0 && s0 < s) apart = apart || col[s] - 1 > col[s - 1] || prev + 1 < col[s0];
+                if (apart) ctl->apart = 1;
+            }
         }
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
@@ -3981,6 +4033,12 @@ __global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, co
             prev = c;
         }
         if (e > s && prev - S.col[s] != e - s - 1) band[i] = 0;
+        if (e > s && !bad) {
+            bool apart = far_from_diagonal(l, S.col[s], prev, e - s);
+            const int s0 = l > 0 ? S.rowptr[l - 1] : s;
+            if (s0 >= 0 && s0 < s) apart = apart || S.col[s] - 1 > S.col[s - 1] || prev + 1 < S.col[s0];
+            if (apart) ctl->apart = 1;
+        }
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
 }
@@ -4489,6 +4547,21 @@ cudaError_t launch_alg1_batch(const Alg1BatchArgs& A, cudaStream_t st) {
 cudaError_t launch_inst_table(int n, int ninst, const int* off, int* inst, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     launch_pdl(k_inst_table, (n + 255) / 256, 256, 0, st, n, ninst, off, inst);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_apart(const psf_csr_t& A, const psf_csr_t& B, bool series, Ctl* ctl, cudaStream_t st) {
+    if (A.n <= 0) return cudaSuccess;
+    launch_pdl(k_count_apart, (unsigned)((A.n + 255) / 256), 256, 0, st, A.n, A.rowptr, A.col, B.rowptr, B.col,
+               series ? 1 : 0, ctl);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_apart_batch(int n, const int* inst, const BatchSrc* src, unsigned* count, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    launch_pdl(k_count_apart_batch, (unsigned)((n + 255) / 256), 256, 0, st, n, inst, src, count);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -57,6 +57,11 @@ cudaError_t launch_norms(const NormArgs& A, cudaStream_t st);
 cudaError_t launch_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot* slot, cudaStream_t st);
 cudaError_t launch_validate(int n, int nnz, const int* rowptr, const int* col, const double* val, Ctl* ctl,
                             cudaStream_t st);
+// rows of A whose product row with B falls apart (k_count_apart), into
+// ctl->apart_rows; series: also those far from the diagonal.  Both matrices
+// are checked.  A batch: per instance, into count
+cudaError_t launch_count_apart(const psf_csr_t& A, const psf_csr_t& B, bool series, Ctl* ctl, cudaStream_t st);
+cudaError_t launch_count_apart_batch(int n, const int* inst, const BatchSrc* src, unsigned* count, cudaStream_t st);
 size_t scan_scratch_len(int n);  // long longs of scratch launch_scan_rows needs
 // (rd: the rows' true entries instead of re - rb)
 cudaError_t launch_scan_rows(int n, const int* rb, const int* re, const RowDesc* rd, int* rowptr, Ctl* ctl,
