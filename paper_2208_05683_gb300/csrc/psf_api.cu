@@ -739,13 +739,15 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
         words_baby = series->words_baby;
         words_giant = series->words_giant;
     }
+    // what e applications of Z reach from one column: no row of a step is longer
+    auto reach_of = [&](double e) { return std::min((double)n, 2.0 * e * w.bandwidth + 1.0); };
     // the window of a step: by its record (of a matrix that may have been a
     // larger one: no row spans more than n), or what e applications of Z reach
     // from a row with `words` words
     auto window_of = [&](const std::vector<unsigned>& span, const std::vector<unsigned>& words, size_t i, double e,
                          double est) {
         if (i < span.size()) return window_for(std::min((double)n, (double)span[i]), i < words.size() ? (double)words[i] : 0.0);
-        return window_for(std::min((double)n, 2.0 * e * w.bandwidth + 1.0), est);
+        return window_for(reach_of(e), est);
     };
     // steps of a band of this size that k_band left to the accumulator
     if (series->general_n != n) {
@@ -820,7 +822,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     for (int i = 2; i <= 10; ++i) {
                         RowView cur;
                         double blen = (size_t)(i - 2) < series->len_z.size() ? series->len_z[(size_t)(i - 2)]
-                                                                              : zlen * (i - 1) * (i - 1);
+                                                                              : std::min(zlen * (i - 1) * (i - 1), reach_of(i - 1));
                         // (a first evaluation: entries of about half a square's growth, a word
                         // or two for each run of them)
                         const int wz = window_of(span_z, words_z, (size_t)(i - 2), i, 0.35 * zlen * i * i);
@@ -903,7 +905,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     // mean row length of the k-th power of the matrix the scheme multiplies by
     auto pow_len = [&](int k) {
         const int e = k * stride;
-        return (e <= 10 && znnz[e] > 0.0) ? znnz[e] / n : zlen * e * e;
+        return (e <= 10 && znnz[e] > 0.0) ? znnz[e] / n : std::min(zlen * e * e, reach_of(e));
     };
     if ((N == 1 && !odd) || n == 0) {
         // f(Z) ~ a_0 I: no product (Eq. 5)
@@ -1034,7 +1036,7 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
                     double thr = nofilter ? 0.0 : p.sigma[(size_t)i];
                     double blen = (size_t)(i - 1) < series->len_giant.size()
                                       ? series->len_giant[(size_t)(i - 1)]
-                                      : (znnz[10] > 0.0 ? znnz[10] / n : zlen * 100.0);
+                                      : std::min(znnz[10] > 0.0 ? znnz[10] / n : zlen * 100.0, reach_of((double)stride * q * i));
                     const double alen = pow_len(q);
                     const double olen =
                         (size_t)(i - 1) < series->out_giant.size() ? series->out_giant[(size_t)(i - 1)] : 0.0;
