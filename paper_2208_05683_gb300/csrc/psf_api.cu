@@ -282,7 +282,7 @@ int run_step(Work& w, const RowView* A, const RowView* B, const std::vector<AddT
     if (dense) {
         const size_t bytes = sizeof(double) * (size_t)w.n * (size_t)w.n;
         for (DevBuf& d : w.dense)
-            if (!d.p) CU(d.alloc(bytes, w.st));
+            if (!d.p) CU(w.take(d, bytes));
         CU(launch_dense_product(P, w.dense[0].as<double>(), w.dense[1].as<double>(), w.dense[2].as<double>(), w.st));
     } else {
         // the bitmap map marks B rows from their column bitmaps (built here,
@@ -387,7 +387,7 @@ int make_result(Work& w, const RowView& M, psf_result_t* out, psf_result_s** mad
     r->stream = w.st;
     int rc = PSF_OK;
     do {
-        cudaError_t e = cudaMallocAsync((void**)&r->rowptr, sizeof(int) * ((size_t)w.n + 1), w.st);
+        cudaError_t e = w.take((void**)&r->rowptr, sizeof(int) * ((size_t)w.n + 1));
         if (e != cudaSuccess) {
             rc = fail(PSF_ENOMEM, "result rowptr: %s", cudaGetErrorString(e));
             break;
@@ -416,8 +416,8 @@ int make_result(Work& w, const RowView& M, psf_result_t* out, psf_result_s** mad
 int finish_result(Work& w, const RowView& M, psf_result_s* r, unsigned long long nnz) {
     if (nnz > (unsigned long long)INT32_MAX) return fail(PSF_ETOOBIG, "result has %llu entries (>= 2^31)", nnz);
     r->nnz = (long long)nnz;
-    CU(cudaMallocAsync((void**)&r->col, sizeof(int) * (nnz ? nnz : 1), w.st));
-    CU(cudaMallocAsync((void**)&r->val, sizeof(double) * (nnz ? nnz : 1), w.st));
+    CU(w.take((void**)&r->col, sizeof(int) * (nnz ? nnz : 1)));
+    CU(w.take((void**)&r->val, sizeof(double) * (nnz ? nnz : 1)));
     if (w.n > 0 && nnz) CU(launch_gather(w.n, M, r->rowptr, r->col, r->val, w.st));
     r->info.nnz = (int64_t)nnz;
     return PSF_OK;

@@ -97,7 +97,9 @@ struct DevBuf {
         release();
         st = s;
         if (bytes == 0) bytes = 16;
-        return cudaMallocAsync(&p, bytes, s);
+        const cudaError_t e = cudaMallocAsync(&p, bytes, s);
+        if (e != cudaSuccess) p = nullptr;
+        return e;
     }
     void release() {
         if (p) cudaFreeAsync(p, st);
@@ -175,6 +177,7 @@ struct Work {
     DevBuf bhdr, pool_bits;  // column bitmaps of a product's B rows: n headers, a word per pool entry
     DevBuf pool_lists;       // the list map's form: a pair per pool entry, allocated on first use
     unsigned long long lists_cap = 0;
+    bool no_lists = false;   // there was no memory for them in this call
     int bandwidth = 0;       // of the checked inputs
     double dense_xover = 1e300;  // dense tiles for a step with at least this many multiply-adds per n^3
     bool dense_estimate = false;  // a step without a recorded count may use the row-length estimate
@@ -231,7 +234,7 @@ struct Work {
             *out = front_stats() + 16;
             if (!again) return PSF_OK;
         } else {
-            if (!again) CU(more_stats.alloc(sizeof(StepStat) * (size_t)count, st));
+            if (!again) CU(take(more_stats, sizeof(StepStat) * (size_t)count));
             *out = more_stats.as<StepStat>();
         }
         CU(cudaMemsetAsync(*out, 0, sizeof(StepStat) * (size_t)count, st));
@@ -241,35 +244,55 @@ struct Work {
     int reset_pool(unsigned long long entries) {
         if (entries > kMaxPool) return fail(PSF_ETOOBIG, "pool of %llu entries exceeds 2^31 - 2^20", entries);
         if (entries > cap) {
-            CU(pool_col.alloc(sizeof(int) * entries, st));
-            CU(pool_val.alloc(sizeof(double) * entries, st));
+            CU(take(pool_col, sizeof(int) * entries));
+            CU(take(pool_val, sizeof(double) * entries));
             cap = entries;
             // two Algorithm 1 candidate lists of half the pool each (a step
             // whose candidates do not fit falls back to full scans)
             ccap = cap / 2 > 1024 ? cap / 2 : 1024;
-            CU(cand_col.alloc(sizeof(int) * 2 * ccap, st));
-            CU(cand_x.alloc(sizeof(unsigned long long) * 2 * ccap, st));
+            CU(take(cand_col, sizeof(int) * 2 * ccap));
+            CU(take(cand_x, sizeof(unsigned long long) * 2 * ccap));
         }
         if (g_row_bitmaps.load() > 0 && bits_cap < cap) {
-            CU(pool_bits.alloc(sizeof(unsigned) * cap, st));
+            CU(take(pool_bits, sizeof(unsigned) * cap));
             bits_cap = cap;
         }
         CU(launch_reset(C(), cap, ccap, cand_chunk(), st));
         return PSF_OK;
     }
     // the lists' memory; null where there is none left (the step then takes the
-    // wide bitmap window, which needs none)
+    // wide bitmap window, which needs none).  It is a convenience: whatever
+    // else the call allocates later may have it (take), a larger pool and the
+    // result among them.
     uint2* lists() {
-        if (lists_cap < cap) {
+        if (lists_cap < cap && !no_lists) {
             lists_cap = 0;
-            if (pool_lists.alloc(sizeof(uint2) * cap, st) != cudaSuccess) {
-                pool_lists.p = nullptr;
+            if (pool_lists.alloc(sizeof(uint2) * cap, st) == cudaSuccess) {
+                lists_cap = cap;
+            } else {
                 cudaGetLastError();
-                return nullptr;
+                no_lists = true;
             }
-            lists_cap = cap;
         }
-        return pool_lists.as<uint2>();
+        return lists_cap >= cap ? pool_lists.as<uint2>() : nullptr;
+    }
+    // bytes of device memory, the lists' if there is no other
+    cudaError_t take(void** p, size_t bytes) {
+        cudaError_t e = cudaMallocAsync(p, bytes, st);
+        if (e == cudaErrorMemoryAllocation && pool_lists.p) {
+            cudaGetLastError();
+            pool_lists.release();
+            lists_cap = 0;
+            no_lists = true;
+            e = cudaMallocAsync(p, bytes, st);
+        }
+        if (e != cudaSuccess) *p = nullptr;
+        return e;
+    }
+    cudaError_t take(DevBuf& b, size_t bytes) {
+        b.release();
+        b.st = st;
+        return take(&b.p, bytes > 0 ? bytes : 16);
     }
     // Entries a warp reserves in a candidate list at a time: up to 128, so
     // that about 12k warps' unused chunk ends take at most a quarter of it.
@@ -289,7 +312,7 @@ struct Work {
         const size_t c = i / kRowsChunk, nn = ((size_t)(n > 0 ? n : 1) + 3) & ~(size_t)3;
         while (rows.size() <= c) rows.push_back(new DevBuf());
         const size_t each = (sizeof(RowDesc) + 2 * sizeof(int)) * nn;
-        if (!rows[c]->p) CU(rows[c]->alloc(each * kRowsChunk, st));
+        if (!rows[c]->p) CU(take(*rows[c], each * kRowsChunk));
         out->rd = reinterpret_cast<RowDesc*>(rows[c]->as<char>() + each * (i % kRowsChunk));
         out->rb = reinterpret_cast<int*>(out->rd + nn);
         out->re = out->rb + nn;
