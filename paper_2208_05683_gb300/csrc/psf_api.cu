@@ -742,12 +742,12 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     // what e applications of Z reach from one column: no row of a step is longer
     auto reach_of = [&](double e) { return std::min((double)n, 2.0 * e * w.bandwidth + 1.0); };
     // the window of a step: by its record (of a matrix that may have been a
-    // larger one: no row spans more than n), or what e applications of Z reach
-    // from a row with `words` words
+    // larger one: no row spans more than n), or what e applications of Z reach;
+    // est: words of a row where none were recorded (a batch, k_band)
     auto window_of = [&](const std::vector<unsigned>& span, const std::vector<unsigned>& words, size_t i, double e,
                          double est) {
-        if (i < span.size()) return window_for(std::min((double)n, (double)span[i]), i < words.size() ? (double)words[i] : 0.0);
-        return window_for(reach_of(e), est);
+        const double known = i < words.size() && words[i] > 0 ? (double)words[i] : est;
+        return i < span.size() ? window_for(std::min((double)n, (double)span[i]), known) : window_for(reach_of(e), est);
     };
     // steps of a band of this size that k_band left to the accumulator
     if (series->general_n != n) {

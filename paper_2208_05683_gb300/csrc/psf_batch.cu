@@ -887,9 +887,14 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
                 if (D.kind == 1 && D.index - 1 >= 0 && (size_t)(D.index - 1) < sg.size()) sg[(size_t)(D.index - 1)] = sp;
             }
             std::lock_guard<std::mutex> lock(series[i]->span_mu);
-            if (chain[(size_t)i]) series[i]->span_z = sz;
+            if (chain[(size_t)i]) {
+                series[i]->span_z = sz;
+                series[i]->words_z.clear();  // (of another evaluation: not counted here)
+            }
             series[i]->span_baby = sb;
             series[i]->span_giant = sg;
+            series[i]->words_baby.clear();
+            series[i]->words_giant.clear();
         }
         psf_info_t& inf = r->info;
         inf.N = p.N;

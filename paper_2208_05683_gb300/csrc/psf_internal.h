@@ -41,7 +41,8 @@ struct psf_series_s {
     // concurrently on one series, read and write them under span_mu
     std::vector<unsigned> span_z, span_baby, span_giant;
     // most words of 32 columns that one of a step's rows has entries in (the
-    // list map is used for wide windows of few words)
+    // list map is used for wide windows of few words), of the evaluation that
+    // recorded the spans; 0 or none: not counted
     std::vector<unsigned> words_z, words_baby, words_giant;
     std::mutex span_mu;
     // steps whose rows k_band mostly left to the accumulator (the filter cuts

@@ -38,3 +38,21 @@ def test_list_steps_then_a_small_matrix_bitwise(small):
     s = psf.Series(a, tol)
     for k in (0, 0, 1, 1, 0):
         check_same(s.eval(dev((large, little)[k])), refs[k], f"{small} {k}")
+
+
+def test_a_batch_between_evaluations_bitwise():
+    # a batch records its windows and no words: the next evaluation must not
+    # pair them with an older matrix's
+    a, tol = syn.coeffs("exp"), 1e-8
+    rng = np.random.default_rng(4)
+    n = 9001
+    c = np.sort(rng.integers(0, n, (n, 3)), axis=1)
+    c += np.arange(3)  # distinct
+    c = np.minimum(c, n - 3 + np.arange(3)).astype(np.int32)
+    many = CSR(n, (3 * np.arange(n + 1)).astype(np.int32), c.reshape(-1), rng.uniform(-0.05, 0.05, 3 * n))
+    Zs = [grid(9, 700, 2.0, 1), many, grid(60, 160, 2.0, 3)]
+    s = psf.Series(a, tol, submult=True)
+    refs = [psscf(Z, a, tol, submult=True) for Z in Zs]
+    for k, batch in ((0, False), (1, True), (0, False), (1, False), (0, True), (1, False), (2, True), (0, False)):
+        got = psf.eval_batch([s], [dev(Zs[k])])[0] if batch else s.eval(dev(Zs[k]))
+        check_same(got, refs[k], f"{k} {batch}")
