@@ -65,6 +65,11 @@ struct BatchStorage {
 // pools of tens of GB).
 std::atomic<double> g_z_per_row{0.0}, g_ps_per_row{0.0};
 double pool_rows(int n) { return std::max((double)n, 28.0 * num_sms()); }
+// and the most rows (of that kind) that taught it: a batch of more than twice
+// as many is sized as a first one is, by its own entries too.  (Learnt from 600
+// rows of 81 entries alone, the pools of a batch of 60000 rows of 41 overflowed
+// and both phases ran twice: 41.9 ms, now 24.2.)
+std::atomic<double> g_rows_learnt{0.0};
 
 void raise_to(std::atomic<double>& a, double v) {
     double cur = a.load();
@@ -226,6 +231,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         d_band = d_isband.as<unsigned char>();
     else
         any_general = true;
+    const bool unlearnt = pool_rows(n) > 2.0 * g_rows_learnt.load();
     const double zlen_all = n > 0 ? (double)nnz_tot / n : 0.0;
     const unsigned long long arena_z = arena_for(zlen_all > 0.0 ? zlen_all : 1.0);
 
@@ -261,7 +267,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
         unsigned long long zcap = (unsigned long long)(g_z_per_row.load() * 1.25 * pool_rows(n)) + 4096ull;
         unsigned long long est = (unsigned long long)nnz_tot * (any_chain ? 128ull : 2ull) + (unsigned long long)n * 8ull +
                                  4096ull * 64ull;
-        if (g_z_per_row.load() == 0.0 && zcap < est) zcap = est;
+        if (unlearnt && zcap < est) zcap = est;
         if (zcap > kMaxPool) zcap = kMaxPool;
         for (int attempt = 0;; ++attempt) {
             CU(cudaMemsetAsync(slots, 0, sizeof(NormSlot) * kMaxNorms * (size_t)count, st));
@@ -594,7 +600,7 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
     {
         unsigned long long est = (unsigned long long)nnz_tot * 64ull + (unsigned long long)n * 64ull + 4096ull * 64ull;
         for (int i = 0; i < count; ++i) est += (unsigned long long)(4.0 * ip[(size_t)i].znnz[10]);
-        if (g_ps_per_row.load() == 0.0 && cap < est) cap = est;
+        if (unlearnt && cap < est) cap = est;
         if (cap > kMaxPool) cap = kMaxPool;
     }
     DevBuf d_rowptr, d_bounds;
@@ -813,7 +819,10 @@ int eval_group(const psf_series_t* series, const psf_csr_t* Zs, int count, cudaS
             if (cap > kMaxPool) cap = kMaxPool;
             continue;
         }
-        if (n > 0) raise_to(g_ps_per_row, (double)cfin.pool_used / pool_rows(n));
+        if (n > 0) {
+            raise_to(g_ps_per_row, (double)cfin.pool_used / pool_rows(n));
+            raise_to(g_rows_learnt, pool_rows(n));
+        }
         break;
     }
     const unsigned long long nnz_out = cfin.nnz_total;
