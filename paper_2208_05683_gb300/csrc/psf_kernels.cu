@@ -3733,10 +3733,11 @@ __global__ void k_absmax(const double* pool_val, const Ctl* ctl, int i, NormSlot
 // side), and a sum of powers of Z is if they lie about the diagonal.  Bands do;
 // runs at unrelated places (permuted blocks, gathers) don't, and k_band would
 // leave every row of their products to the accumulator's narrow map.
-// Row r of length len, columns [first, last], is further from the diagonal
-// than it is long.
-__device__ __forceinline__ bool far_from_diagonal(int r, int first, int last, int len) {
-    return max(first - r, r - last) > len + 1;
+// Row r of length len, columns [first, last] of [0, n), is further from the
+// diagonal than it is long (and not the rest of one that the edge cuts off).
+__device__ __forceinline__ bool far_from_diagonal(int n, int r, int first, int last, int len) {
+    const int gap = max(first - r, r - last);
+    return gap > len + 1 && ((first > 0 && last < n - 1) || gap > 512);
 }
 // Row k of a checked matrix (0 < k < n) does not meet row k - 1.
 __device__ __forceinline__ bool row_apart(const int* rowptr, const int* col, int k) {
@@ -3744,11 +3745,11 @@ __device__ __forceinline__ bool row_apart(const int* rowptr, const int* col, int
     return s0 < s && s < e && (col[s] - 1 > col[s - 1] || col[e - 1] + 1 < col[s0]);
 }
 // Row r of A takes rows of B that do not meet, or (series) is far from the diagonal.
-__device__ __forceinline__ bool row_falls_apart(const int* a_rp, const int* a_col, const int* b_rp, const int* b_col,
-                                                int r, bool series) {
+__device__ __forceinline__ bool row_falls_apart(int n, const int* a_rp, const int* a_col, const int* b_rp,
+                                                const int* b_col, int r, bool series) {
     const int s = a_rp[r], e = a_rp[r + 1];
     if (s >= e) return false;
-    if (series && far_from_diagonal(r, a_col[s], a_col[e - 1], e - s)) return true;
+    if (series && far_from_diagonal(n, r, a_col[s], a_col[e - 1], e - s)) return true;
     for (int q = s + 1; q < e; ++q)
         if (row_apart(b_rp, b_col, a_col[q])) return true;
     return false;
@@ -3759,7 +3760,7 @@ __global__ void k_count_apart(int n, const int* a_rp, const int* a_col, const in
                               Ctl* ctl) {
     pdl_enter();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const int c = warp_sum(r < n && row_falls_apart(a_rp, a_col, b_rp, b_col, r, series != 0) ? 1 : 0);
+    const int c = warp_sum(r < n && row_falls_apart(n, a_rp, a_col, b_rp, b_col, r, series != 0) ? 1 : 0);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(&ctl->apart_rows, (unsigned)c);
 }
 __global__ void k_count_apart_batch(int n, const int* inst, const BatchSrc* src, unsigned* count) {
@@ -3767,7 +3768,7 @@ __global__ void k_count_apart_batch(int n, const int* inst, const BatchSrc* src,
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const BatchSrc S = src[inst[r]];
-    if (row_falls_apart(S.rowptr, S.col, S.rowptr, S.col, r - S.off, true)) atomicAdd(count + inst[r], 1u);
+    if (row_falls_apart(S.n, S.rowptr, S.col, S.rowptr, S.col, r - S.off, true)) atomicAdd(count + inst[r], 1u);
 }
 
 // Check a canonical CSR input: row pointers non-decreasing from 0 to nnz,
@@ -3776,7 +3777,7 @@ __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, co
                            Ctl* ctl) {
     pdl_enter();
     int r = blockIdx.x * blockDim.x + threadIdx.x;
-    bool bad = false;
+    bool bad = false, holes = false, apart = false;
     int bw = 0;
     if (r > n) {
     } else if (r == n) {
@@ -3798,19 +3799,24 @@ __global__ void k_validate(int n, int nnz, const int* rowptr, const int* col, co
                 }
                 prev = c;
             }
-            if (e > s && prev - col[s] != e - s - 1) ctl->not_band = 1;
             if (e > s && !bad) {
                 bw = max(prev - r, r - col[s]);
-                bool apart = far_from_diagonal(r, col[s], prev, e - s);
+                holes = prev - col[s] != e - s - 1;
+                apart = far_from_diagonal(n, r, col[s], prev, e - s);
                 const int s0 = r > 0 ? rowptr[r - 1] : s;  // (the row before may not have passed)
                 if (s0 >= 0 && s0 < s) apart = apart || col[s] - 1 > col[s - 1] || prev + 1 < col[s0];
-                if (apart) ctl->apart = 1;
             }
         }
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
+    // (one store a warp)
     bw = warp_max(bw);
-    if ((threadIdx.x & 31) == 0 && bw > 0) atomicMax(&ctl->bandwidth, (unsigned)bw);
+    const unsigned any_holes = __ballot_sync(kFull, holes), any_apart = __ballot_sync(kFull, apart && !holes);
+    if ((threadIdx.x & 31) == 0) {
+        if (bw > 0) atomicMax(&ctl->bandwidth, (unsigned)bw);
+        if (any_holes) ctl->not_band = 1;
+        if (any_apart) ctl->apart = 1;
+    }
 }
 
 // Exclusive scan of row lengths (re - rb, or a pooled matrix's true entries
@@ -4041,10 +4047,10 @@ __global__ void k_validate_batch(int n, const int* inst, const BatchSrc* src, co
         }
         if (e > s && prev - S.col[s] != e - s - 1) band[i] = 0;
         if (e > s && !bad) {
-            bool apart = far_from_diagonal(l, S.col[s], prev, e - s);
+            bool apart = far_from_diagonal(S.n, l, S.col[s], prev, e - s);
             const int s0 = l > 0 ? S.rowptr[l - 1] : s;
             if (s0 >= 0 && s0 < s) apart = apart || S.col[s] - 1 > S.col[s - 1] || prev + 1 < S.col[s0];
-            if (apart) ctl->apart = 1;
+            if (apart && prev - S.col[s] == e - s - 1 && __ldcg(&ctl->apart) == 0) ctl->apart = 1;
         }
     }
     if (bad) atomicOr(&ctl->status, kDevBadInput);
