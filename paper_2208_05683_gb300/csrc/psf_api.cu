@@ -741,6 +741,18 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     }
     // what e applications of Z reach from one column: no row of a step is longer
     auto reach_of = [&](double e) { return std::min((double)n, 2.0 * e * w.bandwidth + 1.0); };
+    const unsigned long long usual = (unsigned long long)Z->nnz * 256ull + (unsigned long long)n * 64ull + 4096ull;
+    // Entries of a pool without a record: a usual number, or what rows of at most
+    // per_row entries over all `launches` take (a band's are known: a third of
+    // the usual, and a pool that need not grow between the phases), as arenas
+    // leave up to half unused; and an arena that each resident warp may leave
+    // almost empty in each launch (rows of a few entries overflowed the pool of
+    // a few thousand rows once or twice).
+    auto guess_of = [&](unsigned long long entries, double per_row, int launches) {
+        const double most = 2.0 * per_row * n;
+        return (most < (double)entries ? (unsigned long long)most : entries) +
+               512ull * (unsigned long long)launches * (unsigned long long)std::min(n, 4 * 7 * num_sms());
+    };
     // the window of a step: by its record (of a matrix that may have been a
     // larger one: no row spans more than n), or what e applications of Z reach;
     // est: words of a row where none were recorded (a batch, k_band)
@@ -793,7 +805,10 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
     RowView zp{}, zsq{};  // the pooled Z and, when the chain ran, Z^2
     unsigned long long zfma[kMaxNorms] = {0ull};  // multiply-adds of Z^i in the norm phase
     {
-        unsigned long long est = (unsigned long long)Z->nnz * 256ull + (unsigned long long)n * 64ull + 4096ull;
+        // (without the powers only Z is here: the pool is the second phase's)
+        double per_row = chain ? zlen + 4.0 : 1e300;
+        for (int i = 2; i <= 10; ++i) per_row += reach_of(i) + 3.0;
+        const unsigned long long est = guess_of(usual, per_row, 10);
         if (series->z_need == 0 && zcap < est) zcap = est;
         if (zcap > kMaxPool) zcap = kMaxPool;
         for (int attempt = 0;; ++attempt) {
@@ -932,7 +947,12 @@ int psf_eval(psf_series_t series, const psf_csr_t* Z, void* stream, psf_result_t
         // ---- steps 4-14 in one pool
         unsigned long long cap = series->pool_hint;
         if (cap < series->ps_need + series->ps_need / 8) cap = series->ps_need + series->ps_need / 8;
-        unsigned long long est = 4ull * z_used + (unsigned long long)Z->nnz * 64ull + (unsigned long long)n * 64ull;
+        double per_row = zlen + 4.0 + (square ? reach_of(2) + 3.0 : 0.0);
+        for (int k = 2; k <= q; ++k) per_row += reach_of((double)stride * k) + 3.0;
+        for (int i = 0; i < b; ++i) per_row += reach_of((double)stride * q * (i + 1)) + 3.0;
+        if (odd) per_row += reach_of((double)stride * q * b + 1.0) + 3.0;
+        const unsigned long long after = 4ull * z_used + (unsigned long long)Z->nnz * 64ull + (unsigned long long)n * 64ull;
+        const unsigned long long est = chain ? guess_of(std::max(usual, after), per_row, q + b + 2) : after;
         if (series->ps_need == 0 && cap < est) cap = est;
         if (cap > kMaxPool) cap = kMaxPool;
         for (int attempt = 0;; ++attempt) {
