@@ -87,8 +87,8 @@ extern "C" {
                                      (auto picks it for a step whose rows spanned more than
                                      4608 columns in the series' previous evaluation; the list
                                      map instead where they have entries in few 32-column words;
-                                     and no slot map at all for inputs whose rows span
-                                     consecutive columns),
+                                     and no slot map at all for inputs whose rows, and
+                                     their products', are runs of consecutive columns),
                                      4 one row per block of four warps (shared bitmap map,
                                      2560 accumulator slots) for every product */
 #define PSF_PARAM_CHUNK_COLS 5    /* > 0: fewer columns per row chunk (tests of row chunking) */
@@ -305,7 +305,9 @@ PSF_API int psf_server_destroy(psf_server_t server);
  * for each k of A's row r in ascending column order c = fma(a_rk, b_kj, c).
  * Entries that are exactly 0 are not stored.  threshold > 0 runs Algorithm 1
  * with eps_g = threshold / (1 + e_r), so the dropped 1-norm is <= threshold;
- * threshold == 0 keeps every nonzero entry.  Synchronizes `stream` once.
+ * threshold == 0 keeps every nonzero entry.  Synchronizes `stream` twice
+ * (input check, result sizes), and once more where the rows of A and B are
+ * runs of consecutive columns at unrelated places.
  * Limits: nadd <= PSF_MAX_Q + 1.
  * Errors: PSF_EINVAL (malformed or mismatched matrices, nadd out of range,
  * a threshold that is negative or not finite),
@@ -447,8 +449,8 @@ PSF_API int psf_plan(const double* coeffs, int64_t m, int32_t s, double tol, uin
  * product.  With 1 and 2, a product of rows that span more columns than the
  * bitmap map covers, but have entries in few of their words, is marked from
  * lists of those words instead (two words per entry of the entry pool,
- * allocated by the first such product of a call; without memory for them it
- * takes the wide bitmap window).  Results are the same either way; with 0 a
+ * allocated by the first such product of a call and given up to whatever else
+ * the call allocates; without memory for them it takes the wide bitmap window).  Results are the same either way; with 0 a
  * call allocates no bitmap words. */
 #define PSF_TUNE_ROW_BITMAPS 8
 PSF_API int psf_tune_set(int32_t key, double value);

@@ -43,7 +43,7 @@ constexpr size_t kRowsS = 30;        // + (stage & 1): giant-step outputs
 constexpr size_t kRowsPow = 40;      // + k - 2: the norm phase's Z^k (k = 2..10)
 constexpr size_t kRowsW = 62;        // W = Z Z of the PSF_Z_SQUARE instances
 constexpr size_t kRowsLeft = 63;     // composite left factor of the baby steps: Z, or W
-constexpr int kMaxBatchRows = 1 << 24;  // column-sum words: 704 B per row
+constexpr int kMaxBatchRows = 1 << 24;  // column-sum words: 904 B per row
 
 // Device storage shared by the results of one batch.
 struct BatchStorage {

@@ -46,8 +46,15 @@ namespace psf {
 // (launch_pdl) a kernel is brought onto the SMs while the one before it runs;
 // it starts by waiting for that one's end (all of its blocks, and what they
 // wrote) and then lets the next one come.  Every kernel here does so first of
-// all, so that whatever ran two launches earlier has ended too.  A launch
-// that is no such kernel's neighbour behaves as an ordinary one.
+// all, so that whatever ran two launches earlier has ended too, with one
+// exception: k_band in a batch's paired step lets the next one come at once and
+// waits in its last lines.  It may read what earlier steps wrote because the
+// launch just before it is its own step's k_product, launched ordinarily (all
+// before that has ended when it starts), whose blocks have all started when
+// k_band does.  Neither may be changed without the other.  A launch that is no
+// such kernel's neighbour behaves as an ordinary one.  Pointers to what a
+// predecessor writes carry no __restrict__: the compiler may not take the data
+// for constant.
 // Measured on whole calls (us, ordinary / programmatic): norm1 of a 37 x 29 grid
 // 46.5 / 38.3, one banded product of 30001 rows 259 / 246, exp of the 1D
 // Laplacian, n = 256, 511 / 430, cos of banded N(0, 1), n = 1000, 1084 / 1014,
@@ -1903,6 +1910,12 @@ __global__ void __launch_bounds__(kCtaWarps * 32, 7) k_product_cta(const __grid_
 // banded n = 65536, half-bandwidth 5: Z Z^9 361 -> 200 us, the giant steps
 // 470-527 -> 324-423 us (77-81 % of the pipe); banded N(0, 1) n = 20000,
 // w = 15: giant steps 2.31-6.22 -> 1.92-4.59 ms (93-98 %).
+//
+// All instances are held to 72 registers, so that seven blocks fit an SM, and
+// spill (bytes of stores / loads, -Xptxas -v): one row a tile 30-34 / 32-40,
+// shared by the block 8-30 / 4-28; four rows 106-130 / 184-208, shared 70-94 /
+// 100-128; in a batch one row 30-82 / 28-72, four 238-294 / 360-448.  The batch's
+// four rows pay for it (launch_band); elsewhere they are faster all the same.
 //
 // TEAM: the block's four warps share a tile and take its column groups in
 // turn (long rows, or few).  A row with a term that is not full, or whose
@@ -4311,7 +4324,8 @@ cudaError_t launch_product(const ProductArgs& P, bool table, cudaStream_t st, do
 
 // In a batch with instances of both kinds the step is two launches, k_product
 // and k_band, neither of which reads what the other writes.  k_band is
-// launched programmatically: its blocks take the SMs that k_product's leave
+// launched programmatically, right behind its step's k_product (which itself is
+// launched ordinarily: see pdl_enter): its blocks take the SMs that k_product's leave
 // (each kernel's warps end at different times, a quarter of them idle on
 // average), and it waits for k_product's end before it ends the step itself.
 // 128 instances of 64-4096 rows: 17.6 -> 15.8 ms a call, 27: 5.1 -> 4.8 ms.
